@@ -62,7 +62,7 @@ enum { GAR_SUM = 0, GAR_MAX = 1, GAR_MIN = 2 };
  *   combines them with the own block; needs the workspace reported by
  *   gar_plan_bytes; records the bytes read from partners per step.  The launches of
  *   one call are chained by programmatic dependent launch: a launch may become resident
- *   early but reads nothing before every earlier kernel on the stream has completed.
+ *   early but reads no buffer before every earlier kernel on the stream has completed.
  * GAR_FUSED: one launch for the whole Allreduce; per element position the P
  *   contributions are loaded once, the reduction program that the schedule induces
  *   runs in registers, and every rank's result is written once.  The program becomes

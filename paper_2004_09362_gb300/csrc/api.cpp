@@ -72,6 +72,8 @@ int prepare_step_faithful(gar_plan *pl) {
   if (rc) return rc;
   // the step kernels' module, loaded now rather than at the first launch
   if ((rc = load_step_module())) return rc;
+  const bool upload = pl->d_ops == nullptr || pl->d_launches == nullptr || pl->d_barrier == nullptr ||
+                      pl->d_step_bytes == nullptr;
   if (pl->d_ops == nullptr && !pl->ops.empty()) {
     cudaError_t e = cudaMalloc(&pl->d_ops, pl->ops.size() * sizeof(StepOp));
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(op table)");
@@ -81,7 +83,7 @@ int prepare_step_faithful(gar_plan *pl) {
   }
   if (pl->d_launches == nullptr && !pl->launches.empty()) {
     std::vector<LaunchDesc> ld;
-    for (const Launch &ln : pl->launches) ld.push_back({ln.first_op, ln.nops, ln.partner, ln.comm_step});
+    for (const Launch &ln : pl->launches) ld.push_back(launch_desc(*pl, ln));
     cudaError_t e = cudaMalloc(&pl->d_launches, ld.size() * sizeof(LaunchDesc));
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(launch table)");
     e = cudaMemcpy(pl->d_launches, ld.data(), ld.size() * sizeof(LaunchDesc), cudaMemcpyHostToDevice);
@@ -94,11 +96,17 @@ int prepare_step_faithful(gar_plan *pl) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset(barrier state)");
   }
   if (pl->d_step_bytes == nullptr && pl->S > 0) {
-    const size_t cbytes = (size_t)pl->S * STEP_BYTE_SLOTS * sizeof(unsigned long long);
+    const size_t cbytes = (size_t)(pl->S + 1) * STEP_BYTE_SLOTS * sizeof(unsigned long long);
     cudaError_t e = cudaMalloc(&pl->d_step_bytes, cbytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(step counters)");
     e = cudaMemset(pl->d_step_bytes, 0, cbytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset(step counters)");
+  }
+  if (upload) {
+    // the uploads above are ordered before launches on every stream, and before the part
+    // of a launch that runs ahead of its predecessor's end
+    cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize(plan tables)");
   }
   return GAR_OK;
 }
@@ -408,13 +416,15 @@ int run_step_faithful(gar_plan *pl, void *const *rank, gar_stream_t stream, bool
       return GAR_ENOWS;
     }
   }
-  cudaError_t e = cudaMemsetAsync(pl->d_step_bytes, 0,
-                                  (size_t)pl->S * STEP_BYTE_SLOTS * sizeof(unsigned long long),
-                                  (cudaStream_t)stream);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(step counters)");
+  if (pl->step_bytes_stale) {
+    // an earlier sequence stopped part-way: the kernels' own upkeep of the counters did too
+    cudaError_t e = cudaMemsetAsync(pl->d_step_bytes, 0,
+                                    (size_t)(pl->S + 1) * STEP_BYTE_SLOTS * sizeof(unsigned long long),
+                                    (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(step counters)");
+  }
+  pl->step_bytes_stale = true;
   if (persistent) {
-    e = cudaMemsetAsync(pl->d_barrier, 0, barrier_state_bytes(), (cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(barrier state)");
     rc = launch_persistent(*pl, rank, stream);
     if (rc) return rc;
     pl->ran_persistent = true;
@@ -424,6 +434,7 @@ int run_step_faithful(gar_plan *pl, void *const *rank, gar_stream_t stream, bool
       if (rc) return rc;
     }
   }
+  pl->step_bytes_stale = false;
   pl->last_stream = stream;
   pl->ran_step_faithful = true;
   return GAR_OK;
@@ -791,12 +802,14 @@ int gar_plan_status(gar_plan *pl) {
   if (!pl->ran_persistent || pl->d_barrier == nullptr) return GAR_OK;
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)pl->last_stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-  int st[4] = {0, 0, 0, 0};
-  e = cudaMemcpy(st, pl->d_barrier, sizeof st, cudaMemcpyDeviceToHost);
+  std::vector<char> state(barrier_state_bytes());
+  e = cudaMemcpy(state.data(), pl->d_barrier, state.size(), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(barrier state)");
-  if (st[2] != 0) {
+  int error = 0, launch = 0;
+  barrier_outcome(state.data(), &error, &launch);
+  if (error != 0) {
     set_error("persistent step-faithful kernel: a grid-barrier wait gave up after launch " +
-              std::to_string(st[3]));
+              std::to_string(launch));
     return GAR_ETIMEOUT;
   }
   return GAR_OK;

@@ -51,6 +51,7 @@ struct Launch {
 // Launch descriptor as the persistent kernel reads it from device memory.
 struct LaunchDesc {
   int first_op, nops, partner, comm_step;
+  int group;          // element-major mapping: ops per thread
 };
 
 struct CommStep {
@@ -100,7 +101,8 @@ struct gar_plan {
   size_t ws_set_bytes = 0;
   int device = -1;
   gar::StepOp *d_ops = nullptr;
-  unsigned long long *d_step_bytes = nullptr;
+  unsigned long long *d_step_bytes = nullptr;  // S + 1 rows of STEP_BYTE_SLOTS counters
+  bool step_bytes_stale = false;      // a sequence of step launches did not complete
   gar_stream_t last_stream = nullptr;
   bool ran_step_faithful = false;
   gar::JitKernel *fused = nullptr;   // owned by the JIT cache
@@ -171,6 +173,8 @@ int launch_step(const gar_plan &pl, const Launch &ln, int launch_index, void *co
                 gar_stream_t stream);
 int launch_persistent(const gar_plan &pl, void *const *rank, gar_stream_t stream);
 size_t barrier_state_bytes();
+void barrier_outcome(const void *state, int *error, int *launch);
+LaunchDesc launch_desc(const gar_plan &pl, const Launch &ln);
 int load_step_module();
 
 // api.cpp

@@ -9,9 +9,10 @@
 // of one (op, rank) pair (short blocks: one thread per (op, element) instead).  Combine
 // ops batch 2 vectors per thread; same-type copies move raw 16-byte units, 6 per
 // thread; a bf16 plan's first step keeps its 16-byte bf16 loads packed until the
-// combine.  Each warp counts the elements it read from partners and adds the bytes to
-// one of the step's counter slots, so the bytes a step actually moved are recorded.
-// The launches of one Allreduce are chained by programmatic dependent launch.
+// combine.  The kernels add the bytes they read from partners to the step's counter
+// slots, so the bytes a step actually moved are recorded.  The launches of one Allreduce
+// are chained by programmatic dependent launch.  The same work functions serve the
+// per-step launches, the persistent kernel and the no-allocation launches.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -25,20 +26,40 @@
 namespace gar {
 namespace {
 
-#ifndef GAR_STEP_CHUNK
-#define GAR_STEP_CHUNK 16384
-#endif
-#ifndef GAR_STEP_UNROLL
-#define GAR_STEP_UNROLL 2
-#endif
-// Launch shape, from a sweep on GB300 (P=24 x 64 MiB fp32, P=127 x 8 MiB bf16, P=8 x
-// 1 MiB): CTAs own 16384-element chunks (smaller chunks ran up to 2.5x slower) and each
-// thread issues the loads of 2 vectors before combining.  Small vectors drop the chunk
-// to 8192 or 4096 elements to keep at least 4 CTAs per SM.
+// Launch shape, from sweeps on GB300: CTAs own 16384-element chunks of large vectors
+// (smaller chunks ran up to 2.5x slower) and each thread issues the loads of 2 vectors
+// before combining.  Launches of fewer than 4 CTAs per SM halve the chunk, down to one
+// batch of loads per thread (P = 20 x 1 MiB fp32 S = 9 without allocation: 34 us at 2048
+// elements, 36 at 4096 and 1024).
 constexpr int kThreads = 256;
-constexpr uint64_t kChunk = GAR_STEP_CHUNK;  // largest chunk (elements per CTA)
-constexpr int kUnroll = GAR_STEP_UNROLL;     // 4-element vectors a thread loads at once
+constexpr uint64_t kChunk = 16384;      // largest chunk (elements per CTA)
+constexpr uint64_t kMinChunk = 2048;    // smallest chunk
+constexpr uint64_t kMinCtas = 4;        // CTAs per SM below which the chunk is halved
+constexpr int kUnroll = 2;              // 4-element vectors a thread loads at once
 constexpr uint64_t kFlatBelow = 4 * kThreads * kUnroll;  // blocks shorter than this: element-major
+// Element-major launches: threads per SM before a thread takes 2 or 4 ops instead of one.
+// P = 127 x 9 KiB bf16 S = 10: 44.5 us with one op per thread throughout (and the next
+// launch at the end); 33.3 us at 512
+// threads, 36.8 at 256, 35.7 at 1024, 41.8 at 2048 (43.5 with up to 8 ops per thread).
+constexpr int kFlatGroup = 4;
+constexpr uint64_t kFlatThreads = 512;
+// Persistent steps: smallest piece of a block, and what starting a piece costs, in
+// elements.  The chunked steps run in CTAs of 512 threads, 2 per SM: the grid barrier has
+// 304 arrivals and pollers (P = 24 x 4 MiB int32, S = 10: 95.6 us; 98.2 in 1024-thread
+// CTAs, 98.9 in 256-thread ones, 4 per SM).
+constexpr int kPersistThreads = 512;
+constexpr int kPersistPerSM = 2;
+constexpr uint64_t kMinPiece = 1024;
+constexpr uint64_t kPieceCost = 512;
+
+// Counter upkeep of one launch, by its first CTA (after wait_prior_grid): zeroes the
+// counters of the communication step that follows, and moves the first step's counts,
+// which were added to a row of their own, to their place.  So every step's counters are
+// zero when its launch starts, without a memset in the launch sequence.
+struct CounterUpkeep {
+  unsigned long long *zero;                // row to zero, or nullptr
+  unsigned long long *move_from, *move_to; // row to move (and zero), or nullptr
+};
 
 template <int MAXP>
 struct StepArgs {
@@ -47,10 +68,17 @@ struct StepArgs {
   const StepOp *ops;                 // this launch's ops
   unsigned long long *bytes;         // STEP_BYTE_SLOTS counters of the step, or nullptr
   uint64_t q, rem, n_pad;
-  uint64_t chunk;                    // elements per CTA
   uint64_t n;                        // elements per rank
+  uint32_t chunk;                    // elements per CTA
   int P, partner, nops, nchunks;
+  int group;                         // ops per thread (element-major mapping)
   int xor_group;                     // 1: placements and partners combine by XOR (Table 1b)
+  int early;                         // 1: the next launch is this call's (element-major: it may start at once)
+  // 1: work items in descending order.  Every second launch runs so, and then first reads
+  // what its predecessor wrote last, which L2 still holds (P = 127 x 8 MiB bf16 S = 14:
+  // 1114 us instead of 1132).
+  int reverse;
+  CounterUpkeep upkeep;
 };
 
 template <typename T> struct AccOf { using type = T; };
@@ -140,51 +168,40 @@ __device__ __forceinline__ void *buf_ptr(const StepArgs<MAXP> &a, uint8_t buf, i
 // v mod P for v in (-P, 2P).
 __device__ __forceinline__ int wrap_rank(int v, int P) { return v < 0 ? v + P : (v >= P ? v - P : v); }
 
-// This warp's slot of a step's byte counter.
-__device__ __forceinline__ int byte_slot() {
-  return (int)((blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) % STEP_BYTE_SLOTS);
-}
+// Programmatic dependent launch: the step launches of one Allreduce are made with
+// programmatic stream serialisation, so launch i+1's CTAs may become resident while
+// launch i drains.  griddepcontrol.wait blocks until every prerequisite grid has
+// completed and its memory is visible (a no-op without such a dependency); nothing but
+// the kernel's parameters and the plan's op table, which never changes, is read before
+// it.  launch_dependents lets the next launch start once every CTA of this one has issued
+// it or exited.  Chunked launches issue it when their work is done: at the start, the
+// waiting CTAs took slots from the running ones' (P = 127 x 8 MiB bf16 S = 14 1122 us
+// instead of 1112, P = 20 x 1 MiB fp32 S = 9 without allocation 37.6 instead of 34.3).
+__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Per-launch parameters the work functions need besides the buffers.
 struct LaunchView {
   const StepOp *ops;
   unsigned long long *bytes;  // STEP_BYTE_SLOTS counters of the communication step, or nullptr
-  uint64_t chunk;             // elements per CTA item (chunked mapping)
+  uint32_t chunk;             // elements per CTA item (chunked mapping)
   int nops, partner, nchunks;
+  int group;                  // ops per thread (element-major mapping)
 };
 
-// Chunked mapping: work item `item` = (chunk, rank x, op) is done by the whole CTA.
-// kCopyPaths: copy-only ops take the deeper copy loops.  The persistent kernel, which
-// keeps its launch loop's state live around this body, leaves them out: with them it
-// needs 109 registers (2 CTAs per SM) instead of about 75 (3 CTAs per SM).
-template <typename T, int OP, int MAXP, bool kCopyPaths = true>
-__device__ __forceinline__ void chunk_work(const StepArgs<MAXP> &a, const LaunchView &lv, uint64_t item) {
+// Elements [c0, c0 + len) of the block that op `op` touches at rank x, by the CTA's NT threads.
+template <typename T, int OP, int MAXP, int NT>
+__device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const LaunchView &lv, const StepOp &op, int x,
+                                           uint64_t c0, uint32_t len) {
   using A = typename AccOf<T>::type;
-  // 32-bit index arithmetic whenever the item fits (always for a launch's own grid):
-  // 64-bit division is a long software sequence and ran once per CTA.
-  int chunk, x, oi;
-  if (item <= 0xffffffffull) {
-    uint32_t it = (uint32_t)item;
-    chunk = (int)(it % (uint32_t)lv.nchunks);
-    it /= (uint32_t)lv.nchunks;
-    x = (int)(it % (uint32_t)a.P);
-    oi = (int)(it / (uint32_t)a.P);
-  } else {
-    chunk = (int)(item % (uint64_t)lv.nchunks);
-    item /= (uint64_t)lv.nchunks;
-    x = (int)(item % (uint64_t)a.P);
-    oi = (int)(item / (uint64_t)a.P);
-  }
-  if (oi >= lv.nops) return;
-  const StepOp op = lv.ops[oi];
+  constexpr bool kMixed = sizeof(T) != sizeof(A);  // rank buffers hold a narrower type than the slices
   // placements and ranks are in [0, P), partner offsets in (-P, P)
   const int b = a.xor_group ? (x ^ (int)op.dst_place) : wrap_rank(x - (int)op.dst_place, a.P);
   const uint64_t bstart = (uint64_t)b * a.q + ((uint64_t)b < a.rem ? (uint64_t)b : a.rem);
   const uint64_t blen = a.q + ((uint64_t)b < a.rem ? 1 : 0);
-  const uint64_t c0 = (uint64_t)chunk * lv.chunk;
   if (c0 >= blen) return;
   const uint64_t lo = bstart + c0;
-  const uint64_t hi = bstart + (blen < c0 + lv.chunk ? blen : c0 + lv.chunk);
+  const uint64_t hi = bstart + (blen < c0 + len ? blen : c0 + len);
 
   const bool has_recv = op.recv_place >= 0;
   const int partner = a.xor_group ? (x ^ lv.partner) : wrap_rank(x + lv.partner, a.P);
@@ -193,256 +210,207 @@ __device__ __forceinline__ void chunk_work(const StepArgs<MAXP> &a, const Launch
   const void *own0 = buf_ptr<A>(a, op.out0_own, x);
   void *out1 = buf_ptr<A>(a, op.out1_buf, x);
   const void *own1 = buf_ptr<A>(a, op.out1_own, x);
+  // An op with one source and one output is a copy (distribution steps, q* moves); between
+  // buffers of one element type it moves raw 16-byte units (4 fp32 or 8 bf16 elements).
+  const bool copy_only = !out1 && (has_recv != (own0 != nullptr));
+  const uint8_t src_buf = has_recv ? op.recv_buf : op.out0_own;
+  const bool raw = copy_only && (!kMixed || src_buf == op.out0_buf);
+  // bf16 partner block + bf16 own block -> fp32 partial (the first reduction step of a
+  // bf16 plan)
+  const bool packed = kMixed && has_recv && !out1 && own0 != nullptr && op.recv_buf == BUF_RANK &&
+                      op.out0_own == BUF_RANK && op.out0_buf != BUF_RANK;
 
-  uint64_t moved = 0;
-  auto do1 = [&](uint64_t e) {
+  // Element offsets are the same in every buffer, and every buffer base is 16-byte
+  // aligned, so one head/body/tail split serves all operands: `unit` elements per vector,
+  // fewer than one unit at either end.
+  const uint32_t unit = (kMixed && raw && src_buf == BUF_RANK) ? 8 : 4;
+  uint64_t va = (lo + unit - 1) & ~(uint64_t)(unit - 1), vb = hi & ~(uint64_t)(unit - 1);
+  if (va > hi) va = hi;
+  if (vb < va) vb = va;
+  const uint32_t head = (uint32_t)(va - lo), ends = head + (uint32_t)(hi - vb);
+  for (uint32_t k = threadIdx.x; k < ends; k += NT) {
+    const uint64_t e = k < head ? lo + k : vb + (k - head);
     A r = A(0);
-    if (has_recv) {
-      r = load1<T, A>(op.recv_buf, recv, e);
-      ++moved;
-    }
+    if (has_recv) r = load1<T, A>(op.recv_buf, recv, e);
     A o0 = r, o1 = r;
-    if (own0) o0 = has_recv ? combine<OP>(load1<T, A>(op.out0_own, own0, e), r) : load1<T, A>(op.out0_own, own0, e);
-    if (out1 && own1) o1 = has_recv ? combine<OP>(load1<T, A>(op.out1_own, own1, e), r) : load1<T, A>(op.out1_own, own1, e);
+    if (own0) o0 = load1<T, A>(op.out0_own, own0, e);
+    if (own0 && has_recv) o0 = combine<OP>(o0, r);
+    if (own1) o1 = load1<T, A>(op.out1_own, own1, e);
+    if (own1 && has_recv) o1 = combine<OP>(o1, r);
     store1<T, A>(op.out0_buf, out0, e, o0);
     if (out1) store1<T, A>(op.out1_buf, out1, e, o1);
-  };
-  // kUnroll aligned 4-element vectors per thread: every load of the batch is issued
-  // before the first combine, so a thread keeps up to 3 * kUnroll 16-byte loads in flight.
-  auto do4xU = [&](uint64_t e_first, uint64_t stride, uint64_t vend) {
-    A r[kUnroll][4], o0[kUnroll][4], o1[kUnroll][4];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const uint64_t e = e_first + u * stride;
-      if (e < vend) {
-        if (has_recv) {
-          load4<T, A>(op.recv_buf, recv, e, r[u]);
-          moved += 4;
-        }
-        if (own0) load4<T, A>(op.out0_own, own0, e, o0[u]);
-        if (out1 && own1) load4<T, A>(op.out1_own, own1, e, o1[u]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const uint64_t e = e_first + u * stride;
-      if (e < vend) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (!has_recv) {
-            r[u][k] = A(0);
-          }
-          o0[u][k] = own0 ? (has_recv ? combine<OP>(o0[u][k], r[u][k]) : o0[u][k]) : r[u][k];
-          if (out1) o1[u][k] = own1 ? (has_recv ? combine<OP>(o1[u][k], r[u][k]) : o1[u][k]) : r[u][k];
-        }
-        store4<T, A>(op.out0_buf, out0, e, o0[u]);
-        if (out1) store4<T, A>(op.out1_buf, out1, e, o1[u]);
-      }
-    }
-  };
-
-  // Copy-only ops (one source, one output: the distribution steps' copies and the q*
-  // moves) load one operand per vector instead of two, so they batch twice as many
-  // vectors per thread to keep the same bytes in flight.
-  auto copy4xU = [&](uint64_t e_first, uint64_t stride, uint64_t vend) {
-    constexpr int U = 2 * kUnroll;
-    const void *src = has_recv ? recv : own0;
-    const uint8_t sbuf = has_recv ? op.recv_buf : op.out0_own;
-    A v[U][4];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint64_t e = e_first + u * stride;
-      if (e < vend) {
-        load4<T, A>(sbuf, src, e, v[u]);
-        if (has_recv) moved += 4;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint64_t e = e_first + u * stride;
-      if (e < vend) store4<T, A>(op.out0_buf, out0, e, v[u]);
-    }
-  };
-  const bool copy_only = kCopyPaths && !out1 && (has_recv != (own0 != nullptr));
-  const uint8_t copy_src_buf = has_recv ? op.recv_buf : op.out0_own;
-  // A copy between buffers of one element type moves raw 16-byte units (4 fp32 or 8 bf16
-  // elements) with a compile-time stride: few registers, so 6 units per thread in flight
-  // within the 40-register budget.  bf16 copies used 8-byte units before and ran at
-  // about 4 TB/s (48 bytes in flight per thread) against 6.6 TB/s for fp32; elements
-  // before the first and after the last 16-byte boundary go one by one.
-  auto raw_copy = [&](uint64_t va, uint64_t vb) {
+  }
+  const uint32_t units = (uint32_t)((vb - va) / unit);
+  if (raw) {
+    // 6 units per thread in flight within the 40-register budget.  bf16 copies of 8-byte
+    // units ran at about 4 TB/s (48 bytes in flight per thread) against 6.6 TB/s for fp32.
     constexpr int U = 6;
-    const void *srcp = has_recv ? recv : own0;
-    const uint64_t esz = copy_src_buf == BUF_RANK ? sizeof(T) : sizeof(A);
-    const uint64_t epu = 16 / esz;  // elements per 16-byte unit
-    uint64_t ua = (va + epu - 1) / epu * epu, ub = vb / epu * epu;
-    if (ua > vb) ua = vb;
-    if (ub < ua) ub = ua;
-    for (uint64_t e = va + threadIdx.x; e < ua; e += kThreads) do1(e);
-    for (uint64_t e = ub + threadIdx.x; e < vb; e += kThreads) do1(e);
-    const int4 *src = reinterpret_cast<const int4 *>(static_cast<const char *>(srcp) + ua * esz);
-    int4 *dst = reinterpret_cast<int4 *>(static_cast<char *>(out0) + ua * esz);
-    const uint64_t units = (ub - ua) / epu;
-    for (uint64_t k = threadIdx.x; k < units; k += (uint64_t)U * kThreads) {
-      const uint64_t left = units - k;
+    const uint64_t off = va * (src_buf == BUF_RANK ? sizeof(T) : sizeof(A));
+    const int4 *src = reinterpret_cast<const int4 *>(static_cast<const char *>(has_recv ? recv : own0) + off);
+    int4 *dst = reinterpret_cast<int4 *>(static_cast<char *>(out0) + off);
+    for (uint32_t k = threadIdx.x; k < units; k += U * NT) {
       int4 v[U];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if ((uint64_t)u * kThreads < left) v[u] = src[k + (uint64_t)u * kThreads];
+        if (k + u * NT < units) v[u] = src[k + u * NT];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if ((uint64_t)u * kThreads < left) dst[k + (uint64_t)u * kThreads] = v[u];
-      if (has_recv) {
-        const uint64_t cnt = left < (uint64_t)(U - 1) * kThreads + 1 ? (left + kThreads - 1) / kThreads : U;
-        moved += epu * cnt;
-      }
+        if (k + u * NT < units) dst[k + u * NT] = v[u];
     }
-  };
-  const bool raw = copy_only && (sizeof(T) == sizeof(A) || copy_src_buf == op.out0_buf);
-
-  // bf16 partner block + bf16 own block -> fp32 partial (the first reduction step of a
-  // bf16 plan).  Each lane reads 4 bf16 (8 bytes) of both operands and writes their 4
-  // fp32 partials as one 16-byte store, so every warp store covers 512 contiguous bytes.
-  // Reading 8 bf16 per lane instead made each 16-byte store half of a 32-byte stretch, a
-  // warp store then half-filled 32 sectors, and the step ran at 74 % of DRAM throughput
-  // (P = 127 x 8 MiB bf16: whole Allreduce S = 14 1.190 -> 1.164 ms, S = 10 2.323 ->
-  // 2.288 ms).  4 units per thread keep 64 bytes of loads in flight.
-  auto packed_combine = [&](uint64_t va, uint64_t vb) {
+  } else if (packed) {
+    // Each lane reads 4 bf16 (8 bytes) of both operands and writes their 4 fp32 partials as
+    // one 16-byte store, so every warp store covers 512 contiguous bytes.  Reading 8 bf16
+    // per lane instead made each 16-byte store half of a 32-byte stretch, a warp store then
+    // half-filled 32 sectors, and the step ran at 74 % of DRAM throughput (P = 127 x 8 MiB
+    // bf16: whole Allreduce S = 14 1.190 -> 1.164 ms, S = 10 2.323 -> 2.288 ms).  4 units
+    // per thread keep 64 bytes of loads in flight.
     constexpr int U = 4;
-    uint64_t ua = (va + 3) & ~uint64_t(3), ub = vb & ~uint64_t(3);
-    if (ua > vb) ua = vb;
-    if (ub < ua) ub = ua;
-    for (uint64_t e = va + threadIdx.x; e < ua; e += kThreads) do1(e);
-    for (uint64_t e = ub + threadIdx.x; e < vb; e += kThreads) do1(e);
-    const uint2 *rp = reinterpret_cast<const uint2 *>(static_cast<const char *>(recv) + ua * sizeof(T));
-    const uint2 *op_ = reinterpret_cast<const uint2 *>(static_cast<const char *>(own0) + ua * sizeof(T));
-    float4 *dp = reinterpret_cast<float4 *>(static_cast<char *>(out0) + ua * sizeof(A));
-    const uint64_t units = (ub - ua) >> 2;
-    for (uint64_t k = threadIdx.x; k < units; k += (uint64_t)U * kThreads) {
-      const uint64_t left = units - k;
+    const uint2 *rp = reinterpret_cast<const uint2 *>(static_cast<const T *>(recv) + va);
+    const uint2 *wp = reinterpret_cast<const uint2 *>(static_cast<const T *>(own0) + va);
+    float4 *dp = reinterpret_cast<float4 *>(static_cast<A *>(out0) + va);
+    for (uint32_t k = threadIdx.x; k < units; k += U * NT) {
       uint2 rv[U], ov[U];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if ((uint64_t)u * kThreads < left) {
-          rv[u] = rp[k + (uint64_t)u * kThreads];
-          ov[u] = op_[k + (uint64_t)u * kThreads];
+        if (k + u * NT < units) {
+          rv[u] = rp[k + u * NT];
+          ov[u] = wp[k + u * NT];
         }
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if ((uint64_t)u * kThreads < left) {
+        if (k + u * NT < units) {
           float4 f;
           f.x = combine<OP>(__uint_as_float(ov[u].x << 16), __uint_as_float(rv[u].x << 16));
           f.y = combine<OP>(__uint_as_float(ov[u].x & 0xffff0000u), __uint_as_float(rv[u].x & 0xffff0000u));
           f.z = combine<OP>(__uint_as_float(ov[u].y << 16), __uint_as_float(rv[u].y << 16));
           f.w = combine<OP>(__uint_as_float(ov[u].y & 0xffff0000u), __uint_as_float(rv[u].y & 0xffff0000u));
-          dp[k + (uint64_t)u * kThreads] = f;
+          dp[k + u * NT] = f;
         }
-      if (has_recv) {
-        const uint64_t cnt = left < (uint64_t)(U - 1) * kThreads + 1 ? (left + kThreads - 1) / kThreads : U;
-        moved += cnt << 2;
-      }
     }
-  };
-  const bool packed = sizeof(T) == 2 && kCopyPaths && has_recv && !out1 && own0 != nullptr &&
-                      op.recv_buf == BUF_RANK && op.out0_own == BUF_RANK && op.out0_buf != BUF_RANK;
-
-  // Element offsets are the same in every buffer, and every buffer base is 16-byte
-  // aligned, so one head/body/tail split serves all operands.
-  uint64_t va = (lo + 3) & ~uint64_t(3);
-  uint64_t vb = hi & ~uint64_t(3);
-  if (va > hi) va = hi;
-  if (vb < va) vb = va;
-  for (uint64_t e = lo + threadIdx.x; e < va; e += blockDim.x) do1(e);
-  const uint64_t vstride = 4 * (uint64_t)blockDim.x;
-  if (raw) {
-    raw_copy(va, vb);
-  } else if (packed) {
-    packed_combine(va, vb);
-  } else if (copy_only) {
-    for (uint64_t e = va + 4 * (uint64_t)threadIdx.x; e < vb; e += 2 * kUnroll * vstride)
-      copy4xU(e, vstride, vb);
   } else {
-    for (uint64_t e = va + 4 * (uint64_t)threadIdx.x; e < vb; e += kUnroll * vstride)
-      do4xU(e, vstride, vb);
-  }
-  for (uint64_t e = vb + threadIdx.x; e < hi; e += blockDim.x) do1(e);
-
-  // The step's received bytes: summed over the warp, then over the CTA in shared memory,
-  // one atomic add per CTA into one of the step's 32 counter slots.  (Whether an op
-  // receives is the same for the whole CTA, so every thread takes this branch or none.)
-  if (lv.bytes != nullptr && has_recv) {
-    __shared__ unsigned long long s_moved[kThreads / 32];
-    unsigned long long m = moved;
+    // kUnroll aligned 4-element vectors per thread: every load of the batch is issued
+    // before the first combine, so a thread keeps up to 3 * kUnroll 16-byte loads in flight.
+    for (uint32_t k = threadIdx.x; k < units; k += kUnroll * NT) {
+      A r[kUnroll][4], o0[kUnroll][4], o1[kUnroll][4];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m += __shfl_down_sync(0xffffffffu, m, off);
-    if ((threadIdx.x & 31) == 0) s_moved[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned long long t = 0;
+      for (int u = 0; u < kUnroll; ++u)
+        if (k + u * NT < units) {
+          const uint64_t e = va + 4 * (uint64_t)(k + u * NT);
+          if (has_recv) load4<T, A>(op.recv_buf, recv, e, r[u]);
+          if (own0) load4<T, A>(op.out0_own, own0, e, o0[u]);
+          if (own1) load4<T, A>(op.out1_own, own1, e, o1[u]);
+        }
 #pragma unroll
-      for (int w = 0; w < kThreads / 32; ++w) t += s_moved[w];
-      const unsigned long long esize = (op.recv_buf == BUF_RANK) ? sizeof(T) : sizeof(A);
-      if (t) atomicAdd(lv.bytes + blockIdx.x % STEP_BYTE_SLOTS, t * esize);
+      for (int u = 0; u < kUnroll; ++u)
+        if (k + u * NT < units) {
+          const uint64_t e = va + 4 * (uint64_t)(k + u * NT);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            o0[u][c] = own0 ? (has_recv ? combine<OP>(o0[u][c], r[u][c]) : o0[u][c]) : r[u][c];
+            if (out1) o1[u][c] = own1 ? (has_recv ? combine<OP>(o1[u][c], r[u][c]) : o1[u][c]) : r[u][c];
+          }
+          store4<T, A>(op.out0_buf, out0, e, o0[u]);
+          if (out1) store4<T, A>(op.out1_buf, out1, e, o1[u]);
+        }
     }
-    __syncthreads();  // s_moved is written again by the next work item of a persistent CTA
   }
+  // The received bytes: the CTA has read each of its elements from the partner once.
+  if (lv.bytes != nullptr && has_recv && threadIdx.x == 0) {
+    const unsigned long long esize = (op.recv_buf == BUF_RANK) ? sizeof(T) : sizeof(A);
+    atomicAdd(lv.bytes + blockIdx.x % STEP_BYTE_SLOTS, (hi - lo) * esize);
+  }
+}
+
+// Chunked mapping: work item `item` = (chunk, rank x, op) is done by the whole CTA.
+template <typename T, int OP, int MAXP>
+__device__ __forceinline__ void chunk_work(const StepArgs<MAXP> &a, const LaunchView &lv, uint32_t item) {
+  const int chunk = (int)(item % (uint32_t)lv.nchunks);
+  item /= (uint32_t)lv.nchunks;
+  const StepOp op = lv.ops[item / (uint32_t)a.P];
+  range_work<T, OP, MAXP, kThreads>(a, lv, op, (int)(item % (uint32_t)a.P), (uint64_t)chunk * lv.chunk, lv.chunk);
 }
 
 // Element-major mapping, for small blocks: an op touches block b = (x - dst_place) mod P
 // at every rank x, i.e. every element position exactly once across the P ranks, so
-// work item g = (op, element e) maps to rank x = (b(e) + dst_place) mod P.  One thread
-// per item keeps every thread busy however short the blocks are.  Threads g_first,
-// g_first + g_stride, ... of the launch's nops * n items.
+// work item g = (op group, element e) maps to rank x = (b(e) + dst_place) mod P.  One
+// thread per item keeps every thread busy however short the blocks are; an item is
+// `group` (1, 2 or 4) consecutive ops, which share the position's block index and keep
+// their loads in flight together.  `ranks`: the rank pointers in shared memory, because
+// the lanes of a warp work on several blocks, so on several ranks.  The ops are read
+// before wait_prior_grid (they never change), the buffers after it.
 template <typename T, int OP, int MAXP>
-__device__ __forceinline__ void flat_work(const StepArgs<MAXP> &a, const LaunchView &lv, uint64_t g_first,
-                                          uint64_t g_stride) {
+__device__ __forceinline__ void flat_work(const StepArgs<MAXP> &a, const LaunchView &lv, void *const *ranks,
+                                          uint64_t g_first, uint64_t g_stride) {
   using A = typename AccOf<T>::type;
-  const uint64_t total = (uint64_t)lv.nops * a.n;
+  const uint64_t groups = (uint64_t)((lv.nops + lv.group - 1) / lv.group);
+  const uint64_t total = groups * a.n;
   const uint64_t big = a.rem * (a.q + 1);
-  unsigned long long moved_bytes = 0;
+  uint32_t moved = 0;
   // 32-bit index arithmetic when every index fits (the element-major launch serves
   // short blocks, so practically always): 64-bit division is a long software sequence.
   const bool narrow_idx = total + g_stride <= 0xffffffffull;
+  auto slot = [&](uint8_t buf, int rank) -> char * {
+    if (buf == BUF_RANK) return static_cast<char *>(ranks[rank]);
+    return static_cast<char *>(a.ws[buf - BUF_QP0]) + (uint64_t)rank * a.n_pad * sizeof(A);
+  };
   for (uint64_t g = g_first; g < total; g += g_stride) {
-    int oi, b;
+    int gi, b;
     uint64_t e;
     if (narrow_idx) {
       const uint32_t g32 = (uint32_t)g, n32 = (uint32_t)a.n;
-      oi = (int)(g32 / n32);
-      const uint32_t e32 = g32 - (uint32_t)oi * n32;
+      gi = (int)(g32 / n32);
+      const uint32_t e32 = g32 - (uint32_t)gi * n32;
       e = e32;
       b = e32 < (uint32_t)big ? (int)(e32 / (uint32_t)(a.q + 1))
                               : (int)((uint32_t)a.rem + (e32 - (uint32_t)big) / (uint32_t)a.q);
     } else {
-      oi = (int)(g / a.n);
-      e = g - (uint64_t)oi * a.n;
+      gi = (int)(g / a.n);
+      e = g - (uint64_t)gi * a.n;
       b = e < big ? (int)(e / (a.q + 1)) : (int)(a.rem + (e - big) / a.q);
     }
-    const StepOp op = lv.ops[oi];
-    const int x = a.xor_group ? (b ^ (int)op.dst_place) : wrap_rank(b + (int)op.dst_place, a.P);
-    A r = A(0);
-    const bool has_recv = op.recv_place >= 0;
-    if (has_recv) {
-      const int partner = a.xor_group ? (x ^ lv.partner) : wrap_rank(x + lv.partner, a.P);
-      r = load1<T, A>(op.recv_buf, buf_ptr<A>(a, op.recv_buf, partner), e);
-      moved_bytes += (op.recv_buf == BUF_RANK) ? sizeof(T) : sizeof(A);
-    }
-    A o0 = r, o1 = r;
-    if (op.out0_own != BUF_NONE) {
-      const A v = load1<T, A>(op.out0_own, buf_ptr<A>(a, op.out0_own, x), e);
-      o0 = has_recv ? combine<OP>(v, r) : v;
-    }
-    if (op.out1_buf != BUF_NONE && op.out1_own != BUF_NONE) {
-      const A v = load1<T, A>(op.out1_own, buf_ptr<A>(a, op.out1_own, x), e);
-      o1 = has_recv ? combine<OP>(v, r) : v;
-    }
-    store1<T, A>(op.out0_buf, buf_ptr<A>(a, op.out0_buf, x), e, o0);
-    if (op.out1_buf != BUF_NONE) store1<T, A>(op.out1_buf, buf_ptr<A>(a, op.out1_buf, x), e, o1);
-  }
-  if (lv.bytes != nullptr) {
+    const int first = gi * lv.group;
+    const int count = min(lv.group, lv.nops - first);
+    StepOp op[kFlatGroup];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) moved_bytes += __shfl_down_sync(0xffffffffu, moved_bytes, off);
-    if ((threadIdx.x & 31) == 0 && moved_bytes) atomicAdd(lv.bytes + byte_slot(), moved_bytes);
+    for (int k = 0; k < kFlatGroup; ++k)
+      if (k < count) op[k] = lv.ops[first + k];
+    wait_prior_grid();
+    A r[kFlatGroup], o0[kFlatGroup], o1[kFlatGroup];
+#pragma unroll
+    for (int k = 0; k < kFlatGroup; ++k) {
+      if (k >= count) break;
+      const int x = a.xor_group ? (b ^ (int)op[k].dst_place) : wrap_rank(b + (int)op[k].dst_place, a.P);
+      r[k] = o0[k] = o1[k] = A(0);
+      if (op[k].recv_place >= 0) {
+        const int partner = a.xor_group ? (x ^ lv.partner) : wrap_rank(x + lv.partner, a.P);
+        r[k] = load1<T, A>(op[k].recv_buf, slot(op[k].recv_buf, partner), e);
+        moved += (op[k].recv_buf == BUF_RANK) ? sizeof(T) : sizeof(A);
+      }
+      if (op[k].out0_own != BUF_NONE) o0[k] = load1<T, A>(op[k].out0_own, slot(op[k].out0_own, x), e);
+      if (op[k].out1_own != BUF_NONE) o1[k] = load1<T, A>(op[k].out1_own, slot(op[k].out1_own, x), e);
+    }
+#pragma unroll
+    for (int k = 0; k < kFlatGroup; ++k) {
+      if (k >= count) break;
+      const int x = a.xor_group ? (b ^ (int)op[k].dst_place) : wrap_rank(b + (int)op[k].dst_place, a.P);
+      const bool has_recv = op[k].recv_place >= 0;
+      if (op[k].out0_own == BUF_NONE) o0[k] = r[k];
+      else if (has_recv) o0[k] = combine<OP>(o0[k], r[k]);
+      store1<T, A>(op[k].out0_buf, slot(op[k].out0_buf, x), e, o0[k]);
+      if (op[k].out1_buf != BUF_NONE) {
+        if (op[k].out1_own == BUF_NONE) o1[k] = r[k];
+        else if (has_recv) o1[k] = combine<OP>(o1[k], r[k]);
+        store1<T, A>(op[k].out1_buf, slot(op[k].out1_buf, x), e, o1[k]);
+      }
+    }
+  }
+  wait_prior_grid();  // threads without an item: the grid must not complete before its predecessor
+  // one atomic add per warp, of the bytes its threads read from partners
+  if (lv.bytes != nullptr) {
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, moved);
+    if ((threadIdx.x & 31) == 0 && sum)
+      atomicAdd(lv.bytes + (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) % STEP_BYTE_SLOTS,
+                (unsigned long long)sum);
   }
 }
 
@@ -455,33 +423,38 @@ __device__ __forceinline__ LaunchView view_of(const StepArgs<MAXP> &a) {
   lv.nops = a.nops;
   lv.partner = a.partner;
   lv.nchunks = a.nchunks;
+  lv.group = a.group;
   return lv;
 }
 
-// Programmatic dependent launch: the step launches of one Allreduce are made with
-// programmatic stream serialisation, so launch i+1's CTAs may become resident while
-// launch i drains.  griddepcontrol.wait blocks until every prerequisite grid has
-// completed and its memory is visible (a no-op without such a dependency); nothing is
-// read before it.  launch_dependents, issued once a CTA's work is done, lets the next
-// launch start once every CTA of this one has issued it or exited.
-__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void counter_upkeep(const CounterUpkeep &c) {
+  static_assert(STEP_BYTE_SLOTS <= kThreads, "one thread per counter slot");
+  if (threadIdx.x < STEP_BYTE_SLOTS) {
+    if (c.zero != nullptr) c.zero[threadIdx.x] = 0;
+    if (c.move_from != nullptr) c.move_to[threadIdx.x] = atomicExch(c.move_from + threadIdx.x, 0ull);
+  }
+}
 
 // At most 40 registers (6 CTAs per SM): the bf16 launches ran 5-8 % faster than at the
 // 48 registers the compiler picks unbounded, fp32 the same.
 template <typename T, int OP, int MAXP>
 __global__ void __launch_bounds__(kThreads, 6) step_kernel(const __grid_constant__ StepArgs<MAXP> a) {
   wait_prior_grid();
+  if (blockIdx.x == 0) counter_upkeep(a.upkeep);
   chunk_work<T, OP, MAXP>(a, view_of(a), blockIdx.x);
   allow_next_grid();
 }
 
 template <typename T, int OP, int MAXP>
 __global__ void __launch_bounds__(kThreads) step_kernel_flat(const __grid_constant__ StepArgs<MAXP> a) {
-  wait_prior_grid();
-  flat_work<T, OP, MAXP>(a, view_of(a), (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
+  __shared__ void *s_rank[MAXP];
+  if (a.early) allow_next_grid();
+  for (int x = threadIdx.x; x < a.P; x += kThreads) s_rank[x] = a.rank[x];
+  __syncthreads();
+  flat_work<T, OP, MAXP>(a, view_of(a), s_rank, (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
                          (uint64_t)gridDim.x * blockDim.x);
-  allow_next_grid();
+  if (blockIdx.x == 0) counter_upkeep(a.upkeep);
+  if (!a.early) allow_next_grid();
 }
 
 // Launches a step kernel with programmatic stream serialisation (see above).
@@ -509,21 +482,25 @@ cudaError_t launch_pdl(void (*kernel)(Args), unsigned grid, gar_stream_t stream,
 // with gar_plan_status.
 // ---------------------------------------------------------------------------
 
+// Device state of a plan's persistent launches, zero between launches but for the outcome:
+// the last CTA to leave a launch writes the outcome and resets the rest, so no memset
+// precedes a launch.
 struct BarrierState {
-  unsigned int count;   // CTA arrivals since the launch began (zeroed before each launch)
-  unsigned int unused;
+  unsigned int count;   // CTA arrivals since the launch began
+  unsigned int leaving; // CTAs that have finished
   int error;            // 1 once any CTA gave up waiting
   int error_launch;     // launch index after which the first timeout happened
+  int outcome;          // `error` and `error_launch` of the launch that ended last
+  int outcome_launch;
 };
 
 template <int MAXP>
 struct PersistArgs {
   StepArgs<MAXP> s;                 // buffers and sizes (s.ops = whole op table)
   const LaunchDesc *launches;
-  unsigned long long *step_bytes;   // per communication step, or nullptr
+  unsigned long long *step_bytes;   // S rows of STEP_BYTE_SLOTS counters, then the first step's own
   BarrierState *bar;
-  int nlaunch;
-  int flat;                         // element-major mapping (small blocks)
+  int nlaunch, nsteps;
   unsigned int spin_limit;          // polls before a wait gives up
   unsigned int phantom;             // arrivals expected beyond the grid (test hook, normally 0)
 };
@@ -576,28 +553,115 @@ __device__ bool grid_barrier(BarrierState *bar, unsigned expected, unsigned spin
   return s_ok != 0;
 }
 
-template <typename T, int OP, int MAXP>
-__global__ void __launch_bounds__(kThreads) step_kernel_persistent(const __grid_constant__ PersistArgs<MAXP> p) {
-  const unsigned expected = gridDim.x + p.phantom;
-  for (int l = 0; l < p.nlaunch; ++l) {
-    const LaunchDesc d = p.launches[l];
-    LaunchView lv;
-    lv.ops = p.s.ops + d.first_op;
-    lv.nops = d.nops;
-    lv.partner = d.partner;
-    lv.bytes = (p.step_bytes != nullptr && d.comm_step >= 0)
-                   ? p.step_bytes + (size_t)d.comm_step * STEP_BYTE_SLOTS : nullptr;
-    lv.chunk = p.s.chunk;
-    lv.nchunks = p.s.nchunks;
-    if (p.flat) {
-      flat_work<T, OP, MAXP>(p.s, lv, (uint64_t)blockIdx.x * blockDim.x + threadIdx.x,
-                             (uint64_t)gridDim.x * blockDim.x);
-    } else {
-      const uint64_t items = (uint64_t)lv.nchunks * (uint64_t)p.s.P * (uint64_t)lv.nops;
-      for (uint64_t item = blockIdx.x; item < items; item += gridDim.x)
-        chunk_work<T, OP, MAXP, false>(p.s, lv, item);
+// Counter row of a communication step: the step's own, but for the first step's, whose
+// counts wait in row nsteps until the second launch moves them (see CounterUpkeep).
+__host__ __device__ __forceinline__ unsigned long long *counter_row(unsigned long long *rows, int comm_step,
+                                                                    int nsteps) {
+  if (rows == nullptr || comm_step < 0) return nullptr;
+  return rows + (size_t)(comm_step == 0 ? nsteps : comm_step) * STEP_BYTE_SLOTS;
+}
+__host__ __device__ __forceinline__ CounterUpkeep upkeep_of(unsigned long long *rows, int launch, int next_comm_step,
+                                                            int nsteps) {
+  CounterUpkeep c{nullptr, nullptr, nullptr};
+  if (rows == nullptr) return c;
+  if (next_comm_step > 0) c.zero = rows + (size_t)next_comm_step * STEP_BYTE_SLOTS;
+  if (launch == 1) {
+    c.move_from = rows + (size_t)nsteps * STEP_BYTE_SLOTS;
+    c.move_to = rows;
+  }
+  return c;
+}
+
+// One step as a CTA of the persistent kernel sees it, fetched before the barrier that opens
+// it (the op table never changes), so that behind the barrier only the data is waited for.
+struct PersistStep {
+  LaunchDesc d;
+  uint32_t items, nchunks, chunk;  // nchunks pieces of `chunk` elements per block
+  StepOp op;                       // of the CTA's first item
+};
+
+template <int MAXP, bool FLAT>
+__device__ __forceinline__ PersistStep fetch_step(const PersistArgs<MAXP> &p, int l) {
+  PersistStep s{};
+  s.d = p.launches[l];
+  if (FLAT) return s;
+  // A step's blocks (P * nops of maxblk elements) are cut into equal pieces, as many as
+  // give every CTA one piece, or, where there are more blocks than CTAs, as many as waste
+  // least of the last round: every CTA reaches the barrier at about the same time.
+  const uint64_t maxblk = p.s.q + (p.s.rem ? 1 : 0);
+  const uint32_t blocks = (uint32_t)p.s.P * (uint32_t)max(1, s.d.nops);
+  uint32_t k = gridDim.x / blocks;
+  if (k == 0) {
+    uint64_t best = ~0ull;
+    for (uint32_t c = 1; c <= 4; ++c) {
+      const uint64_t cost = (uint64_t)((blocks * c + gridDim.x - 1) / gridDim.x) * (maxblk / c + kPieceCost);
+      if (cost < best) {
+        best = cost;
+        k = c;
+      }
     }
-    if (l + 1 < p.nlaunch && !grid_barrier(p.bar, expected, p.spin_limit, l)) return;
+  }
+  uint64_t chunk = ((maxblk + k - 1) / k + 7) / 8 * 8;
+  if (chunk < kMinPiece) chunk = kMinPiece;
+  s.chunk = (uint32_t)chunk;
+  s.nchunks = (uint32_t)((maxblk + chunk - 1) / chunk);
+  s.items = s.d.nops > 0 ? s.nchunks * blocks : 0;
+  if (blockIdx.x < s.items) s.op = p.s.ops[s.d.first_op + blockIdx.x / s.nchunks / (uint32_t)p.s.P];
+  return s;
+}
+
+// FLAT: element-major mapping (small blocks), else pieces of blocks.
+template <typename T, int OP, int MAXP, bool FLAT>
+__global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, FLAT ? 4 : kPersistPerSM)
+    step_kernel_persistent(const __grid_constant__ PersistArgs<MAXP> p) {
+  __shared__ void *s_rank[FLAT ? MAXP : 1];
+  if (FLAT) {
+    for (int x = threadIdx.x; x < p.s.P; x += kThreads) s_rank[x] = p.s.rank[x];
+    __syncthreads();
+  }
+  const unsigned expected = gridDim.x + p.phantom;
+  bool ok = true;
+  PersistStep st = fetch_step<MAXP, FLAT>(p, 0);
+  for (int l = 0; l < p.nlaunch && ok; ++l) {
+    LaunchView lv;
+    lv.ops = p.s.ops + st.d.first_op;
+    lv.nops = st.d.nops;
+    lv.partner = st.d.partner;
+    lv.bytes = counter_row(p.step_bytes, st.d.comm_step, p.nsteps);
+    lv.chunk = st.chunk;
+    lv.nchunks = (int)st.nchunks;
+    lv.group = st.d.group;
+    if (FLAT) {
+      flat_work<T, OP, MAXP>(p.s, lv, s_rank, (uint64_t)blockIdx.x * kThreads + threadIdx.x,
+                             (uint64_t)gridDim.x * kThreads);
+    } else {
+      for (uint32_t item = blockIdx.x; item < st.items; item += gridDim.x) {
+        const uint32_t blk = item / st.nchunks, op = blk / (uint32_t)p.s.P;
+        if (item != blockIdx.x) st.op = lv.ops[op];
+        range_work<T, OP, MAXP, kPersistThreads>(p.s, lv, st.op, (int)(blk - op * (uint32_t)p.s.P),
+                                                 (uint64_t)(item - blk * st.nchunks) * st.chunk, st.chunk);
+      }
+    }
+    if (l + 1 < p.nlaunch) {
+      st = fetch_step<MAXP, FLAT>(p, l + 1);
+      if (blockIdx.x == 0) counter_upkeep(upkeep_of(p.step_bytes, l, st.d.comm_step, p.nsteps));
+      ok = grid_barrier(p.bar, expected, p.spin_limit, l);
+    } else if (blockIdx.x == 0) {
+      counter_upkeep(upkeep_of(p.step_bytes, l, -1, p.nsteps));
+    }
+  }
+  // The last CTA to leave records the outcome and resets the state for the next launch; a
+  // launch that gave up also drops the first step's counts, which may not have been moved.
+  __syncthreads();
+  if (threadIdx.x == 0 && atom_add_acq_rel_gpu(&p.bar->leaving, 1u) == gridDim.x - 1) {
+    const int error = ld_relaxed_int(&p.bar->error);
+    p.bar->outcome = error;
+    p.bar->outcome_launch = p.bar->error_launch;
+    if (error != 0 && p.step_bytes != nullptr)
+      for (int k = 0; k < STEP_BYTE_SLOTS; ++k) p.step_bytes[(size_t)p.nsteps * STEP_BYTE_SLOTS + k] = 0;
+    p.bar->count = 0;
+    p.bar->leaving = 0;
+    p.bar->error = 0;
   }
 }
 
@@ -619,23 +683,37 @@ int num_sms() {
   return v;
 }
 
-template <typename T, int OP, int MAXP>
-int launch_typed(const gar_plan &pl, const Launch &ln, int launch_index, void *const *rank,
-                 gar_stream_t stream) {
-  (void)launch_index;
+// Elements per CTA of a chunked launch.  Distribution steps copy 2-byte elements with as
+// many bytes per CTA as fp32 chunks hold; launches of few CTAs take smaller chunks; a last
+// chunk shorter than 1/8 of a chunk is spread over the block's others (P = 127 x 8 MiB
+// bf16: blocks of 33,026 elements became 16,384 + 16,384 + 258, a third of the CTAs nearly
+// empty).
+uint32_t pick_chunk(uint64_t maxblk, int P, int nops, int phase, size_t elem_bytes) {
+  uint64_t chunk = (phase == 1 && elem_bytes == 2) ? 2 * kChunk : kChunk;
+  const uint64_t min_ctas = kMinCtas * (uint64_t)num_sms();
+  while (chunk > kMinChunk && ((maxblk + chunk - 1) / chunk) * P * nops < min_ctas) chunk /= 2;
+  const uint64_t nch = (maxblk + chunk - 1) / chunk;
+  if (nch > 1 && maxblk - (nch - 1) * chunk < chunk / 8) chunk = ((maxblk + nch - 2) / (nch - 1) + 7) / 8 * 8;
+  return (uint32_t)chunk;
+}
+
+// Ops per thread of an element-major launch: one while the device has a thread for every
+// (op, element), more beyond.
+int pick_group(uint64_t n, int nops) {
+  const uint64_t threads = kFlatThreads * (uint64_t)num_sms();
+  int group = 1;
+  while (group < kFlatGroup && (uint64_t)((nops + group - 1) / group) * n > threads) group *= 2;
+  return group;
+}
+
+template <int MAXP>
+StepArgs<MAXP> step_args(const gar_plan &pl, const Launch &ln, void *const *rank, void *workspace) {
   StepArgs<MAXP> a{};
   for (int x = 0; x < pl.P; ++x) a.rank[x] = rank[x];
   int slot = 0;
-  for (int k = 0; k < NUM_WS_BUFS; ++k) {
-    if (pl.ws_used[k]) {
-      a.ws[k] = static_cast<char *>(pl.ws) + (size_t)slot * pl.P * pl.n_pad * acc_size(pl.dtype);
-      ++slot;
-    } else {
-      a.ws[k] = nullptr;
-    }
-  }
-  a.ops = pl.d_ops + ln.first_op;
-  a.bytes = (ln.comm_step >= 0) ? pl.d_step_bytes + (size_t)ln.comm_step * STEP_BYTE_SLOTS : nullptr;
+  for (int k = 0; k < NUM_WS_BUFS; ++k)
+    if (pl.ws_used[k])
+      a.ws[k] = static_cast<char *>(workspace) + (size_t)(slot++) * pl.P * pl.n_pad * acc_size(pl.dtype);
   a.q = pl.q;
   a.rem = pl.rem;
   a.n_pad = pl.n_pad;
@@ -644,36 +722,49 @@ int launch_typed(const gar_plan &pl, const Launch &ln, int launch_index, void *c
   a.xor_group = pl.group == GAR_GROUP_XOR ? 1 : 0;
   a.partner = ln.partner;
   a.nops = ln.nops;
+  return a;
+}
+
+// Mapping and grid of one launch; *flat: element-major.
+template <int MAXP>
+int step_grid(const gar_plan &pl, const Launch &ln, StepArgs<MAXP> &a, bool *flat, unsigned *grid) {
   const uint64_t maxblk = pl.q + (pl.rem ? 1 : 0);
-  if (maxblk < kFlatBelow && ln.nops > 0 && pl.n > 0) {
+  *grid = 0;
+  *flat = maxblk < kFlatBelow;
+  if (maxblk == 0 || ln.nops == 0) return GAR_OK;
+  if (*flat) {
     // blocks shorter than one CTA's worth of vectors: element-major launch
-    const uint64_t total = (uint64_t)ln.nops * pl.n;
-    const uint64_t grid = std::min<uint64_t>((total + kThreads - 1) / kThreads,
-                                             (uint64_t)num_sms() * 32);
-    cudaError_t e = launch_pdl(step_kernel_flat<T, OP, MAXP>, (unsigned)grid, stream, a);
-    if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+    a.group = pick_group(pl.n, ln.nops);
+    const uint64_t total = (uint64_t)((ln.nops + a.group - 1) / a.group) * pl.n;
+    *grid = (unsigned)std::min<uint64_t>((total + kThreads - 1) / kThreads, (uint64_t)num_sms() * 32);
     return GAR_OK;
   }
-  // Distribution steps copy 2-byte elements with as many bytes per CTA as fp32 chunks
-  // hold; a last chunk shorter than 1/8 of a chunk is spread over the block's others (P =
-  // 127 x 8 MiB bf16: blocks of 33,026 elements became 16,384 + 16,384 + 258, a third of
-  // the CTAs nearly empty).
-  a.chunk = (ln.phase == 1 && sizeof(T) == 2) ? 2 * kChunk : kChunk;
-  const uint64_t min_ctas = 4 * (uint64_t)num_sms();
-  while (a.chunk > 4096 && ((maxblk + a.chunk - 1) / a.chunk) * pl.P * ln.nops < min_ctas) a.chunk /= 2;
-  {
-    const uint64_t nch = (maxblk + a.chunk - 1) / a.chunk;
-    if (nch > 1 && maxblk - (nch - 1) * a.chunk < a.chunk / 8)
-      a.chunk = ((maxblk + nch - 2) / (nch - 1) + 7) / 8 * 8;
-  }
+  a.chunk = pick_chunk(maxblk, pl.P, ln.nops, ln.phase, (size_t)elem_size(pl.dtype));
   a.nchunks = (int)((maxblk + a.chunk - 1) / a.chunk);
-  if (a.nchunks == 0 || ln.nops == 0) return GAR_OK;
-  const uint64_t grid = (uint64_t)a.nchunks * (uint64_t)pl.P * (uint64_t)ln.nops;
-  if (grid > 0x7fffffffull) {
+  const uint64_t g = (uint64_t)a.nchunks * (uint64_t)pl.P * (uint64_t)ln.nops;
+  if (g > 0x7fffffffull) {
     set_error("step launch grid too large");
     return GAR_EINVAL;
   }
-  cudaError_t e = launch_pdl(step_kernel<T, OP, MAXP>, (unsigned)grid, stream, a);
+  *grid = (unsigned)g;
+  return GAR_OK;
+}
+
+template <typename T, int OP, int MAXP>
+int launch_typed(const gar_plan &pl, const Launch &ln, int launch_index, void *const *rank,
+                 gar_stream_t stream) {
+  StepArgs<MAXP> a = step_args<MAXP>(pl, ln, rank, pl.ws);
+  a.ops = pl.d_ops + ln.first_op;
+  a.bytes = counter_row(pl.d_step_bytes, ln.comm_step, pl.S);
+  const bool last = launch_index + 1 == (int)pl.launches.size();
+  a.upkeep = upkeep_of(pl.d_step_bytes, launch_index, last ? -1 : pl.launches[launch_index + 1].comm_step, pl.S);
+  a.early = 0;
+  bool flat = false;
+  unsigned grid = 0;
+  if (int rc = step_grid(pl, ln, a, &flat, &grid)) return rc;
+  if (grid == 0) return GAR_OK;
+  const cudaError_t e = flat ? launch_pdl(step_kernel_flat<T, OP, MAXP>, grid, stream, a)
+                             : launch_pdl(step_kernel<T, OP, MAXP>, grid, stream, a);
   if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
   return GAR_OK;
 }
@@ -701,52 +792,34 @@ int launch_dt(const gar_plan &pl, const Launch &ln, int li, void *const *rank, g
 template <typename T, int OP, int MAXP>
 int launch_persistent_typed(const gar_plan &pl, void *const *rank, gar_stream_t stream) {
   PersistArgs<MAXP> p{};
-  for (int x = 0; x < pl.P; ++x) p.s.rank[x] = rank[x];
-  int slot = 0;
-  for (int k = 0; k < NUM_WS_BUFS; ++k)
-    p.s.ws[k] = pl.ws_used[k] ? static_cast<char *>(pl.ws) + (size_t)(slot++) * pl.P * pl.n_pad * acc_size(pl.dtype)
-                              : nullptr;
+  p.s = step_args<MAXP>(pl, pl.launches[0], rank, pl.ws);
   p.s.ops = pl.d_ops;
-  p.s.bytes = nullptr;
-  p.s.q = pl.q;
-  p.s.rem = pl.rem;
-  p.s.n_pad = pl.n_pad;
-  p.s.n = pl.n;
-  p.s.P = pl.P;
-  p.s.xor_group = pl.group == GAR_GROUP_XOR ? 1 : 0;
-  const uint64_t maxblk = pl.q + (pl.rem ? 1 : 0);
-  p.flat = maxblk < kFlatBelow ? 1 : 0;
-  // chunks as the per-step launches choose them for their largest step: small vectors
-  // drop to 8192 or 4096 elements so that the grid has work for every CTA it can hold
-  int max_ops = 1;
-  for (const Launch &ln : pl.launches) max_ops = std::max(max_ops, ln.nops);
-  p.s.chunk = kChunk;
-  const uint64_t min_items = 4 * (uint64_t)num_sms();
-  while (p.s.chunk > 4096 && ((maxblk + p.s.chunk - 1) / p.s.chunk) * pl.P * max_ops < min_items) p.s.chunk /= 2;
-  p.s.nchunks = (int)((maxblk + p.s.chunk - 1) / p.s.chunk);
   p.launches = static_cast<const LaunchDesc *>(pl.d_launches);
   p.step_bytes = pl.d_step_bytes;
   p.bar = static_cast<BarrierState *>(pl.d_barrier);
   p.nlaunch = (int)pl.launches.size();
+  p.nsteps = pl.S;
   p.spin_limit = pl.barrier_spin_limit;
   p.phantom = pl.barrier_phantom;
-  const void *fn = (const void *)step_kernel_persistent<T, OP, MAXP>;
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, 0);
-  if (e != cudaSuccess || per_sm < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
-                                                       "persistent kernel occupancy");
-  // As many CTAs as the largest step has work items (one chunk of one block op, or 256
-  // element-major items), at most the co-resident maximum: a small Allreduce then waits
-  // at its barriers for a few CTAs instead of three per SM.
+  // As many CTAs as the largest step has work items, at most the co-resident maximum: a
+  // small Allreduce then waits at its barriers for a few CTAs instead of several per SM.
+  const uint64_t maxblk = pl.q + (pl.rem ? 1 : 0);
+  const bool flat = maxblk < kFlatBelow;
   uint64_t need = 1;
   for (const Launch &ln : pl.launches) {
-    const uint64_t items = p.flat ? ((uint64_t)ln.nops * pl.n + kThreads - 1) / kThreads
-                                  : (uint64_t)p.s.nchunks * (uint64_t)pl.P * (uint64_t)ln.nops;
-    need = std::max(need, items);
+    const int group = pick_group(pl.n, ln.nops);
+    need = std::max<uint64_t>(need, flat ? ((uint64_t)((ln.nops + group - 1) / group) * pl.n + kThreads - 1) / kThreads
+                                         : (uint64_t)ln.nops * pl.P * ((maxblk + kMinPiece - 1) / kMinPiece));
   }
+  const void *fn = flat ? (const void *)step_kernel_persistent<T, OP, MAXP, true>
+                        : (const void *)step_kernel_persistent<T, OP, MAXP, false>;
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, flat ? kThreads : kPersistThreads, 0);
+  if (e != cudaSuccess || per_sm < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
+                                                       "persistent kernel occupancy");
   const unsigned grid = (unsigned)std::min<uint64_t>(need, (uint64_t)per_sm * (uint64_t)num_sms());
   void *args[] = {&p};
-  e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kThreads), args, 0, (cudaStream_t)stream);
+  e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(flat ? kThreads : kPersistThreads), args, 0, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "persistent kernel launch");
   return GAR_OK;
 }
@@ -786,6 +859,16 @@ int launch_persistent(const gar_plan &pl, void *const *rank, gar_stream_t stream
 
 size_t barrier_state_bytes() { return sizeof(BarrierState); }
 
+void barrier_outcome(const void *state, int *error, int *launch) {
+  const BarrierState *st = static_cast<const BarrierState *>(state);
+  *error = st->outcome;
+  *launch = st->outcome_launch;
+}
+
+LaunchDesc launch_desc(const gar_plan &pl, const Launch &ln) {
+  return {ln.first_op, ln.nops, ln.partner, ln.comm_step, pick_group(pl.n, ln.nops)};
+}
+
 }  // namespace gar
 
 // ---------------------------------------------------------------------------
@@ -812,87 +895,30 @@ namespace {
 constexpr int kNoAllocMaxOps = 2 * GAR_NOALLOC_MAX_P;  // |transmit set| + K <= 2P per launch
 
 struct NoAllocArgs {
-  void *rank[GAR_NOALLOC_MAX_P];
-  void *ws[NUM_WS_BUFS];
+  StepArgs<GAR_NOALLOC_MAX_P> s;
   StepOp ops[kNoAllocMaxOps];
-  uint64_t q, rem, n_pad;
-  int P, partner, nops, nchunks;
 };
 
-template <typename A>
-__device__ __forceinline__ void *na_buf_ptr(const NoAllocArgs &a, uint8_t buf, int rank) {
-  if (buf == BUF_RANK) return a.rank[rank];
-  if (buf == BUF_NONE) return nullptr;
-  return static_cast<char *>(a.ws[buf - BUF_QP0]) + (uint64_t)rank * a.n_pad * sizeof(A);
+// The step kernels' work with the ops read from the parameter block and no byte counting.
+template <typename T, int OP>
+__global__ void __launch_bounds__(kThreads, 6) step_kernel_noalloc(const __grid_constant__ NoAllocArgs a) {
+  LaunchView lv = view_of(a.s);
+  lv.ops = a.ops;
+  wait_prior_grid();
+  chunk_work<T, OP>(a.s, lv, blockIdx.x);
+  allow_next_grid();
 }
 
-// Same block-op semantics as step_kernel (one CTA per op x rank x chunk), with the ops
-// read from the parameter block and no byte counting.
 template <typename T, int OP>
-__global__ void __launch_bounds__(kThreads) step_kernel_noalloc(const __grid_constant__ NoAllocArgs a) {
-  using A = typename AccOf<T>::type;
-  uint64_t bid = blockIdx.x;
-  const int chunk = (int)(bid % (uint64_t)a.nchunks);
-  bid /= (uint64_t)a.nchunks;
-  const int x = (int)(bid % (uint64_t)a.P);
-  const int oi = (int)(bid / (uint64_t)a.P);
-  if (oi >= a.nops) return;
-  const StepOp op = a.ops[oi];
-  const int b = ((x - (int)op.dst_place) % a.P + a.P) % a.P;
-  const uint64_t bstart = (uint64_t)b * a.q + ((uint64_t)b < a.rem ? (uint64_t)b : a.rem);
-  const uint64_t blen = a.q + ((uint64_t)b < a.rem ? 1 : 0);
-  const uint64_t c0 = (uint64_t)chunk * kChunk;
-  if (c0 >= blen) return;
-  const uint64_t lo = bstart + c0;
-  const uint64_t hi = bstart + (blen < c0 + kChunk ? blen : c0 + kChunk);
-  const bool has_recv = op.recv_place >= 0;
-  const int partner = ((x + a.partner) % a.P + a.P) % a.P;
-  const void *recv = has_recv ? na_buf_ptr<A>(a, op.recv_buf, partner) : nullptr;
-  void *out0 = na_buf_ptr<A>(a, op.out0_buf, x);
-  const void *own0 = na_buf_ptr<A>(a, op.out0_own, x);
-  void *out1 = na_buf_ptr<A>(a, op.out1_buf, x);
-  const void *own1 = na_buf_ptr<A>(a, op.out1_own, x);
-
-  auto result = [&](const void *own, uint8_t own_buf, uint64_t e, A r) -> A {
-    if (!own) return r;
-    const A o = load1<T, A>(own_buf, own, e);
-    return has_recv ? combine<OP>(o, r) : o;
-  };
-  auto do1 = [&](uint64_t e) {
-    const A r = has_recv ? load1<T, A>(op.recv_buf, recv, e) : A(0);
-    const A o0 = result(own0, op.out0_own, e, r);
-    const A o1 = out1 ? result(own1, op.out1_own, e, r) : r;
-    store1<T, A>(op.out0_buf, out0, e, o0);
-    if (out1) store1<T, A>(op.out1_buf, out1, e, o1);
-  };
-  auto do4 = [&](uint64_t e) {
-    A r[4] = {A(0), A(0), A(0), A(0)};
-    if (has_recv) load4<T, A>(op.recv_buf, recv, e, r);
-    A o0[4], o1[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) o0[k] = o1[k] = r[k];
-    if (own0) {
-      load4<T, A>(op.out0_own, own0, e, o0);
-      if (has_recv)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o0[k] = combine<OP>(o0[k], r[k]);
-    }
-    if (out1 && own1) {
-      load4<T, A>(op.out1_own, own1, e, o1);
-      if (has_recv)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o1[k] = combine<OP>(o1[k], r[k]);
-    }
-    store4<T, A>(op.out0_buf, out0, e, o0);
-    if (out1) store4<T, A>(op.out1_buf, out1, e, o1);
-  };
-  uint64_t va = (lo + 3) & ~uint64_t(3);
-  uint64_t vb = hi & ~uint64_t(3);
-  if (va > hi) va = hi;
-  if (vb < va) vb = va;
-  for (uint64_t e = lo + threadIdx.x; e < va; e += blockDim.x) do1(e);
-  for (uint64_t e = va + 4 * (uint64_t)threadIdx.x; e < vb; e += 4 * (uint64_t)blockDim.x) do4(e);
-  for (uint64_t e = vb + threadIdx.x; e < hi; e += blockDim.x) do1(e);
+__global__ void __launch_bounds__(kThreads) step_kernel_noalloc_flat(const __grid_constant__ NoAllocArgs a) {
+  __shared__ void *s_rank[GAR_NOALLOC_MAX_P];
+  if (a.s.early) allow_next_grid();
+  for (int x = threadIdx.x; x < a.s.P; x += kThreads) s_rank[x] = a.s.rank[x];
+  __syncthreads();
+  LaunchView lv = view_of(a.s);
+  lv.ops = a.ops;
+  flat_work<T, OP>(a.s, lv, s_rank, (uint64_t)blockIdx.x * kThreads + threadIdx.x, (uint64_t)gridDim.x * kThreads);
+  if (!a.s.early) allow_next_grid();
 }
 
 // Device address of the scratch array on the current device, looked up on every call
@@ -919,44 +945,27 @@ int noalloc_scratch(void **out) {
 }
 
 template <typename T, int OP>
-int noalloc_launch(const gar_plan &pl, const Launch &ln, void *const *rank, void *scratch,
-                   gar_stream_t stream) {
+int noalloc_launch(const gar_plan &pl, int launch_index, void *const *rank, void *scratch, gar_stream_t stream) {
+  const Launch &ln = pl.launches[launch_index];
   NoAllocArgs a{};
-  for (int x = 0; x < pl.P; ++x) a.rank[x] = rank[x];
-  int slot = 0;
-  for (int k = 0; k < NUM_WS_BUFS; ++k) {
-    a.ws[k] = pl.ws_used[k] ? static_cast<char *>(scratch) +
-                                  (size_t)(slot++) * pl.P * pl.n_pad * acc_size(pl.dtype)
-                            : nullptr;
-  }
+  a.s = step_args<GAR_NOALLOC_MAX_P>(pl, ln, rank, scratch);
   for (int k = 0; k < ln.nops; ++k) a.ops[k] = pl.ops[ln.first_op + k];
-  a.q = pl.q;
-  a.rem = pl.rem;
-  a.n_pad = pl.n_pad;
-  a.P = pl.P;
-  a.partner = ln.partner;
-  a.nops = ln.nops;
-  const uint64_t maxblk = pl.q + (pl.rem ? 1 : 0);
-  a.nchunks = (int)((maxblk + kChunk - 1) / kChunk);
-  if (a.nchunks == 0 || ln.nops == 0) return GAR_OK;
-  const uint64_t grid = (uint64_t)a.nchunks * (uint64_t)pl.P * (uint64_t)ln.nops;
-  if (grid > 0x7fffffffull) {
-    set_error("no-allocation step launch grid too large");
-    return GAR_EINVAL;
-  }
-  step_kernel_noalloc<T, OP><<<(unsigned)grid, kThreads, 0, (cudaStream_t)stream>>>(a);
-  cudaError_t e = cudaGetLastError();
+  bool flat = false;
+  unsigned grid = 0;
+  if (int rc = step_grid(pl, ln, a.s, &flat, &grid)) return rc;
+  if (grid == 0) return GAR_OK;
+  const cudaError_t e = flat ? launch_pdl(step_kernel_noalloc_flat<T, OP>, grid, stream, a)
+                             : launch_pdl(step_kernel_noalloc<T, OP>, grid, stream, a);
   if (e != cudaSuccess) return cuda_fail(e, "no-allocation step kernel launch");
   return GAR_OK;
 }
 
 template <typename T>
-int noalloc_launch_op(const gar_plan &pl, const Launch &ln, void *const *rank, void *scratch,
-                      gar_stream_t s) {
+int noalloc_launch_op(const gar_plan &pl, int li, void *const *rank, void *scratch, gar_stream_t s) {
   switch (pl.op) {
-    case GAR_SUM: return noalloc_launch<T, GAR_SUM>(pl, ln, rank, scratch, s);
-    case GAR_MAX: return noalloc_launch<T, GAR_MAX>(pl, ln, rank, scratch, s);
-    case GAR_MIN: return noalloc_launch<T, GAR_MIN>(pl, ln, rank, scratch, s);
+    case GAR_SUM: return noalloc_launch<T, GAR_SUM>(pl, li, rank, scratch, s);
+    case GAR_MAX: return noalloc_launch<T, GAR_MAX>(pl, li, rank, scratch, s);
+    case GAR_MIN: return noalloc_launch<T, GAR_MIN>(pl, li, rank, scratch, s);
   }
   return GAR_EINVAL;
 }
@@ -1009,11 +1018,11 @@ extern "C" int gar_allreduce_noalloc(gar_plan *pl, void *const *rank_buffers, ga
   void *scratch = nullptr;
   int rc = noalloc_scratch(&scratch);
   if (rc) return rc;
-  for (const Launch &ln : pl->launches) {
+  for (int li = 0; li < (int)pl->launches.size(); ++li) {
     switch (pl->dtype) {
-      case GAR_F32: rc = noalloc_launch_op<float>(*pl, ln, rank_buffers, scratch, stream); break;
-      case GAR_BF16: rc = noalloc_launch_op<__nv_bfloat16>(*pl, ln, rank_buffers, scratch, stream); break;
-      case GAR_I32: rc = noalloc_launch_op<int>(*pl, ln, rank_buffers, scratch, stream); break;
+      case GAR_F32: rc = noalloc_launch_op<float>(*pl, li, rank_buffers, scratch, stream); break;
+      case GAR_BF16: rc = noalloc_launch_op<__nv_bfloat16>(*pl, li, rank_buffers, scratch, stream); break;
+      case GAR_I32: rc = noalloc_launch_op<int>(*pl, li, rank_buffers, scratch, stream); break;
       default: rc = GAR_EINVAL;
     }
     if (rc) return rc;
