@@ -177,6 +177,9 @@ __device__ __forceinline__ int wrap_rank(int v, int P) { return v < 0 ? v + P : 
 // it or exited.  Chunked launches issue it when their work is done: at the start, the
 // waiting CTAs took slots from the running ones' (P = 127 x 8 MiB bf16 S = 14 1122 us
 // instead of 1112, P = 20 x 1 MiB fp32 S = 9 without allocation 37.6 instead of 34.3).
+// Element-major launches, whose CTAs are few and short, issue it at the start (P = 127 x
+// 9 KiB bf16 S = 10 34.0 instead of 36.4), but for a call's last launch, whose successor
+// is not ours.
 __device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -758,7 +761,7 @@ int launch_typed(const gar_plan &pl, const Launch &ln, int launch_index, void *c
   a.bytes = counter_row(pl.d_step_bytes, ln.comm_step, pl.S);
   const bool last = launch_index + 1 == (int)pl.launches.size();
   a.upkeep = upkeep_of(pl.d_step_bytes, launch_index, last ? -1 : pl.launches[launch_index + 1].comm_step, pl.S);
-  a.early = 0;
+  a.early = last ? 0 : 1;
   bool flat = false;
   unsigned grid = 0;
   if (int rc = step_grid(pl, ln, a, &flat, &grid)) return rc;
@@ -950,6 +953,7 @@ int noalloc_launch(const gar_plan &pl, int launch_index, void *const *rank, void
   NoAllocArgs a{};
   a.s = step_args<GAR_NOALLOC_MAX_P>(pl, ln, rank, scratch);
   for (int k = 0; k < ln.nops; ++k) a.ops[k] = pl.ops[ln.first_op + k];
+  a.s.early = launch_index + 1 < (int)pl.launches.size() ? 1 : 0;
   bool flat = false;
   unsigned grid = 0;
   if (int rc = step_grid(pl, ln, a.s, &flat, &grid)) return rc;
