@@ -444,7 +444,7 @@ template <typename T, int OP, int MAXP>
 __global__ void __launch_bounds__(kThreads, 6) step_kernel(const __grid_constant__ StepArgs<MAXP> a) {
   wait_prior_grid();
   if (blockIdx.x == 0) counter_upkeep(a.upkeep);
-  chunk_work<T, OP, MAXP>(a, view_of(a), blockIdx.x);
+  chunk_work<T, OP, MAXP>(a, view_of(a), a.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
   allow_next_grid();
 }
 
@@ -762,6 +762,7 @@ int launch_typed(const gar_plan &pl, const Launch &ln, int launch_index, void *c
   const bool last = launch_index + 1 == (int)pl.launches.size();
   a.upkeep = upkeep_of(pl.d_step_bytes, launch_index, last ? -1 : pl.launches[launch_index + 1].comm_step, pl.S);
   a.early = last ? 0 : 1;
+  a.reverse = launch_index & 1;
   bool flat = false;
   unsigned grid = 0;
   if (int rc = step_grid(pl, ln, a, &flat, &grid)) return rc;
@@ -908,7 +909,7 @@ __global__ void __launch_bounds__(kThreads, 6) step_kernel_noalloc(const __grid_
   LaunchView lv = view_of(a.s);
   lv.ops = a.ops;
   wait_prior_grid();
-  chunk_work<T, OP>(a.s, lv, blockIdx.x);
+  chunk_work<T, OP>(a.s, lv, a.s.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
   allow_next_grid();
 }
 
@@ -954,6 +955,7 @@ int noalloc_launch(const gar_plan &pl, int launch_index, void *const *rank, void
   a.s = step_args<GAR_NOALLOC_MAX_P>(pl, ln, rank, scratch);
   for (int k = 0; k < ln.nops; ++k) a.ops[k] = pl.ops[ln.first_op + k];
   a.s.early = launch_index + 1 < (int)pl.launches.size() ? 1 : 0;
+  a.s.reverse = launch_index & 1;
   bool flat = false;
   unsigned grid = 0;
   if (int rc = step_grid(pl, ln, a.s, &flat, &grid)) return rc;
