@@ -273,6 +273,23 @@ int grid_for(const JitKernel *k, uint64_t work_items) {
   return (int)std::max<uint64_t>(1, std::min<uint64_t>(need, cap));
 }
 
+// Most CTAs of a fused kernel that works on host memory over NVLink-C2C.  The link needs
+// about 3 MB of loads in flight; with a thread for every vector (tens of MB in flight) all
+// reads were queued first and the writes came after them, so the two directions of the
+// link hardly overlapped.  A thread has at most its P vectors in flight, and at most what
+// its registers hold.  GB300, fused from and to pinned memory, a thread per vector -> this
+// rule: P = 24 x 4 MiB fp32 871 -> 645 us (231 -> 312 GB/s), 24 x 16 MiB 2960 -> 2460
+// (327 GB/s), 24 x 1 MiB 238 -> 180, P = 5 x 8 MiB bf16 348 -> 262, P = 64 x 1 MiB fp32
+// latency-optimal 637 -> 480, P = 127 x 1 MiB bf16 1186 -> 860; half or twice the 3 MB cost
+// up to 10 %.
+int host_grid(const gar_plan &pl) {
+  const JitKernel *k = pl.fused;
+  uint64_t per_thread = (uint64_t)pl.P * (uint64_t)k->width * (uint64_t)elem_size(pl.dtype);
+  if (k->regs > 0) per_thread = std::min<uint64_t>(per_thread, 4 * (uint64_t)k->regs);
+  const uint64_t per_cta = per_thread * (uint64_t)k->threads;
+  return (int)std::max<uint64_t>(1, (3000000 + per_cta - 1) / per_cta);
+}
+
 // Launches a generated kernel with programmatic stream serialisation: back-to-back
 // calls overlap one launch's start with the previous one's drain.  Every generated
 // kernel runs griddepcontrol.wait before its first read, so it still sees all the work
@@ -294,7 +311,7 @@ cudaError_t launch_generated(const JitKernel *k, int grid, void **kargs, gar_str
 // kernel's vector width).  The parameter block is the generated kernel's gar_args:
 // P input pointers, P output pointers, e_lo, e_hi.
 int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, uint64_t e_lo,
-                       uint64_t e_hi, gar_stream_t stream) {
+                       uint64_t e_hi, gar_stream_t stream, bool host_memory = false) {
   if (e_hi <= e_lo) return GAR_OK;
   // gar_args: the in[] table, then the out[] table, each table_copies times in a row,
   // then e_lo, e_hi
@@ -311,7 +328,8 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
   // (two-lane form)
   const uint64_t items = pl->fused->form == GAR_FORM_SPLIT ? (e_hi - e_lo + 15) / 16 * 32
                                                            : (e_hi - e_lo) / pl->fused->width + 1;
-  const int grid = grid_for(pl->fused, items);
+  int grid = grid_for(pl->fused, items);
+  if (host_memory) grid = std::min(grid, host_grid(*pl));
   cudaError_t e = launch_generated(pl->fused, grid, kargs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
   return GAR_OK;
@@ -711,7 +729,7 @@ int gar_allreduce_host(gar_plan *pl, const void *const *host_in, void *const *ho
       // The kernel reads the inputs from and writes the results to host memory itself.
       int rc = prepare_fused(pl);
       if (rc) return rc;
-      return launch_fused_range(pl, host_in, host_out, 0, pl->n, stream);
+      return launch_fused_range(pl, host_in, host_out, 0, pl->n, stream, true);
     }
     if (int rc = check_buffers(pl, dev_bufs)) return rc;
     return run_host_pipelined(pl, host_in, host_out, dev_bufs, stream);
