@@ -129,7 +129,7 @@ typedef struct {
   int32_t fused_local_bytes; /* local (spill) bytes per thread of the loaded fused kernel */
   int32_t group;             /* GAR_GROUP_CYCLIC or GAR_GROUP_XOR */
   int32_t ring;              /* 1 for the Ring schedule (GAR_STEPS_RING) */
-  int32_t fused_form;        /* fused kernel the plan uses: GAR_FORM_SINGLE, _BREADTH or _SPLIT */
+  int32_t fused_form;        /* fused kernel the plan uses: GAR_FORM_* */
 } gar_plan_info;
 
 /* Values of gar_plan_info.fused_form.  GAR_FORM_SINGLE: each thread evaluates the whole
@@ -143,8 +143,12 @@ typedef struct {
  * receiving the vectors a step moves across the halves by a warp shuffle; defined for
  * latency-optimal cyclic schedules (every placement holds its own result copy) and
  * taken only when forced (environment GAR_TUNE_FUSED_FORM=2): on GB300 it was slower
- * than the breadth-first form.  All forms give the same bits. */
-enum { GAR_FORM_SINGLE = 0, GAR_FORM_BREADTH = 1, GAR_FORM_SPLIT = 2 };
+ * than the breadth-first form.  GAR_FORM_STREAM: the program as a stream over placements
+ * with the contributions in shared memory; a prepared plan (gar_plan_prepare or a first
+ * fused call) of a bf16 sum that would take the breadth-first form runs it from 2^19
+ * elements per rank on, an fp32 sum with more than 210 values alive from 2^20 on; before
+ * that its info and source are the breadth-first form's.  All forms give the same bits. */
+enum { GAR_FORM_SINGLE = 0, GAR_FORM_BREADTH = 1, GAR_FORM_SPLIT = 2, GAR_FORM_STREAM = 3 };
 
 /* Creates a schedule for P virtual ranks of n elements each.
  * P: 1..GAR_MAX_P.  n: elements per rank (0 is allowed: every call is a no-op).
@@ -223,7 +227,8 @@ GAR_API int gar_plan_set_workspace(gar_plan *plan, void *dev_ptr, size_t bytes);
 
 /* The CUDA C source of the plan's generated fused kernel (host-only): of the kernel the
  * plan runs once it is prepared (gar_plan_prepare or a first fused call, which rebuild a
- * kernel of more than 128 registers in 64-thread CTAs), else of its first compile.
+ * kernel of more than 128 registers in 64-thread CTAs, and choose the streaming form),
+ * else of its first compile.
  * Copies at most
  * *len bytes (including the terminating NUL) to buf and sets *len to the full size
  * including the NUL; pass buf == NULL to query the size. */
@@ -284,10 +289,11 @@ typedef struct {
 GAR_API int gar_allreduce_batched(gar_plan *const *plans, int nplans, const gar_batch_desc *desc,
                           int count, gar_stream_t stream);
 
-/* Outcome of the plan's most recent GAR_STEP_PERSISTENT Allreduce (no counterpart in
- * the paper: failure reporting of the bounded waits): waits for the stream it ran on,
- * then returns GAR_OK, GAR_ETIMEOUT if a grid-barrier wait gave up (the results are then
- * incomplete), or GAR_ECUDA.  GAR_OK if no persistent call ran. */
+/* Outcome of the plan's most recent GAR_STEP_PERSISTENT Allreduce, and of its fused ones
+ * in the streaming form (no counterpart in the paper: failure reporting of the bounded
+ * waits): waits for the stream it ran on, then returns GAR_OK, GAR_ETIMEOUT if a grid-barrier
+ * wait, or a streaming kernel's wait for its own copies (10 s), gave up (the results are
+ * then incomplete), or GAR_ECUDA.  GAR_OK if no such call ran. */
 GAR_API int gar_plan_status(gar_plan *plan);
 
 /* Barrier parameters of GAR_STEP_PERSISTENT (no counterpart in the paper).  spin_limit: polls (each an L2 round trip,

@@ -139,6 +139,7 @@ int fused_form(const gar_plan &pl) {
   const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
   if (ff && *ff) {
     const int f = std::atoi(ff);
+    if (f == GAR_FORM_STREAM) return stream_form_applies(pl) ? GAR_FORM_STREAM : GAR_FORM_BREADTH;
     if (f == GAR_FORM_SPLIT) return split_form_applies(pl) ? GAR_FORM_SPLIT : GAR_FORM_BREADTH;
     return f == GAR_FORM_BREADTH ? GAR_FORM_BREADTH : GAR_FORM_SINGLE;
   }
@@ -150,6 +151,7 @@ CodegenResult fused_codegen(const gar_plan &pl) {
   switch (fused_form(pl)) {
     case GAR_FORM_BREADTH: return generate_fused_bf_source(pl);
     case GAR_FORM_SPLIT: return generate_fused_split_source(pl);
+    case GAR_FORM_STREAM: return generate_fused_stream_source(pl);
     default: return generate_fused_source(pl);
   }
 }
@@ -186,8 +188,50 @@ int compile_fused(gar_plan *pl) {
 // P = 64 x 16 MiB bf16 S = 8 (96 B: 0.324 against 0.346), P = 127 S = 9 (48 B: 0.407
 // against 0.460).
 // The counts are the loaded kernel's own (the compiler's log does not always carry them).
-int prepare_fused(gar_plan *pl) {
-  int rc = compile_fused(pl);
+// Whether a prepared plan runs the streaming form (cyclic programs in long vectors).  bf16
+// sums that would take the breadth-first form do from 2^19 positions on (GB300, against the
+// breadth-first form, P = 84 to 127 at S = 7 and 8: 1.13 to 1.67 times as fast from 2^19 to
+// 2^22 positions; 0.91 to 1.21 at 2^18, where an SM has too few tiles); fp32 sums only with
+// more than 210 values alive (P = 110 to 127 at S = 7 1.05 to 1.5 times as fast from 2^20
+// positions on, 0.97 to 0.99 at 2^19; P = 100 0.89, P = 127 S = 8 0.89).  Other programs
+// fit their registers and run at HBM rate as they are (P = 24 to 64: 0.81 to 0.98), as do
+// max, min and int32 (0.92 to 1.27, no clear line).
+bool takes_stream(const gar_plan &pl) {
+  const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
+  if (ff && *ff) return false;
+  if (pl.op != GAR_SUM || pl.dtype == GAR_I32 || pl.n < (1u << 19) || !stream_form_applies(pl)) return false;
+  const int live = fused_peak_live(pl);
+  return pl.dtype == GAR_BF16 ? live > 160 : live > 210 && pl.n >= (1u << 20);
+}
+
+int prepare_stream(gar_plan *pl) {
+  JitKernel *k = nullptr;
+  for (int groups = 0;;) {
+    CodegenResult cg;
+    try {
+      cg = generate_fused_stream_source(*pl, groups);
+    } catch (const std::exception &ex) {
+      set_error(std::string("fused code generation: ") + ex.what());
+      return GAR_EINVAL;
+    }
+    if (int rc = jit_compile(cg, &k)) return rc;
+    if (int rc = jit_load(k)) return rc;
+    groups = k->threads / 128 - 1;
+    if (k->local_bytes == 0 || groups < 2) break;  // spilled: one group less, with its registers
+  }
+  pl->fused = k;
+  pl->fused_width = k->width;
+  return GAR_OK;
+}
+
+int build_fused(gar_plan *pl) {
+  int rc = check_fused_size(pl);
+  if (rc) return rc;
+  if (takes_stream(*pl)) {
+    if ((rc = ensure_device(pl))) return rc;
+    return prepare_stream(pl);
+  }
+  rc = compile_fused(pl);
   if (rc) return rc;
   rc = ensure_device(pl);
   if (rc) return rc;
@@ -226,6 +270,14 @@ int prepare_fused(gar_plan *pl) {
   }
   pl->fused = k;
   pl->fused_width = k->width;
+  return GAR_OK;
+}
+
+// The plan's fused kernel, chosen, compiled and loaded once.
+int prepare_fused(gar_plan *pl) {
+  if (pl->fused_ready) return ensure_device(pl);
+  if (int rc = build_fused(pl)) return rc;
+  pl->fused_ready = true;
   return GAR_OK;
 }
 
@@ -286,7 +338,7 @@ int host_grid(const gar_plan &pl) {
   const JitKernel *k = pl.fused;
   uint64_t per_thread = (uint64_t)pl.P * (uint64_t)k->width * (uint64_t)elem_size(pl.dtype);
   if (k->regs > 0) per_thread = std::min<uint64_t>(per_thread, 4 * (uint64_t)k->regs);
-  const uint64_t per_cta = per_thread * (uint64_t)k->threads;
+  const uint64_t per_cta = k->tile > 0 ? (uint64_t)k->smem : per_thread * (uint64_t)k->threads;
   return (int)std::max<uint64_t>(1, (3000000 + per_cta - 1) / per_cta);
 }
 
@@ -298,6 +350,7 @@ cudaError_t launch_generated(const JitKernel *k, int grid, void **kargs, gar_str
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(k->threads);
+  cfg.dynamicSmemBytes = (size_t)k->smem;
   cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -329,9 +382,17 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
   const uint64_t items = pl->fused->form == GAR_FORM_SPLIT ? (e_hi - e_lo + 15) / 16 * 32
                                                            : (e_hi - e_lo) / pl->fused->width + 1;
   int grid = grid_for(pl->fused, items);
+  if (pl->fused->tile > 0) {  // persistent: as many CTAs as the device holds at once
+    const uint64_t tiles = std::max<uint64_t>(1, (e_hi - e_lo + pl->fused->tile - 1) / pl->fused->tile);
+    grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms() * (uint64_t)pl->fused->blocks_per_sm);
+  }
   if (host_memory) grid = std::min(grid, host_grid(*pl));
   cudaError_t e = launch_generated(pl->fused, grid, kargs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
+  if (pl->fused->stuck != nullptr) {
+    pl->fused_stream = stream;
+    pl->ran_waiting = true;
+  }
   return GAR_OK;
 }
 
@@ -817,8 +878,23 @@ int gar_last_step_bytes(const gar_plan *pl, uint64_t *per_step) {
 
 int gar_plan_status(gar_plan *pl) {
   if (int rc = check_plan(pl)) return rc;
+  cudaError_t e = cudaSuccess;
+  if (pl->ran_waiting && pl->fused != nullptr && pl->fused->stuck != nullptr) {
+    e = cudaStreamSynchronize((cudaStream_t)pl->fused_stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    unsigned int stuck = 0;
+    e = cudaMemcpy(&stuck, pl->fused->stuck, sizeof stuck, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(wait state)");
+    pl->ran_waiting = false;
+    if (stuck != 0) {
+      e = cudaMemset(pl->fused->stuck, 0, sizeof stuck);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaMemset(wait state)");
+      set_error("fused kernel: a wait for a tile gave up");
+      return GAR_ETIMEOUT;
+    }
+  }
   if (!pl->ran_persistent || pl->d_barrier == nullptr) return GAR_OK;
-  cudaError_t e = cudaStreamSynchronize((cudaStream_t)pl->last_stream);
+  e = cudaStreamSynchronize((cudaStream_t)pl->last_stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
   std::vector<char> state(barrier_state_bytes());
   e = cudaMemcpy(state.data(), pl->d_barrier, state.size(), cudaMemcpyDeviceToHost);

@@ -172,7 +172,8 @@ template <> __device__ __forceinline__ void gar_store<4>(gar_io *p, const gar_ac
 // suffix of the global loads / stores (default ".cs", streaming); GAR_TUNE_DOUBLED (0 or
 // 1): whether a rotated cyclic single-thread kernel stores its pointer tables twice;
 // GAR_TUNE_BF_ORDER / _BF_WARPS / _BF_MINB: combine order and CTA shape of the
-// breadth-first form; GAR_TUNE_SP_PAIR (0: no paired adds, 1: pairs of tracked operand
+// breadth-first form; GAR_TUNE_ST_GROUPS / _RING: thread groups and tiles of the streaming form;
+// GAR_TUNE_SP_PAIR (0: no paired adds, 1: pairs of tracked operand
 // pairs, 2: any adjacent placements) / _SP_WARPS / _SP_MINB: the same for the two-lane
 // form.
 int tune_int(const char *name, int dflt) {
@@ -981,6 +982,454 @@ CodegenResult generate_fused_split_source(const gar_plan &pl) {
   return cg;
 }
 
+
+// ---------------------------------------------------------------------------
+// Streaming fused kernel, for cyclic programs with several result copies that keep many
+// values alive.
+//
+// The schedule's shifts all point one way: the vector received at placement p comes from
+// placement p + d.  Unrolled along the circle (a value at placement p may be needed both
+// at position p and at position p + P), a value at position t depends only on
+// contributions at positions t and beyond, up to a fixed distance.  So the program can be
+// evaluated as a stream over positions: contributions enter in ascending order, every
+// combine runs as soon as its last contribution has entered, and each level of the
+// schedule only keeps a sliding window of its shift (P = 127, S = 7: 32 + 16 + 8 + 4 + 2 +
+// 1 = 63 values instead of 254 step by step).  The values of the first positions are
+// needed again at the end of the circle and are computed a second time there (1638
+// combines instead of 1524; none for S = 8).  A result's own (q*) chain is evaluated when
+// its last operand exists, right before its stores: its operands are alive until then
+// anyway.  The small windows leave room for 4 bytes of element positions per thread: two
+// bf16 positions share every load, store and address, and every combine of a float sum is
+// one paired fp32 add.
+//
+// A contribution is used at several distant positions, so all P of them go to shared
+// memory, a 512-byte row per contribution and tile (128 threads), by 16-byte asynchronous
+// copies past L1: no registers, and a warp copies a whole row at a time.  (4-byte copies
+// through L1 needed an L1 line each while in flight, of the 28 KB that the tiles leave:
+// P = 127 x 8 MiB bf16 S = 11, which has next to no arithmetic, 405 us; bulk copies, which
+// take uniform operands and so a loop over the lanes, S = 7 403 us instead of 384.)  A
+// persistent CTA per SM runs several 128-thread groups over a ring of tiles; a tile's rows
+// arrive in four parts, and the stream starts when the first parts are there.  The in-place
+// Allreduce's stores cannot reach contributions that are still needed: those are in the
+// tile.
+//
+// 16-byte units that span two blocks of a rotated program, and the last incomplete unit of
+// a vector, are evaluated from a table of the program, by one CTA each, before its tiles.
+//
+// P = 127 x 8 MiB bf16: S = 7 0.549 -> 0.375 ms (0.57 -> 0.84 of measured HBM; 5692 -> 3750
+// warp instructions per 64 positions), S = 8 0.469 -> 0.357.  What
+// is left at S = 7 is issue (51 % of the slots at 12 warps per SM), at S = 8 and beyond the
+// 4-byte stores and the tiles' start and end.
+// ---------------------------------------------------------------------------
+
+namespace {
+
+const char *kStreamHelpers = R"CUDA(
+#define GAR_ROW (4 * GAR_COLS)                 // bytes of a contribution's row of a tile
+#define GAR_UNIT (16 / (int)sizeof(gar_io))    // elements per 16 bytes
+#define GAR_TILE (GAR_ROW / (int)sizeof(gar_io))
+#if GAR_DTYPE == 1
+struct gar_v { float x, y; };                  // two element positions
+#else
+struct gar_v { gar_acc x; };
+#endif
+static __device__ __forceinline__ gar_u32 gar_leaf(gar_u32 at) {
+  gar_u32 r;
+  // volatile: the compiler neither keeps a value from an earlier use in a register nor
+  // gathers the reads far ahead of their uses
+  asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(r) : "r"(at));
+  return r;
+}
+static __device__ __forceinline__ gar_v gar_open(gar_u32 r) {
+  gar_v v;
+#if GAR_DTYPE == 1
+  v.x = gar_bf16_lo(r);
+  v.y = gar_bf16_hi(r);
+#elif GAR_DTYPE == 2
+  v.x = (int)r;
+#else
+  v.x = __uint_as_float(r);
+#endif
+  return v;
+}
+static __device__ __forceinline__ gar_v gar_comb2(gar_v a, gar_v b) {
+  gar_v r;
+#if GAR_DTYPE == 1 && GAR_OP == 0
+  const float2 s = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+  r.x = s.x;
+  r.y = s.y;
+#else
+  r.x = gar_op(a.x, b.x);
+#if GAR_DTYPE == 1
+  r.y = gar_op(a.y, b.y);
+#endif
+#endif
+  return r;
+}
+// a (+) contribution: a bf16 contribution enters a sum through the mixed-precision add
+// (the widening is exact, one rounding), so it is not unpacked
+static __device__ __forceinline__ gar_v gar_combl(gar_v a, gar_u32 l) {
+#if GAR_DTYPE == 1 && GAR_OP == 0
+  gar_v r;
+  gar_u16 lo, hi;
+  asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(l));
+  asm("add.rn.f32.bf16 %0, %1, %2;" : "=f"(r.x) : "h"(lo), "f"(a.x));
+  asm("add.rn.f32.bf16 %0, %1, %2;" : "=f"(r.y) : "h"(hi), "f"(a.y));
+  return r;
+#else
+  return gar_comb2(a, gar_open(l));
+#endif
+}
+// result pointer, from the table in shared memory: volatile for the same reason (as kernel
+// parameters the compiler read dozens of them ahead and spilled)
+static __device__ __forceinline__ gar_io *gar_row(gar_u32 at) {
+  gar_u64 r;
+  asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(r) : "r"(at));
+  return (gar_io *)r;
+}
+static __device__ __forceinline__ void gar_put(gar_io *p, gar_v v) {
+#if GAR_DTYPE == 1
+  gar_acc w[2] = {v.x, v.y};
+  gar_store<2>(p, w);
+#else
+  gar_acc w[1] = {v.x};
+  gar_store<1>(p, w);
+#endif
+}
+// 16 bytes to shared memory, past L1
+static __device__ __forceinline__ void gar_copy(gar_u32 dst, const gar_io *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src) : "memory");
+}
+// 1 once a wait gave up
+extern "C" { __device__ gar_u32 gar_stuck = 0; }
+// Waits until a tile's slot has been handed on `turn` times and its copies of this turn
+// have arrived.  The count comes first: a parity alone would take the phase before last
+// for the last one.  Gives up after 10 s, which no copy in flight takes.
+static __device__ __forceinline__ bool gar_wait(volatile int *handed, gar_u32 bar, int turn) {
+  gar_u64 begin = 0;
+  for (;;) {
+    gar_u32 done = 0;
+    if (*handed >= turn)
+      asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                   : "=r"(done) : "r"(bar), "r"(turn & 1) : "memory");
+    if (done) return true;
+    gar_u64 now;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+    if (begin == 0) begin = now;
+    if (now - begin > 10000000000ULL) return false;
+  }
+}
+)CUDA";
+
+// One value of the program at one position of the unrolled circle.
+struct StreamItem {
+  int value, pos;      // value id (< P: contribution) and unrolled position
+  int when;            // last contribution position it waits for
+  int a = -1, b = -1;  // operand items
+};
+
+struct StreamOrder {
+  std::vector<StreamItem> items;   // operands before their users
+  std::vector<int> emit;           // combine items in emission order
+  std::vector<int> result;         // item of result copy s
+  int peak = 0;                    // combine values alive at once
+};
+
+StreamOrder stream_order(const FusedProgram &fp) {
+  const int P = fp.P;
+  StreamOrder so;
+  std::map<std::pair<int, int>, int> id;
+  auto place = [&](int v) { return v < P ? v : (int)fp.place[v - P]; };
+  std::function<int(int, int)> need = [&](int v, int pos) -> int {
+    auto it = id.find({v, pos});
+    if (it != id.end()) return it->second;
+    StreamItem t;
+    t.value = v;
+    t.pos = pos;
+    t.when = pos;
+    if (v >= P) {
+      const int a = fp.a[v - P], b = fp.b[v - P];
+      t.a = need(a, pos + (place(a) - place(v) + P) % P);
+      t.b = need(b, pos + (place(b) - place(v) + P) % P);
+      t.when = std::max(so.items[t.a].when, so.items[t.b].when);
+    }
+    so.items.push_back(t);
+    return id[{v, pos}] = (int)so.items.size() - 1;
+  };
+  for (int s = 0; s < fp.K; ++s) so.result.push_back(need(fp.out[s], s));
+  const int ni = (int)so.items.size();
+  // items used only along a result's own chain wait for that result
+  std::vector<int> uses(ni, 0);
+  for (const StreamItem &t : so.items)
+    if (t.a >= 0) {
+      ++uses[t.a];
+      ++uses[t.b];
+    }
+  std::vector<int> when(ni), owner(ni, -1);
+  for (int k = 0; k < ni; ++k) when[k] = so.items[k].when;
+  for (int s = 0; s < fp.K; ++s) {
+    int k = so.result[s];
+    const int t_end = so.items[k].when;
+    bool first = true;
+    while (so.items[k].a >= 0 && (first ? uses[k] == 0 : uses[k] == 1) && owner[k] < 0) {
+      owner[k] = s;
+      when[k] = t_end;
+      first = false;
+      k = so.items[k].a;
+    }
+  }
+  for (int k = 0; k < ni; ++k)
+    if (so.items[k].a >= 0) so.emit.push_back(k);
+  std::stable_sort(so.emit.begin(), so.emit.end(), [&](int x, int y) {
+    if (when[x] != when[y]) return when[x] < when[y];
+    if ((owner[x] >= 0) != (owner[y] >= 0)) return owner[x] < 0;
+    return owner[x] < owner[y];
+  });
+  std::vector<int> last(ni, -1);
+  for (int t = 0; t < (int)so.emit.size(); ++t) {
+    const StreamItem &it = so.items[so.emit[t]];
+    last[it.a] = last[it.b] = t;
+  }
+  int live = 0;
+  std::vector<int> dies(so.emit.size() + 1, 0);
+  for (int t = 0; t < (int)so.emit.size(); ++t) {
+    const int k = so.emit[t];
+    ++live;
+    so.peak = std::max(so.peak, live);
+    ++dies[last[k] >= 0 ? last[k] : t];
+    live -= dies[t];
+  }
+  return so;
+}
+
+}  // namespace
+
+bool stream_form_applies(const gar_plan &pl) {
+  const FusedProgram &fp = pl.prog;
+  return pl.K > 1 && pl.group != GAR_GROUP_XOR && pl.P <= 200 && fp.place.size() == fp.a.size() &&
+         pl.n / (uint64_t)pl.P >= 512;  // a tile holds at most one block boundary
+}
+
+CodegenResult generate_fused_stream_source(const gar_plan &pl, int max_groups) {
+  const FusedProgram &fp = pl.prog;
+  const int P = pl.P;
+  const int nc = (int)fp.a.size();
+  const bool rotate = pl.K != P;
+  const StreamOrder so = stream_order(fp);
+  constexpr int cols = 128;  // threads per group, and 4-byte columns per tile
+  const int tile_bytes = 4 * cols * P;
+  const int most = (224 * 1024 - 16 * P) / tile_bytes;   // tiles that fit an SM's shared memory
+  // As many groups as fit the registers (a thread needs its windows and about 34 more for
+  // addresses and reads in flight) and the tiles: P = 127 S = 7 495 us with 2 groups of 242
+  // registers and a tile to spare, 375 with 3 of 164 and none.
+  const int regs = so.peak * (4 / elem_size(pl.dtype)) + 34;
+  const int fit = max_groups > 0 ? max_groups : regs <= 128 ? 4 : regs <= 168 ? 3 : 2;
+  const int groups = std::max(1, std::min(15, tune_int("GAR_TUNE_ST_GROUPS", std::min(most, fit))));
+  const int ring = std::max(1, std::min(most, tune_int("GAR_TUNE_ST_RING", std::max(groups + 1, 128 * 1024 / tile_bytes))));
+  CodegenResult cg;
+  cg.width = 4 / elem_size(pl.dtype);
+  cg.table_copies = rotate ? 2 : 1;
+  cg.threads = cols * groups;
+  cg.form = GAR_FORM_STREAM;
+  cg.tile = 4 * cols / elem_size(pl.dtype);
+  cg.smem = std::max(ring * tile_bytes, 32 * (P + nc));
+  cg.kernel_name = fmt("gar_fusedst_P%d_S%d_K%d_", P, pl.S, pl.K) + dtype_tag(pl.dtype) + "_" + op_tag(pl.op);
+
+  std::string s;
+  s += fmt("#define GAR_DTYPE %d\n#define GAR_OP %d\n#define GAR_FADD2 0\n", pl.dtype, pl.op);
+  s += fmt("#define GAR_COLS %d\n", cols);
+  s += "#define GAR_LDH \"" + tune_str("GAR_TUNE_LDH", ".cs") + "\"\n";
+  s += "#define GAR_STH \"" + tune_str("GAR_TUNE_STH", ".cs") + "\"\n";
+  s += kSkeleton;
+  s += kStreamHelpers;
+  // a tile's rows arrive in up to four parts of part_rows rows, each with a barrier
+  const int part_rows = ((P + 3) / 4 + 3) / 4 * 4;
+  const int parts = (P + part_rows - 1) / part_rows;
+  s += fmt("#define GAR_P %d\n#define GAR_NC %d\n#define GAR_GROUPS %d\n#define GAR_RING %d\n", P, nc, groups, ring);
+  s += fmt("#define GAR_PARTS %d\n#define GAR_PART_ROWS %d\n", parts, part_rows);
+  s += fmt("struct gar_args { const gar_io *in[%d]; gar_io *out[%d]; gar_u64 e_lo, e_hi; };\n",
+           cg.table_copies * P, cg.table_copies * P);
+  if (rotate) s += emit_block_of("gar_block_of", P, pl.n);
+  const uint64_t q = pl.n / (uint64_t)P, rem = pl.n % (uint64_t)P;
+  // first element of block b
+  s += fmt("static __device__ __forceinline__ gar_u64 gar_start(int b) { return (gar_u64)b * %lluULL + (b < %llu ? b : %lluULL); }\n",
+           (unsigned long long)q, (unsigned long long)rem, (unsigned long long)rem);
+
+  // the stream: contribution j of this thread's positions is at sl + j * GAR_ROW, the
+  // pointer of rank t_p(b) at rows + 8 p
+  std::string f = "static __device__ __forceinline__ bool gar_eval_st(gar_u32 rows, gar_u32 sl, gar_u64 e, volatile int *handed, gar_u32 bar, int turn) {\n";
+  std::vector<char> here(parts, 0);
+  auto leaf = [&](int k) { return fmt("gar_leaf(sl + %d * GAR_ROW)", so.items[k].value); };
+  std::vector<std::vector<int>> places(fp.K);
+  for (int p = 0; p < P; ++p) places[fp.origin[p]].push_back(p);
+  std::map<int, int> result_of;
+  for (int c = 0; c < fp.K; ++c) result_of[so.result[c]] = c;
+  for (int k : so.emit) {
+    const StreamItem &it = so.items[k];
+    const bool la = so.items[it.a].value < P, lb = so.items[it.b].value < P;
+    for (int o : {it.a, it.b}) {
+      const int v = so.items[o].value;
+      if (v >= P || here[v / part_rows]) continue;
+      here[v / part_rows] = 1;
+      f += fmt("  if (!gar_wait(handed, bar + %d, turn)) return false;\n", 8 * (v / part_rows));
+    }
+    std::string x;
+    if (la && lb)
+      x = "gar_combl(gar_open(" + leaf(it.a) + "), " + leaf(it.b) + ")";
+    else if (la)
+      x = fmt("gar_combl(v%d, ", it.b) + leaf(it.a) + ")";
+    else if (lb)
+      x = fmt("gar_combl(v%d, ", it.a) + leaf(it.b) + ")";
+    else
+      x = fmt("gar_comb2(v%d, v%d)", it.a, it.b);
+    f += fmt("  const gar_v v%d = ", k) + x + ";\n";
+    auto r = result_of.find(k);
+    if (r != result_of.end())
+      for (int p : places[r->second]) f += fmt("  gar_put(gar_row(rows + %d) + e, v%d);\n", 8 * p, k);
+  }
+  f += "  return true;\n}\n";
+  s += f;
+
+  // up to GAR_UNIT positions [e, e + count) from the program's table, by the whole CTA:
+  // values in shared memory, the combines of one level at a time
+  std::vector<int> level(P + nc, 0), by_level(nc);
+  int levels = 0;
+  for (int k = 0; k < nc; ++k) {
+    level[P + k] = 1 + std::max(level[fp.a[k]], level[fp.b[k]]);
+    levels = std::max(levels, level[P + k]);
+    by_level[k] = k;
+  }
+  std::stable_sort(by_level.begin(), by_level.end(), [&](int x, int y) { return level[P + x] < level[P + y]; });
+  s += fmt("static __device__ const gar_u16 gar_ops[%d] = {", 3 * nc);
+  for (int k : by_level) s += fmt("%d,%d,%d,", P + k, fp.a[k], fp.b[k]);
+  s += fmt("};\nstatic __device__ const gar_u16 gar_ends[%d] = {", levels);
+  for (int l = 1, k = 0; l <= levels; ++l) {
+    while (k < nc && level[P + by_level[k]] == l) ++k;
+    s += fmt("%d,", k);
+  }
+  s += fmt("};\nstatic __device__ const gar_u16 gar_outs[%d] = {", P);
+  for (int p = 0; p < P; ++p) s += fmt("%d,", fp.out[fp.origin[p]]);
+  s += "};\n";
+  const std::string block = rotate ? "gar_block_of(e + c)" : "0";
+  s += "static __device__ __noinline__ void gar_edge(const gar_args &a, gar_acc *v, gar_u64 e, int count) {\n"
+       "  const int c = threadIdx.x % 8, t0 = threadIdx.x / 8, step = blockDim.x / 8;\n"
+       "  const bool ok = c < count;\n"
+       "  const int b = ok ? " + block + " : 0;\n"
+       "  for (int j = t0; ok && j < GAR_P; j += step) gar_load<1>(a.in[b + j] + e + c, v + 8 * j + c);\n"
+       "  __syncthreads();\n"
+       "  int k = 0;\n";
+  s += fmt("  for (int l = 0; l < %d; ++l) {\n", levels);
+  s += "    const int end = gar_ends[l];\n"
+       "    for (int t = k + t0; ok && t < end; t += step)\n"
+       "      v[8 * gar_ops[3 * t] + c] = gar_op(v[8 * gar_ops[3 * t + 1] + c], v[8 * gar_ops[3 * t + 2] + c]);\n"
+       "    k = end;\n"
+       "    __syncthreads();\n"
+       "  }\n"
+       "  for (int p = t0; ok && p < GAR_P; p += step) gar_store<1>(a.out[b + p] + e + c, v + 8 * gar_outs[p] + c);\n"
+       "  __syncthreads();\n"
+       "}\n";
+
+  // block of the positions at e, or -1 where a block boundary cuts their unit
+  if (rotate)
+    s += "static __device__ __forceinline__ int gar_whole(gar_u64 e) {\n"
+         "  const gar_u64 unit = e / GAR_UNIT * GAR_UNIT;\n"
+         "  const int b = gar_block_of(unit);\n"
+         "  return unit + GAR_UNIT <= gar_start(b + 1) ? b : -1;\n"
+         "}\n";
+  else
+    s += "static __device__ __forceinline__ int gar_whole(gar_u64) { return 0; }\n";
+  // copies of tile `tile` to the ring slot at sm, by one group: a row is GAR_COLS / 4 units
+  // of 16 bytes, one per thread, and the group takes 4 rows at a time; a part's barrier
+  // counts every thread's copies as one arrival.  A unit that a block boundary cuts is left
+  // out.
+  s += "static __device__ __forceinline__ void gar_issue(const gar_args &a, gar_u32 sm, gar_u32 bar, gar_u64 tile, gar_u64 hi) {\n"
+       "  const int lane = threadIdx.x % GAR_COLS, unit = lane % (GAR_COLS / 4), row = lane / (GAR_COLS / 4);\n"
+       "  const gar_u64 e = a.e_lo + tile * GAR_TILE + unit * GAR_UNIT;\n"
+       "  const int b = e < hi ? gar_whole(e) : -1;\n"
+       "  const gar_u32 dst = sm + row * GAR_ROW + 16 * unit;\n"
+       "#pragma unroll 1\n"
+       "  for (int p = 0; p < GAR_PARTS; ++p) {\n"
+       "    if (b >= 0) {\n"
+       "#pragma unroll 8\n"
+       "      for (int i = 0; i < GAR_PART_ROWS; i += 4) {\n"
+       "        const int j = p * GAR_PART_ROWS + i + row;\n"
+       "        if (j < GAR_P) gar_copy(dst + (p * GAR_PART_ROWS + i) * GAR_ROW, a.in[b + j] + e);\n"
+       "      }\n"
+       "    }\n"
+       "    asm volatile(\"cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\" :: \"r\"(bar + 8 * p) : \"memory\");\n"
+       "  }\n"
+       "}\n";
+
+  s += fmt("extern \"C\" __global__ void __launch_bounds__(%d, 1) ", cg.threads) + cg.kernel_name +
+       "(const __grid_constant__ gar_args a) {\n";
+  s += "  extern __shared__ __align__(128) unsigned char gar_sm[];\n"
+       "  __shared__ __align__(8) gar_u64 s_full[GAR_RING * GAR_PARTS];\n"
+       "  __shared__ int s_handed[GAR_RING];\n"
+       "  __shared__ gar_io *s_rows[sizeof(gar_args::out) / 8];\n"
+       "  for (int i = threadIdx.x; i < (int)(sizeof(gar_args::out) / 8); i += blockDim.x) s_rows[i] = a.out[i];\n"
+       "  const gar_u32 rows = (gar_u32)__cvta_generic_to_shared(s_rows);\n"
+       "  const gar_u32 sm = (gar_u32)__cvta_generic_to_shared(gar_sm), full = (gar_u32)__cvta_generic_to_shared(s_full);\n"
+       "  if (threadIdx.x == 0) {\n"
+       "    for (int i = 0; i < GAR_RING; ++i) s_handed[i] = 0;\n"
+       "    for (int i = 0; i < GAR_RING * GAR_PARTS; ++i) {\n"
+       "      asm volatile(\"mbarrier.init.shared::cta.b64 [%0], %1;\" :: \"r\"(full + 8 * i), \"r\"(GAR_COLS) : \"memory\");\n"
+       "    }\n"
+       "  }\n";
+  // launched with programmatic stream serialisation: nothing is read before every
+  // earlier kernel on the stream has completed
+  s += "  asm volatile(\"griddepcontrol.wait;\" ::: \"memory\");\n"
+       "  const gar_u64 hi = a.e_hi / GAR_UNIT * GAR_UNIT;\n"
+       "  const gar_u64 tiles = hi > a.e_lo ? (hi - a.e_lo + GAR_TILE - 1) / GAR_TILE : 0;\n";
+  // the table-driven units, in the whole ring, before any copy is issued
+  s += "  gar_acc *const ev = reinterpret_cast<gar_acc *>(gar_sm);\n";
+  if (rotate) {
+    s += "  for (int k = blockIdx.x; k < GAR_P; k += gridDim.x) {\n"
+         "    if (k == 0) {\n"
+         "      if (a.e_hi > hi) gar_edge(a, ev, hi, (int)(a.e_hi - hi));\n"
+         "    } else {\n"
+         "      const gar_u64 cut = gar_start(k), unit = cut / GAR_UNIT * GAR_UNIT;\n"
+         "      if (cut != unit && unit >= a.e_lo && unit < hi) gar_edge(a, ev, unit, GAR_UNIT);\n"
+         "    }\n"
+         "  }\n";
+  } else {
+    s += "  if (blockIdx.x == 0 && a.e_hi > hi) gar_edge(a, ev, hi, (int)(a.e_hi - hi));\n";
+  }
+  s += "  __syncthreads();\n"
+       "  const int group = threadIdx.x / GAR_COLS, lane = threadIdx.x % GAR_COLS;\n"
+       "  for (int k = group; k < GAR_RING; k += GAR_GROUPS) {\n"
+       "    const gar_u64 tile = blockIdx.x + (gar_u64)k * gridDim.x;\n"
+       "    if (tile < tiles) gar_issue(a, sm + k * (GAR_P * GAR_ROW), full + 8 * GAR_PARTS * k, tile, hi);\n"
+       "  }\n"
+       "  int slot = group % GAR_RING, turn = group / GAR_RING;\n"
+       "  bool ok = true;\n"
+       "  for (gar_u64 tile = blockIdx.x + (gar_u64)group * gridDim.x; tile < tiles; tile += (gar_u64)GAR_GROUPS * gridDim.x) {\n"
+       "    const gar_u32 at = sm + slot * (GAR_P * GAR_ROW), bar = full + 8 * GAR_PARTS * slot;\n"
+       ;
+  s += fmt("    const gar_u64 e = a.e_lo + tile * GAR_TILE + lane * %d;\n", cg.width);
+  // a thread whose wait gave up stores nothing and issues nothing any more, but keeps to
+  // its group's barriers
+  s += "    const int b = ok && e < hi ? gar_whole(e) : -1;\n"
+       "    if (b >= 0 && !gar_eval_st(rows + 8 * b, at + 4 * lane, e, s_handed + slot, bar, turn)) {\n"
+       "      ok = false;\n"
+       "      gar_stuck = 1;\n"
+       "    }\n"
+       // every thread of the group has read its column: the slot takes the tile RING turns on
+       "    __syncwarp();\n"
+       "    asm volatile(\"bar.sync %0, %1;\" :: \"r\"(1 + group), \"n\"(GAR_COLS) : \"memory\");\n"
+       "    if (lane == 0) *(volatile int *)(s_handed + slot) = turn + 1;\n"
+       "    const gar_u64 next = tile + (gar_u64)GAR_RING * gridDim.x;\n"
+       "    if (ok && next < tiles) gar_issue(a, at, bar, next, hi);\n"
+       "    slot += GAR_GROUPS;\n"
+       "    while (slot >= GAR_RING) {\n"
+       "      slot -= GAR_RING;\n"
+       "      ++turn;\n"
+       "    }\n"
+       "  }\n"
+       "  asm volatile(\"cp.async.wait_all;\" ::: \"memory\");\n"
+       "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n}\n";
+  cg.source = s;
+  return cg;
+}
 
 CodegenResult generate_batched_source(const std::vector<const gar_plan *> &plans) {
   const gar_plan &p0 = *plans[0];

@@ -106,7 +106,10 @@ struct gar_plan {
   gar_stream_t last_stream = nullptr;
   bool ran_step_faithful = false;
   gar::JitKernel *fused = nullptr;   // owned by the JIT cache
+  gar_stream_t fused_stream = nullptr;  // of the last launch of a kernel with bounded waits
+  bool ran_waiting = false;
   int fused_width = 0;
+  bool fused_ready = false;          // the kernel to run has been chosen and loaded
   // persistent step-faithful mode: launch table, barrier state, barrier parameters
   void *d_launches = nullptr;
   void *d_barrier = nullptr;
@@ -137,7 +140,9 @@ struct CodegenResult {
   int width = 1;
   int table_copies = 1;  // fused kernels: copies of the in[] / out[] pointer tables (1 or 2)
   int threads = 256;     // threads per CTA
-  int form = 0;          // fused kernels: 0 single-thread program, 1 breadth-first
+  int form = 0;          // fused kernels: GAR_FORM_*
+  int smem = 0;          // dynamic shared memory per CTA
+  int tile = 0;          // element positions per tile of a persistent kernel (0: one vector per thread)
 };
 // threads / minb > 0 override the CTA size and the minimum resident CTAs per SM
 CodegenResult generate_fused_source(const gar_plan &pl, int threads = 0, int minb = 0, int fadd2 = -1);
@@ -147,6 +152,9 @@ CodegenResult generate_fused_bf_source(const gar_plan &pl);
 // two lanes per element position for rotation-invariant (latency-optimal cyclic) programs
 bool split_form_applies(const gar_plan &pl);
 CodegenResult generate_fused_split_source(const gar_plan &pl);
+// as a stream over placements (cyclic programs with several result copies)
+bool stream_form_applies(const gar_plan &pl);
+CodegenResult generate_fused_stream_source(const gar_plan &pl, int max_groups = 0);
 int fused_peak_live(const gar_plan &pl);
 CodegenResult generate_batched_source(const std::vector<const gar_plan *> &plans);
 
@@ -161,7 +169,10 @@ struct JitKernel {
   int table_copies = 1;
   int threads = 256;
   int form = 0;
+  int smem = 0;
+  int tile = 0;
   int blocks_per_sm = 0;
+  void *stuck = nullptr;     // streaming form: device flag, 1 once a wait gave up
   int regs = 0, local_bytes = 0;
   bool loaded = false;
 };
@@ -169,6 +180,7 @@ int jit_compile(const CodegenResult &cg, JitKernel **out);
 int jit_load(JitKernel *k);
 
 // step_kernels.cu
+int num_sms();
 int launch_step(const gar_plan &pl, const Launch &ln, int launch_index, void *const *rank,
                 gar_stream_t stream);
 int launch_persistent(const gar_plan &pl, void *const *rank, gar_stream_t stream);

@@ -62,6 +62,8 @@ int jit_compile(const CodegenResult &cg, JitKernel **out) {
   k->table_copies = cg.table_copies;
   k->threads = cg.threads;
   k->form = cg.form;
+  k->smem = cg.smem;
+  k->tile = cg.tile;
   *out = k.get();
   g_cache.emplace(cg.source, std::move(k));
   return GAR_OK;
@@ -80,8 +82,15 @@ int jit_load(JitKernel *k) {
     cudaLibraryUnload(lib);
     return cuda_fail(e, "cudaLibraryGetKernel");
   }
+  if (k->smem > 32 * 1024) {  // (and the kernel's static shared memory)
+    e = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, k->smem);
+    if (e != cudaSuccess) {
+      cudaLibraryUnload(lib);
+      return cuda_fail(e, "cudaFuncSetAttribute(dynamic shared memory)");
+    }
+  }
   int nb = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)kern, k->threads, 0);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)kern, k->threads, k->smem);
   if (e != cudaSuccess || nb <= 0) {
     cudaGetLastError();
     nb = 1;
@@ -92,6 +101,14 @@ int jit_load(JitKernel *k) {
     k->local_bytes = (int)fa.localSizeBytes;
   } else {
     cudaGetLastError();
+  }
+  if (k->form == GAR_FORM_STREAM) {
+    size_t bytes = 0;
+    e = cudaLibraryGetGlobal(&k->stuck, &bytes, lib, "gar_stuck");
+    if (e != cudaSuccess) {
+      cudaLibraryUnload(lib);
+      return cuda_fail(e, "cudaLibraryGetGlobal");
+    }
   }
   k->library = lib;
   k->kernel = (void *)kern;

@@ -24,6 +24,25 @@
 #include "gar_internal.hpp"
 
 namespace gar {
+
+// SM count of the current device (cached per device ordinal).
+int num_sms() {
+  static int cache[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) {
+    cudaGetLastError();
+    dev = 0;
+  }
+  if (dev < 64 && cache[dev] > 0) return cache[dev];
+  int v = 0;
+  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
+    cudaGetLastError();
+    v = 1;
+  }
+  if (dev < 64) cache[dev] = v;
+  return v;
+}
+
 namespace {
 
 // Launch shape, from sweeps on GB300: CTAs own 16384-element chunks of large vectors
@@ -668,23 +687,6 @@ __global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, FLAT ? 4 : 
   }
 }
 
-// SM count of the current device (cached per device ordinal).
-int num_sms() {
-  static int cache[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) {
-    cudaGetLastError();
-    dev = 0;
-  }
-  if (dev < 64 && cache[dev] > 0) return cache[dev];
-  int v = 0;
-  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
-    cudaGetLastError();
-    v = 1;
-  }
-  if (dev < 64) cache[dev] = v;
-  return v;
-}
 
 // Elements per CTA of a chunked launch.  Distribution steps copy 2-byte elements with as
 // many bytes per CTA as fp32 chunks hold; launches of few CTAs take smaller chunks; a last
