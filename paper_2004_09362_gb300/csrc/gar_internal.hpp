@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <cstddef>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/gar.h"
@@ -109,6 +110,8 @@ struct gar_plan {
   gar_stream_t fused_stream = nullptr;  // of the last launch of a kernel with bounded waits
   bool ran_waiting = false;
   int fused_width = 0;
+  // kernels of the batches whose first plan this is, by (n, dtype, op) and the plans' programs
+  std::vector<std::pair<std::vector<uint64_t>, gar::JitKernel *>> batched;
   bool fused_ready = false;          // the kernel to run has been chosen and loaded
   // persistent step-faithful mode: launch table, barrier state, barrier parameters
   void *d_launches = nullptr;

@@ -258,11 +258,29 @@ def gar_plan_prepare(plan: Plan, mode="fused") -> None:
     _check(_lib.gar_plan_prepare(plan.handle, _code(mode, MODES, "mode")), "gar_plan_prepare")
 
 
+_raw_stream = None
+
+
+def _current_stream() -> int:
+    """PyTorch's current stream of the current device, as an integer.  Building the Stream
+    object that torch.cuda.current_stream() returns took 3.3 us of a 6.7 us call; the raw
+    handle takes a few tenths."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+        else:
+            device = torch.cuda.current_device
+            _raw_stream = lambda: raw(device())
+    return _raw_stream()
+
+
 def _stream_handle(stream) -> ctypes.c_void_p:
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    if hasattr(stream, "cuda_stream"):
+        stream = _current_stream()
+    elif hasattr(stream, "cuda_stream"):
         stream = stream.cuda_stream
     return ctypes.c_void_p(int(stream) or None)
 
