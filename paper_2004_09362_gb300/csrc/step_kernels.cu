@@ -62,14 +62,14 @@ constexpr uint64_t kFlatBelow = 4 * kThreads * kUnroll;  // blocks shorter than 
 // threads, 36.8 at 256, 35.7 at 1024, 41.8 at 2048 (43.5 with up to 8 ops per thread).
 constexpr int kFlatGroup = 4;
 constexpr uint64_t kFlatThreads = 512;
-// Persistent steps: smallest piece of a block, and what starting a piece costs, in
-// elements.  The chunked steps run in CTAs of 512 threads, 2 per SM: the grid barrier has
-// 304 arrivals and pollers (P = 24 x 4 MiB int32, S = 10: 95.6 us; 98.2 in 1024-thread
-// CTAs, 98.9 in 256-thread ones, 4 per SM).
-constexpr int kPersistThreads = 512;
+// Persistent steps: smallest piece of a block.  The chunked steps run in CTAs of 256
+// threads, 2 per SM without spills: P = 24 x 4 MiB int32 max S = 10 87.6 us (92.8 with 3 per
+// SM, 98.9 with 4, 95.6 in 512-thread CTAs that spilled; 119 cut as the largest step), P = 24
+// x 240 KB fp32 S = 10 33.0 (37.1, 48.7, 45.3; 40.5), P = 18 x 460 KB int32 S = 6 38.8
+// (33.4, 41.1, 44.1; 40.0).
+constexpr int kPersistThreads = 256;
 constexpr int kPersistPerSM = 2;
-constexpr uint64_t kMinPiece = 1024;
-constexpr uint64_t kPieceCost = 512;
+constexpr uint64_t kMinPiece = 2048;
 
 // Counter upkeep of one launch, by its first CTA (after wait_prior_grid): zeroes the
 // counters of the communication step that follows, and moves the first step's counts,
@@ -595,11 +595,10 @@ __host__ __device__ __forceinline__ CounterUpkeep upkeep_of(unsigned long long *
 }
 
 // One step as a CTA of the persistent kernel sees it, fetched before the barrier that opens
-// it (the op table never changes), so that behind the barrier only the data is waited for.
+// it (the tables never change).
 struct PersistStep {
   LaunchDesc d;
   uint32_t items, nchunks, chunk;  // nchunks pieces of `chunk` elements per block
-  StepOp op;                       // of the CTA's first item
 };
 
 template <int MAXP, bool FLAT>
@@ -608,15 +607,18 @@ __device__ __forceinline__ PersistStep fetch_step(const PersistArgs<MAXP> &p, in
   s.d = p.launches[l];
   if (FLAT) return s;
   // A step's blocks (P * nops of maxblk elements) are cut into equal pieces, as many as
-  // give every CTA one piece, or, where there are more blocks than CTAs, as many as waste
-  // least of the last round: every CTA reaches the barrier at about the same time.
+  // give every CTA one piece, or, where there are more blocks than CTAs, as many as take
+  // the fewest batches of loads (and starts of pieces) in all rounds: every CTA reaches the
+  // barrier at about the same time.
   const uint64_t maxblk = p.s.q + (p.s.rem ? 1 : 0);
   const uint32_t blocks = (uint32_t)p.s.P * (uint32_t)max(1, s.d.nops);
+  constexpr uint32_t batch = 4 * kUnroll * kPersistThreads;
   uint32_t k = gridDim.x / blocks;
   if (k == 0) {
     uint64_t best = ~0ull;
     for (uint32_t c = 1; c <= 4; ++c) {
-      const uint64_t cost = (uint64_t)((blocks * c + gridDim.x - 1) / gridDim.x) * (maxblk / c + kPieceCost);
+      const uint64_t piece = (maxblk + c - 1) / c;
+      const uint64_t cost = (uint64_t)((blocks * c + gridDim.x - 1) / gridDim.x) * ((piece + batch - 1) / batch + 1);
       if (cost < best) {
         best = cost;
         k = c;
@@ -628,7 +630,6 @@ __device__ __forceinline__ PersistStep fetch_step(const PersistArgs<MAXP> &p, in
   s.chunk = (uint32_t)chunk;
   s.nchunks = (uint32_t)((maxblk + chunk - 1) / chunk);
   s.items = s.d.nops > 0 ? s.nchunks * blocks : 0;
-  if (blockIdx.x < s.items) s.op = p.s.ops[s.d.first_op + blockIdx.x / s.nchunks / (uint32_t)p.s.P];
   return s;
 }
 
@@ -659,8 +660,7 @@ __global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, FLAT ? 4 : 
     } else {
       for (uint32_t item = blockIdx.x; item < st.items; item += gridDim.x) {
         const uint32_t blk = item / st.nchunks, op = blk / (uint32_t)p.s.P;
-        if (item != blockIdx.x) st.op = lv.ops[op];
-        range_work<T, OP, MAXP, kPersistThreads>(p.s, lv, st.op, (int)(blk - op * (uint32_t)p.s.P),
+        range_work<T, OP, MAXP, kPersistThreads>(p.s, lv, lv.ops[op], (int)(blk - op * (uint32_t)p.s.P),
                                                  (uint64_t)(item - blk * st.nchunks) * st.chunk, st.chunk);
       }
     }
