@@ -97,3 +97,29 @@ def test_stream_form_on_host_vectors(P, n, dtype, S, monkeypatch):
                                          (120, (1 << 20) + 1, "f32", 7)])
 def test_plans_that_take_the_stream_form(P, n, dtype, S):
     _check(P, n, dtype, "sum", S, samples=500)
+
+
+@pytest.mark.parametrize("P,n,dtype,op,S", [(24, 24 * 1000 + 7, "bf16", "sum", 6), (24, 24 * 1000 + 7, "f32", "sum", 6),
+                                            (24, 24 * 1000 + 7, "bf16", "max", 6), (127, 127 * 519 + 5, "bf16", "sum", 7)])
+def test_special_values(P, n, dtype, op, S, monkeypatch):
+    """Infinities, NaN, signed zeros, subnormals and overflowing sums: the bits of the
+    single-thread form (order of combines and roundings are the schedule's in both)."""
+    g = torch.Generator().manual_seed(P + n + S)
+    big = 3.0e38
+    values = torch.tensor([0.0, -0.0, 1.0, -1.0, 1e-40, -1e-40, 9e-41, big, -big, float("inf"), -float("inf"), float("nan")])
+    # the large and non-finite values are rare: most positions stay finite
+    weights = torch.tensor([8.0, 8, 8, 8, 8, 8, 8, 0.1, 0.1, 0.1, 0.1, 0.1])
+    x = values[torch.multinomial(weights, P * n, replacement=True, generator=g)].view(P, n)
+    x[:, ::3] = x[:, ::3].clamp(-2e-40, 2e-40).nan_to_num()       # subnormal sums
+    pad = -n % 8
+    got = []
+    for form in (0, 3):
+        monkeypatch.setenv("GAR_TUNE_FUSED_FORM", str(form))
+        store = torch.zeros((P, n + pad), dtype=getattr(torch, {"bf16": "bfloat16", "f32": "float32"}[dtype]), device="cuda")
+        store[:, :n] = x.cuda()
+        plan = gar.gar_plan_create(P, n, dtype, op, S)
+        gar.gar_allreduce(plan, gar.rank_pointer_array([store[r] for r in range(P)]), "fused")
+        torch.cuda.synchronize()
+        assert gar.gar_plan_get_info(plan)["fused_form"] == form
+        got.append(store.view(torch.int16 if dtype == "bf16" else torch.int32).cpu())
+    assert torch.equal(got[0], got[1])
