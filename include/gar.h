@@ -147,8 +147,11 @@ typedef struct {
  * with the contributions in shared memory; a prepared plan (gar_plan_prepare or a first
  * fused call) of a bf16 sum that would take the breadth-first form runs it from 2^19
  * elements per rank on, an fp32 sum with more than 210 values alive from 2^20 on; before
- * that its info and source are the breadth-first form's.  All forms give the same bits. */
-enum { GAR_FORM_SINGLE = 0, GAR_FORM_BREADTH = 1, GAR_FORM_SPLIT = 2, GAR_FORM_STREAM = 3 };
+ * that its info and source are the breadth-first form's.  GAR_FORM_COOP: a CTA takes a tile
+ * of a few positions and spreads the program over its threads; a prepared plan of 16 and
+ * more ranks with few element positions (some thousands; the line depends on P and S) runs
+ * it.  All forms give the same bits. */
+enum { GAR_FORM_SINGLE = 0, GAR_FORM_BREADTH = 1, GAR_FORM_SPLIT = 2, GAR_FORM_STREAM = 3, GAR_FORM_COOP = 4 };
 
 /* Creates a schedule for P virtual ranks of n elements each.
  * P: 1..GAR_MAX_P.  n: elements per rank (0 is allowed: every call is a no-op).
@@ -227,10 +230,9 @@ GAR_API int gar_plan_set_workspace(gar_plan *plan, void *dev_ptr, size_t bytes);
 
 /* The CUDA C source of the plan's generated fused kernel (host-only): of the kernel the
  * plan runs once it is prepared (gar_plan_prepare or a first fused call, which rebuild a
- * kernel of more than 128 registers in 64-thread CTAs, and choose the streaming form),
- * else of its first compile.
- * Copies at most
- * *len bytes (including the terminating NUL) to buf and sets *len to the full size
+ * kernel of more than 128 registers in 64-thread CTAs, and choose the streaming or the
+ * cooperative form), else of its first compile.
+ * Copies at most *len bytes (including the terminating NUL) to buf and sets *len to the full size
  * including the NUL; pass buf == NULL to query the size. */
 GAR_API int gar_plan_fused_source(const gar_plan *plan, char *buf, size_t *len);
 

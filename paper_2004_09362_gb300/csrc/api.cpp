@@ -125,6 +125,13 @@ int check_fused_size(const gar_plan *pl) {
   return GAR_OK;
 }
 
+// Whether the cooperative form can run a plan: the values of 32 positions, the program's
+// table and the rank pointers fit a CTA's shared memory.
+bool coop_form_applies(const gar_plan &pl) {
+  const size_t values = pl.prog.a.size() + (size_t)pl.P;
+  return pl.P > 1 && values * (32 * 4 + 4) + (size_t)pl.P * 16 <= 220 * 1024;
+}
+
 // The fused kernel a plan uses.  Float sums with several result copies whose
 // single-thread program keeps more than 160 values alive per element position (P = 127
 // at S = 7 and 8: 254 and 192) are register-bound in that form and take the
@@ -135,8 +142,9 @@ int check_fused_size(const gar_plan *pl) {
 // 127 x 8 MiB bf16 S = 7: 0.78 ms against 0.60 ms breadth-first in one pass, 0.55 ms in
 // two; fp32: 0.416 against 0.409 ms in one pass).
 int fused_form(const gar_plan &pl) {
-  if (pl.K <= 1) return GAR_FORM_SINGLE;
   const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
+  if (ff && *ff && std::atoi(ff) == GAR_FORM_COOP) return coop_form_applies(pl) ? GAR_FORM_COOP : GAR_FORM_SINGLE;
+  if (pl.K <= 1) return GAR_FORM_SINGLE;
   if (ff && *ff) {
     const int f = std::atoi(ff);
     if (f == GAR_FORM_STREAM) return stream_form_applies(pl) ? GAR_FORM_STREAM : GAR_FORM_BREADTH;
@@ -152,6 +160,7 @@ CodegenResult fused_codegen(const gar_plan &pl) {
     case GAR_FORM_BREADTH: return generate_fused_bf_source(pl);
     case GAR_FORM_SPLIT: return generate_fused_split_source(pl);
     case GAR_FORM_STREAM: return generate_fused_stream_source(pl);
+    case GAR_FORM_COOP: return generate_fused_coop_source(pl);
     default: return generate_fused_source(pl);
   }
 }
@@ -204,6 +213,51 @@ bool takes_stream(const gar_plan &pl) {
   return pl.dtype == GAR_BF16 ? live > 160 : live > 210 && pl.n >= (1u << 20);
 }
 
+// Whether a prepared plan runs the cooperative form.  GB300, us per fused call in graph
+// replay, the other form -> cooperative (bf16; fp32 within a few per cent):
+//  * P below 16 gains little or loses (P = 12, S = 8 2.3 -> 1.7, S = 5 1.7 -> 1.7; P = 6
+//    1.3 -> 1.5), and so do the many levels of the Ring and of most folds (P = 48 2.5 -> 4.3).
+//  * One result copy: up to a tile of 32 positions per SM (152 SMs; P = 48, S = 12, 2500
+//    positions 2.4 -> 2.0, 10000 2.4 -> 3.3; P = 127, S = 14, 212 6.5 -> 1.9, 2500 5.4 -> 3.1,
+//    5000 4.5 -> 3.7, 10000 4.5 -> 5.6), two tiles up to P = 32 (P = 24, S = 10, 10000
+//    2.4 -> 2.0, 20000 2.6 -> 3.1).
+//  * Several copies: up to a tile per SM too (P = 24, S = 8, 5000 positions 2.5 -> 1.8;
+//    P = 127, S = 10, 100 11.7 -> 2.0, 5000 5.8 -> 4.5, 10000 4.9 -> 5.9), and 2.75e6 loads,
+//    combines and stores in all (P = 80, S = 8, 5000, 2.6e6, 5.9 -> 4.7; 10000 3.8 -> 6.6),
+//    0.7e6 below P = 48 (P = 24, S = 6, 5000, 0.6e6, 2.3 -> 2.1; P = 33, S = 7, 4864, 0.9e6,
+//    2.2 either way), 1.2e6 against the breadth-first form (P = 127, S = 8, 1000, 1.1e6,
+//    5.7 -> 3.7; 2500 5.3 -> 6.9).
+//  * Not with a copy at every placement: that program reads without rotation, and has the
+//    most combines (P = 24, S = 5, 400 1.6 -> 1.7; P = 40, S = 6, 2800 2.4 -> 2.6; P = 80,
+//    S = 7, 1000 4.2 -> 2.2, 2500 4.3 -> 7.8; P = 127, S = 7, 500 4.2 -> 3.7, but with the
+//    GPU waited for 17.3 -> 19.6).
+bool takes_coop(const gar_plan &pl) {
+  for (const char *name : {"GAR_TUNE_FUSED_FORM", "GAR_TUNE_FUSED_W", "GAR_TUNE_FUSED_THREADS", "GAR_TUNE_FUSED_MINB"})
+    if (const char *v = std::getenv(name); v && *v) return false;
+  const uint64_t wave = 32 * 152;
+  if (pl.P < 16 || pl.n > 2 * wave || !coop_form_applies(pl) || fused_levels(pl) > 10) return false;
+  if (pl.K == 1) return pl.n <= (pl.P <= 32 ? 2 * wave : wave);
+  const uint64_t work = pl.n * (2 * (uint64_t)pl.P + pl.prog.a.size());
+  const uint64_t most = fused_peak_live(pl) > 160 ? 1200000 : pl.P < 48 ? 700000 : 2750000;
+  return pl.K < pl.P && pl.n <= wave && work <= most;
+}
+
+int prepare_coop(gar_plan *pl) {
+  JitKernel *k = nullptr;
+  CodegenResult cg;
+  try {
+    cg = generate_fused_coop_source(*pl);
+  } catch (const std::exception &ex) {
+    set_error(std::string("fused code generation: ") + ex.what());
+    return GAR_EINVAL;
+  }
+  if (int rc = jit_compile(cg, &k)) return rc;
+  if (int rc = jit_load(k)) return rc;
+  pl->fused = k;
+  pl->fused_width = k->width;
+  return GAR_OK;
+}
+
 int prepare_stream(gar_plan *pl) {
   JitKernel *k = nullptr;
   for (int groups = 0;;) {
@@ -230,6 +284,10 @@ int build_fused(gar_plan *pl) {
   if (takes_stream(*pl)) {
     if ((rc = ensure_device(pl))) return rc;
     return prepare_stream(pl);
+  }
+  if (takes_coop(*pl)) {
+    if ((rc = ensure_device(pl))) return rc;
+    return prepare_coop(pl);
   }
   rc = compile_fused(pl);
   if (rc) return rc;
@@ -341,7 +399,9 @@ int host_grid(const gar_plan &pl) {
   const JitKernel *k = pl.fused;
   uint64_t per_thread = (uint64_t)pl.P * (uint64_t)k->width * (uint64_t)elem_size(pl.dtype);
   if (k->regs > 0) per_thread = std::min<uint64_t>(per_thread, 4 * (uint64_t)k->regs);
-  const uint64_t per_cta = k->tile > 0 ? (uint64_t)k->smem : per_thread * (uint64_t)k->threads;
+  const uint64_t per_cta = k->form == GAR_FORM_STREAM ? (uint64_t)k->smem
+                           : k->form == GAR_FORM_COOP ? (uint64_t)pl.P * (uint64_t)k->tile * (uint64_t)elem_size(pl.dtype)
+                                                      : per_thread * (uint64_t)k->threads;
   return (int)std::max<uint64_t>(1, (3000000 + per_cta - 1) / per_cta);
 }
 

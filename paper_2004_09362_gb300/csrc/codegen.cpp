@@ -520,6 +520,22 @@ static __device__ __forceinline__ float gar_addbf(gar_u16 h, float c) {
 
 int fused_peak_live(const gar_plan &pl) { return order_program(pl.prog).peak_live; }
 
+namespace {
+
+// level of every value: 0 for the contributions, one more than its operands for a combine
+std::vector<int> value_levels(const FusedProgram &fp) {
+  std::vector<int> level(fp.P + fp.a.size(), 0);
+  for (size_t k = 0; k < fp.a.size(); ++k) level[fp.P + k] = 1 + std::max(level[fp.a[k]], level[fp.b[k]]);
+  return level;
+}
+
+}  // namespace
+
+int fused_levels(const gar_plan &pl) {
+  const std::vector<int> level = value_levels(pl.prog);
+  return *std::max_element(level.begin(), level.end());
+}
+
 CodegenResult generate_fused_bf_source(const gar_plan &pl) {
   const FusedProgram &fp = pl.prog;
   const int P = pl.P;
@@ -1427,6 +1443,154 @@ CodegenResult generate_fused_stream_source(const gar_plan &pl, int max_groups) {
        "  }\n"
        "  asm volatile(\"cp.async.wait_all;\" ::: \"memory\");\n"
        "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n}\n";
+  cg.source = s;
+  return cg;
+}
+
+// ---------------------------------------------------------------------------
+// Cooperative fused kernel, for short vectors.
+//
+// A thread of the forms above takes an element position through the whole program: P
+// loads, the combines one after the other, P stores.  A short vector has too few positions
+// to fill the device with that, and the call takes as long as one thread does.  Here a CTA
+// takes a tile of a few positions and spreads the program over its threads: the
+// contributions go to shared memory, a few loads per thread; the combines of one level,
+// which never depend on each other, are shared out from a table of the program, with a
+// barrier after each level; every result is stored by another thread.  The table and the
+// rank pointers are copied to shared memory before the launch waits for its predecessor,
+// and the next launch may do so at once (0.2 to 1 us a call in a sequence of them).
+// Bound by latency: the launch, one trip to memory and back, a few hundred cycles per level.
+// P = 127, 425 B bf16 S = 14 6.5 -> 1.9 us in graph replay, 9 KiB S = 10 5.7 -> 3.6.
+// ---------------------------------------------------------------------------
+
+namespace {
+
+const char *kCoopHelpers = R"CUDA(
+#define GAR_ROWS (GAR_THREADS / GAR_COLS)   // program rows the CTA works on at once
+#define GAR_BATCH 4                         // rows a thread has in flight
+// The combines [k0, k1) of one level.
+static __device__ __forceinline__ void gar_level(gar_acc *v, const gar_u32 *ops, int k0, int k1, int row, int c) {
+  for (int k = k0 + row; k < k1; k += GAR_BATCH * GAR_ROWS) {
+    gar_u32 o[GAR_BATCH];
+    gar_acc r[GAR_BATCH];
+#pragma unroll
+    for (int u = 0; u < GAR_BATCH; ++u)
+      if (k + u * GAR_ROWS < k1) o[u] = ops[k + u * GAR_ROWS];
+#pragma unroll
+    for (int u = 0; u < GAR_BATCH; ++u)
+      if (k + u * GAR_ROWS < k1) r[u] = gar_op(v[(o[u] & 0xffff) * GAR_COLS + c], v[(o[u] >> 16) * GAR_COLS + c]);
+#pragma unroll
+    for (int u = 0; u < GAR_BATCH; ++u)
+      if (k + u * GAR_ROWS < k1) v[(GAR_P + k + u * GAR_ROWS) * GAR_COLS + c] = r[u];
+  }
+  __syncthreads();
+}
+)CUDA";
+
+}  // namespace
+
+CodegenResult generate_fused_coop_source(const gar_plan &pl) {
+  const FusedProgram &fp = pl.prog;
+  const int P = pl.P;
+  const int nc = (int)fp.a.size();
+  const bool rotate = pl.K != P;
+  // As many positions per tile, up to 32, as give every SM a tile (wider tiles load and
+  // store longer rows, and take the barriers of a level for more positions), and as many
+  // threads as keep about 4 rows each.  P = 127: 212 positions 1.9 us with 4 positions and
+  // 128 or 256 threads (2.0 with 2, 2.1 with 8, 3.0 to 5.3 with 16); 4608 at S = 10 3.4 with
+  // 16 and 512, 3.6 with 32 and 512 (4.0 with 8, 3.6 and 6.6 in 256 threads); P = 24, 10000
+  // at S = 10 1.9 with 32 and 256 (2.1 with 16 and 128, 2.6 with 512).
+  int cols = 4, threads = 128;
+  while (cols < 32 && pl.n > 152u * (uint64_t)cols) cols *= 2;
+  while (threads < 512 && threads < P * cols / 4) threads *= 2;
+  CodegenResult cg;
+  cg.width = 1;
+  cg.threads = threads;
+  cg.form = GAR_FORM_COOP;
+  cg.tile = cols;
+  cg.smem = P * 16 + (nc + P) * 4 + (P + nc) * cols * 4;
+  cg.kernel_name = fmt("gar_fusedco_P%d_S%d_K%d_", P, pl.S, pl.K) + dtype_tag(pl.dtype) + "_" + op_tag(pl.op);
+
+  // values renumbered in level order: contributions, then the combines of one level after
+  // the other
+  const std::vector<int> level = value_levels(fp);
+  const int levels = fused_levels(pl);
+  std::vector<int> order(nc), id(P + nc);
+  for (int k = 0; k < nc; ++k) order[k] = k;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return level[P + x] < level[P + y]; });
+  for (int j = 0; j < P; ++j) id[j] = j;
+  for (int t = 0; t < nc; ++t) id[P + order[t]] = P + t;
+
+  std::string s;
+  s += fmt("#define GAR_DTYPE %d\n#define GAR_OP %d\n#define GAR_FADD2 0\n", pl.dtype, pl.op);
+  s += "#define GAR_LDH \"" + tune_str("GAR_TUNE_LDH", ".cs") + "\"\n";
+  s += "#define GAR_STH \"" + tune_str("GAR_TUNE_STH", ".cs") + "\"\n";
+  s += kSkeleton;
+  s += fmt("#define GAR_P %d\n#define GAR_NC %d\n#define GAR_COLS %d\n#define GAR_THREADS %d\n", P, nc, cols, threads);
+  s += kCoopHelpers;
+  s += fmt("struct gar_args { const gar_io *in[%d]; gar_io *out[%d]; gar_u64 e_lo, e_hi; };\n", P, P);
+  s += emit_block_of("gar_block_of", P, pl.n);
+  // rank of contribution / placement j for an element of block b: t_j(b)
+  s += "static __device__ __forceinline__ int gar_rank(int b, int j) {\n";
+  if (!rotate) s += "  return j;\n}\n";
+  else if (pl.group == GAR_GROUP_XOR) s += "  return b ^ j;\n}\n";
+  else s += "  return b + j >= GAR_P ? b + j - GAR_P : b + j;\n}\n";
+  s += fmt("static __device__ const gar_u32 gar_ops[%d] = {", nc);
+  for (int t = 0; t < nc; ++t) s += fmt("%uu,", (unsigned)id[fp.a[order[t]]] | (unsigned)id[fp.b[order[t]]] << 16);
+  s += fmt("};\nstatic __device__ const gar_u16 gar_outs[%d] = {", P);
+  for (int p = 0; p < P; ++p) s += fmt("%d,", id[fp.out[fp.origin[p]]]);
+  s += "};\n";
+  s += "extern \"C\" __global__ void __launch_bounds__(GAR_THREADS) " + cg.kernel_name +
+       "(const __grid_constant__ gar_args a) {\n"
+       "  extern __shared__ __align__(16) unsigned char gar_sm[];\n"
+       "  const gar_io **const s_in = reinterpret_cast<const gar_io **>(gar_sm);\n"
+       "  gar_io **const s_out = reinterpret_cast<gar_io **>(gar_sm) + GAR_P;\n"
+       "  gar_u32 *const s_ops = reinterpret_cast<gar_u32 *>(s_out + GAR_P);\n"
+       "  gar_u32 *const s_src = s_ops + GAR_NC;\n"
+       "  gar_acc *const v = reinterpret_cast<gar_acc *>(s_src + GAR_P);\n"
+       "  for (int i = threadIdx.x; i < GAR_P; i += GAR_THREADS) {\n"
+       "    s_in[i] = a.in[i];\n"
+       "    s_out[i] = a.out[i];\n"
+       "    s_src[i] = gar_outs[i];\n"
+       "  }\n"
+       "  for (int i = threadIdx.x; i < GAR_NC; i += GAR_THREADS) s_ops[i] = gar_ops[i];\n"
+       "  __syncthreads();\n"
+       // launched with programmatic stream serialisation: no buffer is read before every
+       // earlier kernel on the stream has completed
+       "  asm volatile(\"griddepcontrol.wait;\" ::: \"memory\");\n"
+       // the next launch may copy its tables while this one works
+       "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n"
+       "  const int c = threadIdx.x % GAR_COLS, row = threadIdx.x / GAR_COLS;\n"
+       "  for (gar_u64 e0 = a.e_lo + (gar_u64)blockIdx.x * GAR_COLS; e0 < a.e_hi; e0 += (gar_u64)gridDim.x * GAR_COLS) {\n"
+       "    const gar_u64 e = e0 + c;\n"
+       "    const bool ok = e < a.e_hi;\n";
+  s += rotate ? "    const int b = ok ? gar_block_of(e) : 0;\n" : "    const int b = 0;\n";
+  s += "#pragma unroll 1\n"
+       "    for (int j0 = row; j0 < GAR_P; j0 += GAR_BATCH * GAR_ROWS) {\n"
+       "      gar_acc r[GAR_BATCH];\n"
+       "#pragma unroll\n"
+       "      for (int u = 0; u < GAR_BATCH; ++u) {\n"
+       "        const int j = j0 + u * GAR_ROWS;\n"
+       "        r[u] = 0;\n"
+       "        if (ok && j < GAR_P) gar_load<1>(s_in[gar_rank(b, j)] + e, r + u);\n"
+       "      }\n"
+       "#pragma unroll\n"
+       "      for (int u = 0; u < GAR_BATCH; ++u)\n"
+       "        if (j0 + u * GAR_ROWS < GAR_P) v[(j0 + u * GAR_ROWS) * GAR_COLS + c] = r[u];\n"
+       "    }\n"
+       "    __syncthreads();\n";
+  for (int l = 1, k = 0; l <= levels; ++l) {
+    int end = k;
+    while (end < nc && level[P + order[end]] == l) ++end;
+    s += fmt("    gar_level(v, s_ops, %d, %d, row, c);\n", k, end);
+    k = end;
+  }
+  s += "    if (ok) {\n"
+       "#pragma unroll 4\n"
+       "      for (int p = row; p < GAR_P; p += GAR_ROWS) gar_store<1>(s_out[gar_rank(b, p)] + e, v + s_src[p] * GAR_COLS + c);\n"
+       "    }\n"
+       "    __syncthreads();\n"
+       "  }\n}\n";
   cg.source = s;
   return cg;
 }

@@ -158,7 +158,10 @@ CodegenResult generate_fused_split_source(const gar_plan &pl);
 // as a stream over placements (cyclic programs with several result copies)
 bool stream_form_applies(const gar_plan &pl);
 CodegenResult generate_fused_stream_source(const gar_plan &pl, int max_groups = 0);
+// a tile of element positions per CTA, the program spread over its threads (short vectors)
+CodegenResult generate_fused_coop_source(const gar_plan &pl);
 int fused_peak_live(const gar_plan &pl);
+int fused_levels(const gar_plan &pl);  // of combines that depend on one another
 CodegenResult generate_batched_source(const std::vector<const gar_plan *> &plans);
 
 // jit.cpp
