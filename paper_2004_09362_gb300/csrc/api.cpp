@@ -136,8 +136,9 @@ bool coop_form_applies(const gar_plan &pl) {
 // single-thread program keeps more than 160 values alive per element position (P = 127
 // at S = 7 and 8: 254 and 192) are register-bound in that form and take the
 // breadth-first form (0.59 instead of 0.68 ms, and 0.47 instead of 0.56 ms, at P = 127 x
-// 8 MiB bf16 on GB300); every other plan takes the single-thread form.  GAR_TUNE_FUSED_FORM
-// (0, 1 or 2) forces one form, for parity tests and launch-shape sweeps; the two-lane
+// 8 MiB bf16 on GB300); every other plan takes the single-thread form.  Preparation may
+// choose the streaming or the cooperative form instead (takes_stream, takes_coop).
+// GAR_TUNE_FUSED_FORM (0 to 4) forces one form, for parity tests and launch-shape sweeps; the two-lane
 // form (2) exists for latency-optimal cyclic programs only and is never the default (P =
 // 127 x 8 MiB bf16 S = 7: 0.78 ms against 0.60 ms breadth-first in one pass, 0.55 ms in
 // two; fp32: 0.416 against 0.409 ms in one pass).

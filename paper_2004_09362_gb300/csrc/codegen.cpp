@@ -1032,10 +1032,10 @@ CodegenResult generate_fused_split_source(const gar_plan &pl) {
 // 16-byte units that span two blocks of a rotated program, and the last incomplete unit of
 // a vector, are evaluated from a table of the program, by one CTA each, before its tiles.
 //
-// P = 127 x 8 MiB bf16: S = 7 0.549 -> 0.375 ms (0.57 -> 0.84 of measured HBM; 5692 -> 3750
-// warp instructions per 64 positions), S = 8 0.469 -> 0.357.  What
-// is left at S = 7 is issue (51 % of the slots at 12 warps per SM), at S = 8 and beyond the
-// 4-byte stores and the tiles' start and end.
+// P = 127 x 8 MiB bf16: S = 7 0.549 -> 0.375 ms (0.57 -> 0.84 of measured HBM; 5692 -> 3838
+// warp instructions per 64 positions), S = 8 0.469 -> 0.357.  What is left at S = 7 is issue
+// (60 % of the slots at 12 warps per SM), at S = 8 and beyond the 4-byte stores and the
+// tiles' start and end.
 // ---------------------------------------------------------------------------
 
 namespace {

@@ -6,8 +6,8 @@
 // block index; eq. comm_op_0).  "Sending" is a coalesced 16-byte vector read of the
 // partner rank's block; the read value is combined in registers with the own block
 // (eq. distr_vectors_combination) and stored.  Every CTA owns one chunk of one block
-// of one (op, rank) pair (short blocks: one thread per (op, element) instead).  Combine
-// ops batch 2 vectors per thread; same-type copies move raw 16-byte units, 6 per
+// of one (op, rank) pair (short blocks: one thread per element and one to four ops).
+// Combine ops batch 2 vectors per thread; same-type copies move raw 16-byte units, 6 per
 // thread; a bf16 plan's first step keeps its 16-byte bf16 loads packed until the
 // combine.  The kernels add the bytes they read from partners to the step's counter
 // slots, so the bytes a step actually moved are recorded.  The launches of one Allreduce
@@ -63,10 +63,10 @@ constexpr uint64_t kFlatBelow = 4 * kThreads * kUnroll;  // blocks shorter than 
 constexpr int kFlatGroup = 4;
 constexpr uint64_t kFlatThreads = 512;
 // Persistent steps: smallest piece of a block.  The chunked steps run in CTAs of 256
-// threads, 2 per SM without spills: P = 24 x 4 MiB int32 max S = 10 87.6 us (92.8 with 3 per
-// SM, 98.9 with 4, 95.6 in 512-thread CTAs that spilled; 119 cut as the largest step), P = 24
-// x 240 KB fp32 S = 10 33.0 (37.1, 48.7, 45.3; 40.5), P = 18 x 460 KB int32 S = 6 38.8
-// (33.4, 41.1, 44.1; 40.0).
+// threads, 2 per SM without spills: P = 24 x 4 MiB int32 max S = 10 87.6 us call after call
+// (98 on vectors that L2 does not hold; 92.8 with 3 per SM, 98.9 with 4, 95.6 in 512-thread
+// CTAs that spilled; 119 cut as the largest step), P = 24 x 240 KB fp32 S = 10 33.0 (37.1,
+// 48.7, 45.3; 40.5), P = 18 x 460 KB int32 S = 6 38.8 (33.4, 41.1, 44.1; 40.0).
 constexpr int kPersistThreads = 256;
 constexpr int kPersistPerSM = 2;
 constexpr uint64_t kMinPiece = 2048;
