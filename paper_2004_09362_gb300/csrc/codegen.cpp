@@ -365,6 +365,18 @@ CodegenResult generate_fused_source(const gar_plan &pl, int threads_override, in
   // load latencies then overlap across warps instead of queueing in one (P = 127 bf16
   // with 212 positions: 92 us at W = 8, 24 us at W = 1).
   while (W > 1 && pl.n / (uint64_t)W < 16384) W /= 2;
+  // A vector that a block boundary of a rotated program cuts is evaluated one position after
+  // the other, W programs in a row: in short vectors the call waits for those threads.  So
+  // blocks of 4-byte elements that do not start at multiples of W take W = 1 up to 2^18
+  // positions (2^17 below 8 ranks).  GB300, us in graph replay, W by the line above -> W = 1:
+  // P = 24 S = 10 fp32, 33000 positions 4.9 -> 2.3, 100000 6.7 -> 3.1, 260000 8.8 -> 6.2; P = 48
+  // S = 9 64000 11.0 -> 4.4, 520000 25.6 -> 26.8; P = 12 S = 8 260000 5.3 -> 3.6; P = 5 260000
+  // 2.0 -> 2.1; from and to pinned host memory P = 24, 33000 37 -> 38, 100000 84 -> 77.  bf16
+  // gains as much on the GPU (P = 127 S = 14 33000 9.4 -> 5.3), but its 2-byte accesses cost
+  // more over NVLink-C2C (P = 8, 250000 38 -> 49), and whole vectors only gain from W (P = 64
+  // S = 12 bf16 160000 9.0 at W = 1, 5.3 at 4).
+  const bool cut = rotate && (pl.n % (uint64_t)P != 0 || pl.n / (uint64_t)P % (uint64_t)W != 0);
+  if (cut && elem_size(pl.dtype) == 4 && pl.n < (P < 8 ? 1u << 17 : 1u << 18)) W = 1;
   if (int w = tune_int("GAR_TUNE_FUSED_W", 0))
     if (w > 0 && (w & (w - 1)) == 0 && w * elem_size(pl.dtype) <= 16) W = w;
   const int minb = minb_override > 0 ? minb_override : tune_int("GAR_TUNE_FUSED_MINB", small_cta ? 16 : 0);
