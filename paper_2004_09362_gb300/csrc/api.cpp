@@ -245,6 +245,7 @@ bool takes_coop(const gar_plan &pl) {
 
 int prepare_coop(gar_plan *pl) {
   JitKernel *k = nullptr;
+  JitOnDevice on;
   CodegenResult cg;
   try {
     cg = generate_fused_coop_source(*pl);
@@ -253,14 +254,16 @@ int prepare_coop(gar_plan *pl) {
     return GAR_EINVAL;
   }
   if (int rc = jit_compile(cg, &k)) return rc;
-  if (int rc = jit_load(k)) return rc;
+  if (int rc = jit_load(k, &on)) return rc;
   pl->fused = k;
+  pl->fused_on = on;
   pl->fused_width = k->width;
   return GAR_OK;
 }
 
 int prepare_stream(gar_plan *pl) {
   JitKernel *k = nullptr;
+  JitOnDevice on;
   for (int groups = 0;;) {
     CodegenResult cg;
     try {
@@ -270,11 +273,12 @@ int prepare_stream(gar_plan *pl) {
       return GAR_EINVAL;
     }
     if (int rc = jit_compile(cg, &k)) return rc;
-    if (int rc = jit_load(k)) return rc;
+    if (int rc = jit_load(k, &on)) return rc;
     groups = k->threads / 128 - 1;
     if (k->local_bytes == 0 || groups < 2) break;  // spilled: one group less, with its registers
   }
   pl->fused = k;
+  pl->fused_on = on;
   pl->fused_width = k->width;
   return GAR_OK;
 }
@@ -294,7 +298,7 @@ int build_fused(gar_plan *pl) {
   if (rc) return rc;
   rc = ensure_device(pl);
   if (rc) return rc;
-  if ((rc = jit_load(pl->fused))) return rc;
+  if ((rc = jit_load(pl->fused, &pl->fused_on))) return rc;
   const bool shape_forced = std::getenv("GAR_TUNE_FUSED_THREADS") || std::getenv("GAR_TUNE_FUSED_MINB");
   if (pl->fused->form != 0 || pl->fused->threads != 256 || shape_forced || pl->fused->regs <= 128)
     return GAR_OK;
@@ -327,6 +331,7 @@ int build_fused(gar_plan *pl) {
     if ((rc = build(k->threads, k->threads == 64 ? 5 : 8, 1, &paired))) return rc;
     if (paired->local_bytes <= k->local_bytes) k = paired;
   }
+  if ((rc = jit_load(k, &pl->fused_on))) return rc;
   pl->fused = k;
   pl->fused_width = k->width;
   return GAR_OK;
@@ -368,7 +373,7 @@ int check_buffers(const gar_plan *pl, void *const *bufs) {
   return GAR_OK;
 }
 
-int grid_for(const JitKernel *k, uint64_t work_items) {
+int grid_for(const JitKernel *k, const JitOnDevice &on, uint64_t work_items) {
   // One work item per thread: with many more CTAs than fit at once the block scheduler
   // keeps every SM full and each thread's loads are in flight together (a persistent
   // grid-stride loop serialises a thread's iterations and ran 6% slower on GB300).
@@ -382,7 +387,7 @@ int grid_for(const JitKernel *k, uint64_t work_items) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms <= 0) sms = 1;
-    cap = (uint64_t)sms * (uint64_t)std::max(1, k->blocks_per_sm) * (uint64_t)std::atoi(wv);
+    cap = (uint64_t)sms * (uint64_t)std::max(1, on.blocks_per_sm) * (uint64_t)std::atoi(wv);
   }
   return (int)std::max<uint64_t>(1, std::min<uint64_t>(need, cap));
 }
@@ -445,15 +450,15 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
   // (two-lane form)
   const uint64_t items = pl->fused->form == GAR_FORM_SPLIT ? (e_hi - e_lo + 15) / 16 * 32
                                                            : (e_hi - e_lo) / pl->fused->width + 1;
-  int grid = grid_for(pl->fused, items);
+  int grid = grid_for(pl->fused, pl->fused_on, items);
   if (pl->fused->tile > 0) {  // persistent: as many CTAs as the device holds at once
     const uint64_t tiles = std::max<uint64_t>(1, (e_hi - e_lo + pl->fused->tile - 1) / pl->fused->tile);
-    grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms() * (uint64_t)pl->fused->blocks_per_sm);
+    grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms() * (uint64_t)pl->fused_on.blocks_per_sm);
   }
   if (host_memory) grid = std::min(grid, host_grid(*pl));
   cudaError_t e = launch_generated(pl->fused, grid, kargs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
-  if (pl->fused->stuck != nullptr) {
+  if (pl->fused_on.stuck != nullptr) {
     pl->fused_stream = stream;
     pl->ran_waiting = true;
   }
@@ -484,7 +489,6 @@ int batched_kernel(gar_plan *owner, const std::vector<const gar_plan *> &ps, Jit
   CodegenResult cg = generate_batched_source(ps);
   int rc = jit_compile(cg, out);
   if (rc) return rc;
-  if ((rc = jit_load(*out))) return rc;
   if (owner->batched.size() >= 8) owner->batched.erase(owner->batched.begin());
   owner->batched.emplace_back(std::move(key), *out);
   return GAR_OK;
@@ -926,14 +930,16 @@ int gar_allreduce_batched(gar_plan *const *plans, int nplans, const gar_batch_de
     return GAR_EALIGN;
   }
   JitKernel *k = nullptr;
+  JitOnDevice on;
   if (int rc = batched_kernel(plans[0], ps, &k)) return rc;
+  if (int rc = jit_load(k, &on)) return rc;
   struct {
     const gar_batch_desc *desc;
     unsigned long long count;
   } a = {desc, (unsigned long long)count};
   void *kargs[] = {&a};
   const uint64_t per = plans[0]->n / k->width + plans[0]->n % k->width;
-  const int grid = grid_for(k, per * (uint64_t)count);
+  const int grid = grid_for(k, on, per * (uint64_t)count);
   cudaError_t e = launch_generated(k, grid, kargs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "batched kernel launch");
   return GAR_OK;
@@ -963,15 +969,15 @@ int gar_last_step_bytes(const gar_plan *pl, uint64_t *per_step) {
 int gar_plan_status(gar_plan *pl) {
   if (int rc = check_plan(pl)) return rc;
   cudaError_t e = cudaSuccess;
-  if (pl->ran_waiting && pl->fused != nullptr && pl->fused->stuck != nullptr) {
+  if (pl->ran_waiting && pl->fused_on.stuck != nullptr) {
     e = cudaStreamSynchronize((cudaStream_t)pl->fused_stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     unsigned int stuck = 0;
-    e = cudaMemcpy(&stuck, pl->fused->stuck, sizeof stuck, cudaMemcpyDeviceToHost);
+    e = cudaMemcpy(&stuck, pl->fused_on.stuck, sizeof stuck, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(wait state)");
     pl->ran_waiting = false;
     if (stuck != 0) {
-      e = cudaMemset(pl->fused->stuck, 0, sizeof stuck);
+      e = cudaMemset(pl->fused_on.stuck, 0, sizeof stuck);
       if (e != cudaSuccess) return cuda_fail(e, "cudaMemset(wait state)");
       set_error("fused kernel: a wait for a tile gave up");
       return GAR_ETIMEOUT;

@@ -76,6 +76,12 @@ struct FusedProgram {
 
 struct JitKernel;  // jit.cpp
 
+// What a loaded kernel has of its own on each device.
+struct JitOnDevice {
+  int blocks_per_sm = 0;     // resident CTAs (0: not loaded on the device yet)
+  void *stuck = nullptr;     // streaming form: device flag, 1 once a wait gave up
+};
+
 constexpr int GAR_HOST_CHUNKS_MAX = 16;  // element chunks of the pipelined host path
 
 }  // namespace gar
@@ -107,6 +113,7 @@ struct gar_plan {
   gar_stream_t last_stream = nullptr;
   bool ran_step_faithful = false;
   gar::JitKernel *fused = nullptr;   // owned by the JIT cache
+  gar::JitOnDevice fused_on;         // the loaded kernel on the plan's device
   gar_stream_t fused_stream = nullptr;  // of the last launch of a kernel with bounded waits
   bool ran_waiting = false;
   int fused_width = 0;
@@ -177,13 +184,14 @@ struct JitKernel {
   int form = 0;
   int smem = 0;
   int tile = 0;
-  int blocks_per_sm = 0;
-  void *stuck = nullptr;     // streaming form: device flag, 1 once a wait gave up
   int regs = 0, local_bytes = 0;
   bool loaded = false;
+  std::vector<JitOnDevice> on;  // by device ordinal (jit_load's)
 };
 int jit_compile(const CodegenResult &cg, JitKernel **out);
-int jit_load(JitKernel *k);
+// Loads a kernel once per process and sets it up once per device, for the current one;
+// *here: what it has there.
+int jit_load(JitKernel *k, JitOnDevice *here = nullptr);
 
 // step_kernels.cu
 int num_sms();

@@ -69,9 +69,9 @@ int jit_compile(const CodegenResult &cg, JitKernel **out) {
   return GAR_OK;
 }
 
-int jit_load(JitKernel *k) {
-  std::lock_guard<std::mutex> lock(g_mu);
-  if (k->loaded) return GAR_OK;
+namespace {
+
+int load_library(JitKernel *k) {
   cudaLibrary_t lib = nullptr;
   cudaError_t e = cudaLibraryLoadData(&lib, k->cubin.data(), nullptr, nullptr, 0, nullptr,
                                       nullptr, 0);
@@ -82,19 +82,6 @@ int jit_load(JitKernel *k) {
     cudaLibraryUnload(lib);
     return cuda_fail(e, "cudaLibraryGetKernel");
   }
-  if (k->smem > 32 * 1024) {  // (and the kernel's static shared memory)
-    e = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, k->smem);
-    if (e != cudaSuccess) {
-      cudaLibraryUnload(lib);
-      return cuda_fail(e, "cudaFuncSetAttribute(dynamic shared memory)");
-    }
-  }
-  int nb = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)kern, k->threads, k->smem);
-  if (e != cudaSuccess || nb <= 0) {
-    cudaGetLastError();
-    nb = 1;
-  }
   cudaFuncAttributes fa{};
   if (cudaFuncGetAttributes(&fa, (const void *)kern) == cudaSuccess) {
     k->regs = fa.numRegs;
@@ -102,18 +89,44 @@ int jit_load(JitKernel *k) {
   } else {
     cudaGetLastError();
   }
-  if (k->form == GAR_FORM_STREAM) {
-    size_t bytes = 0;
-    e = cudaLibraryGetGlobal(&k->stuck, &bytes, lib, "gar_stuck");
-    if (e != cudaSuccess) {
-      cudaLibraryUnload(lib);
-      return cuda_fail(e, "cudaLibraryGetGlobal");
-    }
-  }
   k->library = lib;
   k->kernel = (void *)kern;
-  k->blocks_per_sm = nb;
   k->loaded = true;
+  return GAR_OK;
+}
+
+}  // namespace
+
+// The library and its kernel serve every device; the shared-memory limit, the resident CTAs
+// and the addresses of the kernel's variables are a device's own.
+int jit_load(JitKernel *k, JitOnDevice *here) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  if (!k->loaded)
+    if (int rc = load_library(k)) return rc;
+  if (k->on.size() <= (size_t)dev) k->on.resize((size_t)dev + 1);
+  JitOnDevice &on = k->on[(size_t)dev];
+  if (on.blocks_per_sm == 0) {
+    if (k->smem > 32 * 1024) {  // (and the kernel's static shared memory)
+      e = cudaFuncSetAttribute((const void *)k->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, k->smem);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(dynamic shared memory)");
+    }
+    if (k->form == GAR_FORM_STREAM) {
+      size_t bytes = 0;
+      e = cudaLibraryGetGlobal(&on.stuck, &bytes, (cudaLibrary_t)k->library, "gar_stuck");
+      if (e != cudaSuccess) return cuda_fail(e, "cudaLibraryGetGlobal");
+    }
+    int nb = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)k->kernel, k->threads, k->smem);
+    if (e != cudaSuccess || nb <= 0) {
+      cudaGetLastError();
+      nb = 1;
+    }
+    on.blocks_per_sm = nb;
+  }
+  if (here != nullptr) *here = on;
   return GAR_OK;
 }
 

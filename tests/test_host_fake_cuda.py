@@ -1,0 +1,50 @@
+"""Host code of the library on a fake CUDA runtime (no GPU, no CUDA libraries): what it asks
+of the runtime for several devices, plans, threads and settings.  fake_cuda_check.cpp holds
+the checks, fake_cuda.hpp the runtime."""
+
+import concurrent.futures as cf
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2004_09362_gb300 import build
+
+TESTS = os.path.dirname(os.path.abspath(__file__))
+SOURCES = ["api.cpp", "codegen.cpp", "jit.cpp", "plan.cpp"]
+
+
+def _cuda_include():
+    return os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
+
+
+def _program(out, flags):
+    cmd = ["g++", "-std=c++17", *flags, "-I", build.INCLUDE, "-I", build.CSRC, "-I", TESTS, "-isystem", _cuda_include()]
+    sources = [os.path.join(build.CSRC, s) for s in SOURCES] + [os.path.join(TESTS, "fake_cuda_check.cpp")]
+
+    def compile_one(src):
+        obj = str(out / (os.path.basename(src) + ".o"))
+        subprocess.run([*cmd, "-c", src, "-o", obj], check=True)
+        return obj
+
+    with cf.ThreadPoolExecutor(len(sources)) as ex:
+        objs = list(ex.map(compile_one, sources))
+    subprocess.run([*cmd, *objs, "-pthread", "-o", str(out / "check")], check=True)
+    return str(out / "check")
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("needs g++")
+    return _program(tmp_path_factory.mktemp("fake_cuda"), ["-O1"])
+
+
+def _run(program, check, **env):
+    r = subprocess.run([program, check], capture_output=True, text=True, timeout=120, env={**os.environ, **env})
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_equal_plans_on_two_devices(program):
+    _run(program, "two_devices")
