@@ -292,10 +292,12 @@ GAR_API int gar_allreduce_batched(gar_plan *const *plans, int nplans, const gar_
                           int count, gar_stream_t stream);
 
 /* Outcome of the plan's most recent GAR_STEP_PERSISTENT Allreduce, and of its fused ones
- * in the streaming form (no counterpart in the paper: failure reporting of the bounded
- * waits): waits for the stream it ran on, then returns GAR_OK, GAR_ETIMEOUT if a grid-barrier
- * wait, or a streaming kernel's wait for its own copies (10 s), gave up (the results are
- * then incomplete), or GAR_ECUDA.  GAR_OK if no such call ran. */
+ * in the streaming form since the last status call that reported one of them (no counterpart
+ * in the paper: failure reporting of the bounded waits): waits for the stream of the last such
+ * call, which must still exist, then returns GAR_OK, GAR_ETIMEOUT if a grid-barrier wait, or a
+ * streaming kernel's wait for its own copies (10 s), gave up (the results are then incomplete),
+ * or GAR_ECUDA.  GAR_OK if no such call ran.  Fused calls on other streams and replays of
+ * captured ones count once they have completed. */
 GAR_API int gar_plan_status(gar_plan *plan);
 
 /* Barrier parameters of GAR_STEP_PERSISTENT (no counterpart in the paper).  spin_limit: polls (each an L2 round trip,

@@ -341,6 +341,7 @@ int build_fused(gar_plan *pl) {
 int prepare_fused(gar_plan *pl) {
   if (pl->fused_ready) return ensure_device(pl);
   if (int rc = build_fused(pl)) return rc;
+  if (pl->fused_on.gave_up != nullptr) pl->wait_slot = jit_take_slot(pl->fused, pl->device, &pl->waits_seen);
   pl->fused_ready = true;
   return GAR_OK;
 }
@@ -436,15 +437,17 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
                        uint64_t e_hi, gar_stream_t stream, bool host_memory = false) {
   if (e_hi <= e_lo) return GAR_OK;
   // gar_args: the in[] table, then the out[] table, each table_copies times in a row,
-  // then e_lo, e_hi
+  // then e_lo, e_hi and, in the streaming form, the wait slot
   const size_t pb = 8 * (size_t)pl->P;
   const int copies = pl->fused->table_copies;
-  unsigned char args[4 * 8 * GAR_MAX_P + 16];
+  unsigned char args[4 * 8 * GAR_MAX_P + 24];
   unsigned char *w = args;
   for (int c = 0; c < copies; ++c, w += pb) std::memcpy(w, in, pb);
   for (int c = 0; c < copies; ++c, w += pb) std::memcpy(w, out, pb);
   std::memcpy(w, &e_lo, 8);
   std::memcpy(w + 8, &e_hi, 8);
+  const uint64_t slot = pl->wait_slot < 0 ? 0 : (uint64_t)pl->wait_slot;
+  std::memcpy(w + 16, &slot, 8);
   void *kargs[] = {args};
   // threads: one per vector of `width` positions, or two per position in groups of 16
   // (two-lane form)
@@ -458,7 +461,7 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
   if (host_memory) grid = std::min(grid, host_grid(*pl));
   cudaError_t e = launch_generated(pl->fused, grid, kargs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
-  if (pl->fused_on.stuck != nullptr) {
+  if (pl->fused_on.gave_up != nullptr) {
     pl->fused_stream = stream;
     pl->ran_waiting = true;
   }
@@ -692,6 +695,7 @@ int gar_plan_create_group(gar_plan **out, int P, uint64_t n, int dtype, int op, 
 
 void gar_plan_destroy(gar_plan *pl) {
   if (pl == nullptr) return;
+  if (pl->wait_slot >= 0) jit_drop_slot(pl->fused, pl->device, pl->wait_slot);
   if (pl->d_ops) cudaFree(pl->d_ops);
   if (pl->d_step_bytes) cudaFree(pl->d_step_bytes);
   if (pl->d_launches) cudaFree(pl->d_launches);
@@ -969,18 +973,29 @@ int gar_last_step_bytes(const gar_plan *pl, uint64_t *per_step) {
 int gar_plan_status(gar_plan *pl) {
   if (int rc = check_plan(pl)) return rc;
   cudaError_t e = cudaSuccess;
-  if (pl->ran_waiting && pl->fused_on.stuck != nullptr) {
-    e = cudaStreamSynchronize((cudaStream_t)pl->fused_stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    unsigned int stuck = 0;
-    e = cudaMemcpy(&stuck, pl->fused_on.stuck, sizeof stuck, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(wait state)");
-    pl->ran_waiting = false;
-    if (stuck != 0) {
-      e = cudaMemset(pl->fused_on.stuck, 0, sizeof stuck);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaMemset(wait state)");
-      set_error("fused kernel: a wait for a tile gave up");
-      return GAR_ETIMEOUT;
+  if (pl->ran_waiting) {
+    // launches on a stream that is being captured are recorded, not run: nothing to wait for
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing((cudaStream_t)pl->fused_stream, &capture);
+    if (e == cudaErrorStreamCaptureImplicit) {
+      cudaGetLastError();
+      capture = cudaStreamCaptureStatusActive;
+    } else if (e != cudaSuccess) {
+      return cuda_fail(e, "cudaStreamIsCapturing");
+    }
+    if (capture == cudaStreamCaptureStatusNone) {
+      e = cudaStreamSynchronize((cudaStream_t)pl->fused_stream);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+      unsigned int waits = 0;
+      e = cudaMemcpy(&waits, static_cast<unsigned int *>(pl->fused_on.gave_up) + pl->wait_slot, sizeof waits,
+                     cudaMemcpyDeviceToHost);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(wait state)");
+      if (waits != pl->waits_seen) {
+        pl->waits_seen = waits;
+        jit_seen_slot(pl->fused, pl->device, pl->wait_slot, waits);
+        set_error("fused kernel: a wait for a tile gave up");
+        return GAR_ETIMEOUT;
+      }
     }
   }
   if (!pl->ran_persistent || pl->d_barrier == nullptr) return GAR_OK;

@@ -173,6 +173,8 @@ template <> __device__ __forceinline__ void gar_store<4>(gar_io *p, const gar_ac
 // 1): whether a rotated cyclic single-thread kernel stores its pointer tables twice;
 // GAR_TUNE_BF_ORDER / _BF_WARPS / _BF_MINB: combine order and CTA shape of the
 // breadth-first form; GAR_TUNE_ST_GROUPS / _RING: thread groups and tiles of the streaming form;
+// GAR_TUNE_ST_WAIT_MS / _PHANTOM: its wait limit, and arrivals that its waits expect beyond
+// those that come (test hooks);
 // GAR_TUNE_SP_PAIR (0: no paired adds, 1: pairs of tracked operand
 // pairs, 2: any adjacent placements) / _SP_WARPS / _SP_MINB: the same for the two-lane
 // form.
@@ -1128,11 +1130,11 @@ static __device__ __forceinline__ void gar_put(gar_io *p, gar_v v) {
 static __device__ __forceinline__ void gar_copy(gar_u32 dst, const gar_io *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src) : "memory");
 }
-// 1 once a wait gave up
-extern "C" { __device__ gar_u32 gar_stuck = 0; }
+// waits that gave up, by the launch's slot
+extern "C" { __device__ gar_u32 gar_gave_up[GAR_SLOTS]; }
 // Waits until a tile's slot has been handed on `turn` times and its copies of this turn
 // have arrived.  The count comes first: a parity alone would take the phase before last
-// for the last one.  Gives up after 10 s, which no copy in flight takes.
+// for the last one.  Gives up after GAR_WAIT_NS (10 s, which no copy in flight takes).
 static __device__ __forceinline__ bool gar_wait(volatile int *handed, gar_u32 bar, int turn) {
   gar_u64 begin = 0;
   for (;;) {
@@ -1144,7 +1146,7 @@ static __device__ __forceinline__ bool gar_wait(volatile int *handed, gar_u32 ba
     gar_u64 now;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
     if (begin == 0) begin = now;
-    if (now - begin > 10000000000ULL) return false;
+    if (now - begin > GAR_WAIT_NS) return false;
   }
 }
 )CUDA";
@@ -1269,13 +1271,15 @@ CodegenResult generate_fused_stream_source(const gar_plan &pl, int max_groups) {
   s += "#define GAR_LDH \"" + tune_str("GAR_TUNE_LDH", ".cs") + "\"\n";
   s += "#define GAR_STH \"" + tune_str("GAR_TUNE_STH", ".cs") + "\"\n";
   s += kSkeleton;
+  s += fmt("#define GAR_SLOTS %d\n#define GAR_WAIT_NS %lldULL\n#define GAR_PHANTOM %d\n", GAR_WAIT_SLOTS,
+           1000000LL * tune_int("GAR_TUNE_ST_WAIT_MS", 10000), tune_int("GAR_TUNE_ST_PHANTOM", 0));
   s += kStreamHelpers;
   // a tile's rows arrive in up to four parts of part_rows rows, each with a barrier
   const int part_rows = ((P + 3) / 4 + 3) / 4 * 4;
   const int parts = (P + part_rows - 1) / part_rows;
   s += fmt("#define GAR_P %d\n#define GAR_NC %d\n#define GAR_GROUPS %d\n#define GAR_RING %d\n", P, nc, groups, ring);
   s += fmt("#define GAR_PARTS %d\n#define GAR_PART_ROWS %d\n", parts, part_rows);
-  s += fmt("struct gar_args { const gar_io *in[%d]; gar_io *out[%d]; gar_u64 e_lo, e_hi; };\n",
+  s += fmt("struct gar_args { const gar_io *in[%d]; gar_io *out[%d]; gar_u64 e_lo, e_hi, slot; };\n",
            cg.table_copies * P, cg.table_copies * P);
   if (rotate) s += emit_block_of("gar_block_of", P, pl.n);
   const uint64_t q = pl.n / (uint64_t)P, rem = pl.n % (uint64_t)P;
@@ -1400,7 +1404,7 @@ CodegenResult generate_fused_stream_source(const gar_plan &pl, int max_groups) {
        "  if (threadIdx.x == 0) {\n"
        "    for (int i = 0; i < GAR_RING; ++i) s_handed[i] = 0;\n"
        "    for (int i = 0; i < GAR_RING * GAR_PARTS; ++i) {\n"
-       "      asm volatile(\"mbarrier.init.shared::cta.b64 [%0], %1;\" :: \"r\"(full + 8 * i), \"r\"(GAR_COLS) : \"memory\");\n"
+       "      asm volatile(\"mbarrier.init.shared::cta.b64 [%0], %1;\" :: \"r\"(full + 8 * i), \"r\"(GAR_COLS + GAR_PHANTOM) : \"memory\");\n"
        "    }\n"
        "  }\n";
   // launched with programmatic stream serialisation: nothing is read before every
@@ -1439,7 +1443,7 @@ CodegenResult generate_fused_stream_source(const gar_plan &pl, int max_groups) {
   s += "    const int b = ok && e < hi ? gar_whole(e) : -1;\n"
        "    if (b >= 0 && !gar_eval_st(rows + 8 * b, at + 4 * lane, e, s_handed + slot, bar, turn)) {\n"
        "      ok = false;\n"
-       "      gar_stuck = 1;\n"
+       "      atomicAdd(gar_gave_up + a.slot, 1u);\n"
        "    }\n"
        // every thread of the group has read its column: the slot takes the tile RING turns on
        "    __syncwarp();\n"

@@ -79,7 +79,17 @@ struct JitKernel;  // jit.cpp
 // What a loaded kernel has of its own on each device.
 struct JitOnDevice {
   int blocks_per_sm = 0;     // resident CTAs (0: not loaded on the device yet)
-  void *stuck = nullptr;     // streaming form: device flag, 1 once a wait gave up
+  void *gave_up = nullptr;   // streaming form: GAR_WAIT_SLOTS device counters of waits that gave up
+};
+
+// Plans that share a streaming kernel count its failed waits apart, each in a slot of its
+// own (beyond GAR_WAIT_SLOTS plans on a device a slot has several, which all report its
+// failures).  The counters are the kernel's, so launches captured into a graph may outlive
+// their plan.
+constexpr int GAR_WAIT_SLOTS = 64;
+struct WaitSlots {
+  int users[GAR_WAIT_SLOTS] = {};
+  unsigned int seen[GAR_WAIT_SLOTS] = {};  // count that a status call has read
 };
 
 constexpr int GAR_HOST_CHUNKS_MAX = 16;  // element chunks of the pipelined host path
@@ -115,7 +125,9 @@ struct gar_plan {
   gar::JitKernel *fused = nullptr;   // owned by the JIT cache
   gar::JitOnDevice fused_on;         // the loaded kernel on the plan's device
   gar_stream_t fused_stream = nullptr;  // of the last launch of a kernel with bounded waits
-  bool ran_waiting = false;
+  bool ran_waiting = false;             // such a launch was made
+  int wait_slot = -1;                   // its counter, and the count that is known
+  unsigned int waits_seen = 0;
   int fused_width = 0;
   // kernels of the batches whose first plan this is, by (n, dtype, op) and the plans' programs
   std::vector<std::pair<std::vector<uint64_t>, gar::JitKernel *>> batched;
@@ -187,11 +199,16 @@ struct JitKernel {
   int regs = 0, local_bytes = 0;
   bool loaded = false;
   std::vector<JitOnDevice> on;  // by device ordinal (jit_load's)
+  std::vector<WaitSlots> slots; // by device ordinal
 };
 int jit_compile(const CodegenResult &cg, JitKernel **out);
 // Loads a kernel once per process and sets it up once per device, for the current one;
 // *here: what it has there.
 int jit_load(JitKernel *k, JitOnDevice *here = nullptr);
+// A wait slot of a kernel that is loaded on device dev, its known count, and its return
+int jit_take_slot(JitKernel *k, int dev, unsigned int *seen);
+void jit_seen_slot(JitKernel *k, int dev, int slot, unsigned int seen);
+void jit_drop_slot(JitKernel *k, int dev, int slot);
 
 // step_kernels.cu
 int num_sms();

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <nvrtc.h>
 
+#include <algorithm>
 #include <memory>
 #include <mutex>
 #include <string>
@@ -16,8 +17,10 @@
 namespace gar {
 namespace {
 
-std::mutex g_mu;
-std::unordered_map<std::string, std::unique_ptr<JitKernel>> g_cache;
+// never destroyed: a plan may be destroyed after this file's static objects would be
+std::mutex &g_mu = *new std::mutex;
+std::unordered_map<std::string, std::unique_ptr<JitKernel>> &g_cache =
+    *new std::unordered_map<std::string, std::unique_ptr<JitKernel>>;
 
 }  // namespace
 
@@ -115,7 +118,7 @@ int jit_load(JitKernel *k, JitOnDevice *here) {
     }
     if (k->form == GAR_FORM_STREAM) {
       size_t bytes = 0;
-      e = cudaLibraryGetGlobal(&on.stuck, &bytes, (cudaLibrary_t)k->library, "gar_stuck");
+      e = cudaLibraryGetGlobal(&on.gave_up, &bytes, (cudaLibrary_t)k->library, "gar_gave_up");
       if (e != cudaSuccess) return cuda_fail(e, "cudaLibraryGetGlobal");
     }
     int nb = 0;
@@ -128,6 +131,26 @@ int jit_load(JitKernel *k, JitOnDevice *here) {
   }
   if (here != nullptr) *here = on;
   return GAR_OK;
+}
+
+int jit_take_slot(JitKernel *k, int dev, unsigned int *seen) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (k->slots.size() <= (size_t)dev) k->slots.resize((size_t)dev + 1);
+  WaitSlots &w = k->slots[(size_t)dev];
+  const int slot = (int)(std::min_element(w.users, w.users + GAR_WAIT_SLOTS) - w.users);
+  ++w.users[slot];
+  *seen = w.seen[slot];
+  return slot;
+}
+
+void jit_seen_slot(JitKernel *k, int dev, int slot, unsigned int seen) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  k->slots[(size_t)dev].seen[slot] = seen;
+}
+
+void jit_drop_slot(JitKernel *k, int dev, int slot) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  --k->slots[(size_t)dev].users[slot];
 }
 
 }  // namespace gar

@@ -340,7 +340,8 @@ def ensure_workspace(plan: Plan, device=None):
 
 
 def gar_plan_status(plan: Plan) -> int:
-    """GAR_OK, or the status code of the last persistent Allreduce (raises on CUDA errors)."""
+    """GAR_OK, or GAR_ETIMEOUT (-8) if a bounded wait of the last persistent Allreduce, or of a
+    fused one in the streaming form, gave up (raises on CUDA errors)."""
     rc = _lib.gar_plan_status(plan.handle)
     if rc not in (GAR_OK, -8):
         _check(rc, "gar_plan_status")

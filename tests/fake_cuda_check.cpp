@@ -48,10 +48,65 @@ void two_devices() {
   }
 }
 
+// Plans that share a streaming kernel report their own failed waits, each failure once,
+// also of a replay that the host made no call for; a capture is not waited for.
+void wait_status() {
+  const int P = 127, first = 16 * P + 16;            // gar_args of a program without rotation
+  const std::vector<void *> r = rows(P);
+  std::vector<gar_plan *> pl;
+  uint64_t slot = 0;
+  fake::Function *f = nullptr;
+  fake::on_launch = [&](fake::Function &k, const fake::Launch &ln) {
+    f = &k;
+    std::memcpy(&slot, static_cast<char *>(ln.args[0]) + first, 8);
+    return cudaSuccess;
+  };
+  // a kernel's wait that gives up, on the device
+  auto give_up = [&](uint64_t s) {
+    CHECK(f->globals.size() == 1);
+    const std::string name = f->globals.begin()->first.second;
+    ++reinterpret_cast<unsigned *>(f->globals.begin()->second.data())[name == "gar_gave_up" ? s : 0];
+  };
+  std::vector<uint64_t> slots;
+  for (int k = 0; k < 2; ++k) {
+    pl.push_back(plan_of(P, 1u << 20, GAR_BF16, 7));
+    CHECK(gar_plan_status(pl[k]) == GAR_OK);
+    CHECK(gar_allreduce(pl[k], r.data(), GAR_FUSED, nullptr) == GAR_OK && form_of(pl[k]) == GAR_FORM_STREAM);
+    slots.push_back(slot);
+  }
+  give_up(slots[1]);
+  CHECK(gar_plan_status(pl[0]) == GAR_OK);
+  CHECK(gar_plan_status(pl[1]) == GAR_ETIMEOUT);
+  CHECK(gar_plan_status(pl[1]) == GAR_OK);
+  give_up(slots[0]);                                  // a replay
+  CHECK(gar_plan_status(pl[1]) == GAR_OK);
+  CHECK(gar_plan_status(pl[0]) == GAR_ETIMEOUT);
+  fake::capture = cudaStreamCaptureStatusActive;
+  fake::on_synchronize = [](cudaStream_t) { return cudaErrorStreamCaptureUnsupported; };
+  CHECK(gar_plan_status(pl[0]) == GAR_OK);
+  fake::capture = cudaStreamCaptureStatusNone;
+  fake::on_synchronize = nullptr;
+  // more plans than slots: nobody's failure is lost, and a destroyed plan's slot is free again
+  while (pl.size() < 70) {
+    pl.push_back(plan_of(P, 1u << 20, GAR_BF16, 7));
+    CHECK(gar_allreduce(pl.back(), r.data(), GAR_FUSED, nullptr) == GAR_OK);
+    CHECK(gar_plan_status(pl.back()) == GAR_OK);
+    slots.push_back(slot);
+  }
+  CHECK(slots[69] == slots[5]);
+  give_up(slots[69]);
+  for (size_t k = 0; k < pl.size(); ++k) CHECK(gar_plan_status(pl[k]) == (k == 5 || k == 69 ? GAR_ETIMEOUT : GAR_OK));
+  for (gar_plan *p : pl) gar_plan_destroy(p);
+  gar_plan *again = plan_of(P, 1u << 20, GAR_BF16, 7);
+  CHECK(gar_allreduce(again, r.data(), GAR_FUSED, nullptr) == GAR_OK && slot == 0);
+  CHECK(gar_plan_status(again) == GAR_OK);
+  gar_plan_destroy(again);
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}};
+  const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

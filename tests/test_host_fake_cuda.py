@@ -48,3 +48,7 @@ def _run(program, check, **env):
 
 def test_equal_plans_on_two_devices(program):
     _run(program, "two_devices")
+
+
+def test_failed_waits_of_plans_that_share_a_kernel(program):
+    _run(program, "wait_status")
