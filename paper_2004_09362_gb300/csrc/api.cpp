@@ -264,7 +264,7 @@ int prepare_coop(gar_plan *pl) {
 int prepare_stream(gar_plan *pl) {
   JitKernel *k = nullptr;
   JitOnDevice on;
-  for (int groups = 0;;) {
+  for (int groups = 0, threads = 0;;) {
     CodegenResult cg;
     try {
       cg = generate_fused_stream_source(*pl, groups);
@@ -275,7 +275,9 @@ int prepare_stream(gar_plan *pl) {
     if (int rc = jit_compile(cg, &k)) return rc;
     if (int rc = jit_load(k, &on)) return rc;
     groups = k->threads / 128 - 1;
-    if (k->local_bytes == 0 || groups < 2) break;  // spilled: one group less, with its registers
+    // spilled: one group less, with its registers (unless the groups are forced)
+    if (k->local_bytes == 0 || groups < 2 || k->threads == threads) break;
+    threads = k->threads;
   }
   pl->fused = k;
   pl->fused_on = on;

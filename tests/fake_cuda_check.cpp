@@ -103,10 +103,23 @@ void wait_status() {
   gar_plan_destroy(again);
 }
 
+// A streaming kernel that spills is built with fewer groups, down to two; a forced number of
+// groups is kept.
+void stream_groups() {
+  fake::local_bytes = 64;
+  gar_plan *pl = plan_of(127, 1u << 20, GAR_BF16, 7);
+  CHECK(gar_plan_prepare(pl, GAR_FUSED) == GAR_OK && form_of(pl) == GAR_FORM_STREAM);
+  const std::vector<void *> r = rows(127);
+  CHECK(gar_allreduce(pl, r.data(), GAR_FUSED, nullptr) == GAR_OK);
+  const char *forced = std::getenv("GAR_TUNE_ST_GROUPS");
+  CHECK(fake::launches[0].block == 128u * (forced ? std::atoi(forced) : 2));
+  gar_plan_destroy(pl);
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}};
+  const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

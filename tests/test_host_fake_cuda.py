@@ -42,7 +42,7 @@ def program(tmp_path_factory):
 
 
 def _run(program, check, **env):
-    r = subprocess.run([program, check], capture_output=True, text=True, timeout=120, env={**os.environ, **env})
+    r = subprocess.run([program, check], capture_output=True, text=True, timeout=30, env={**os.environ, **env})
     assert r.returncode == 0, r.stdout + r.stderr
 
 
@@ -52,3 +52,8 @@ def test_equal_plans_on_two_devices(program):
 
 def test_failed_waits_of_plans_that_share_a_kernel(program):
     _run(program, "wait_status")
+
+
+@pytest.mark.parametrize("forced", ["", "3", "4"])
+def test_groups_of_a_streaming_kernel_that_spills(program, forced):
+    _run(program, "stream_groups", **({"GAR_TUNE_ST_GROUPS": forced} if forced else {}))
