@@ -486,14 +486,18 @@ int batched_kernel(gar_plan *owner, const std::vector<const gar_plan *> &ps, Jit
   key.insert(key.end(), {owner->n, (uint64_t)owner->dtype, (uint64_t)owner->op});
   for (const gar_plan *pl : ps)
     key.insert(key.end(), {(uint64_t)pl->P, (uint64_t)pl->S, (uint64_t)pl->group, (uint64_t)pl->ring});
-  for (const auto &known : owner->batched)
-    if (known.first == key) {
-      *out = known.second;
-      return GAR_OK;
-    }
+  {
+    std::lock_guard<std::mutex> lock(owner->batched_mu);
+    for (const auto &known : owner->batched)
+      if (known.first == key) {
+        *out = known.second;
+        return GAR_OK;
+      }
+  }
   CodegenResult cg = generate_batched_source(ps);
   int rc = jit_compile(cg, out);
   if (rc) return rc;
+  std::lock_guard<std::mutex> lock(owner->batched_mu);
   if (owner->batched.size() >= 8) owner->batched.erase(owner->batched.begin());
   owner->batched.emplace_back(std::move(key), *out);
   return GAR_OK;

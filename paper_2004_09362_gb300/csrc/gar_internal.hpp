@@ -4,6 +4,7 @@
 
 #include <cstdint>
 #include <cstddef>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -129,8 +130,10 @@ struct gar_plan {
   int wait_slot = -1;                   // its counter, and the count that is known
   unsigned int waits_seen = 0;
   int fused_width = 0;
-  // kernels of the batches whose first plan this is, by (n, dtype, op) and the plans' programs
+  // kernels of the batches whose first plan this is, by (n, dtype, op) and the plans' programs;
+  // batches of several threads may share their plans
   std::vector<std::pair<std::vector<uint64_t>, gar::JitKernel *>> batched;
+  std::mutex batched_mu;
   bool fused_ready = false;          // the kernel to run has been chosen and loaded
   // persistent step-faithful mode: launch table, barrier state, barrier parameters
   void *d_launches = nullptr;

@@ -3,6 +3,7 @@
 #include "fake_cuda.hpp"
 
 #include <cstdint>
+#include <thread>
 
 namespace {
 
@@ -116,10 +117,29 @@ void stream_groups() {
   gar_plan_destroy(pl);
 }
 
+// Threads batch over shared plans, in more sets than a plan remembers.
+void batched_threads() {
+  std::vector<gar_plan *> pl;
+  for (int P = 2; P < 14; ++P) pl.push_back(plan_of(P, 100, GAR_F32, GAR_STEPS_BO));
+  alignas(8) static gar_batch_desc desc[1];
+  std::vector<std::thread> threads;
+  for (int t = 0; t < 4; ++t)
+    threads.emplace_back([&, t] {
+      for (int k = 0; k < 60; ++k) {
+        gar_plan *set[2] = {pl[0], pl[1 + (5 * t + k) % 11]};
+        CHECK(gar_allreduce_batched(set, 2, desc, 1, nullptr) == GAR_OK);
+      }
+    });
+  for (std::thread &t : threads) t.join();
+  CHECK(fake::compiles == 11 && fake::launches.size() == 240);
+  for (gar_plan *p : pl) gar_plan_destroy(p);
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
-  const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups}};
+  const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups},
+      {"batched_threads", batched_threads}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

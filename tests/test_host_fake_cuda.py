@@ -57,3 +57,13 @@ def test_failed_waits_of_plans_that_share_a_kernel(program):
 @pytest.mark.parametrize("forced", ["", "3", "4"])
 def test_groups_of_a_streaming_kernel_that_spills(program, forced):
     _run(program, "stream_groups", **({"GAR_TUNE_ST_GROUPS": forced} if forced else {}))
+
+
+def test_threads_that_batch_over_shared_plans(tmp_path):
+    """Under the thread sanitizer (exit code 66 of a race)."""
+    (tmp_path / "t.cpp").write_text("int main() {}")
+    flags = ["-O1", "-g", "-fsanitize=thread"]
+    probe = f"g++ {' '.join(flags)} {tmp_path}/t.cpp -o {tmp_path}/t && {tmp_path}/t"
+    if subprocess.run(probe, shell=True, capture_output=True).returncode != 0:
+        pytest.skip("no thread sanitizer here")
+    _run(_program(tmp_path, flags), "batched_threads")
