@@ -132,6 +132,15 @@ bool coop_form_applies(const gar_plan &pl) {
   return pl.P > 1 && values * (32 * 4 + 4) + (size_t)pl.P * 16 <= 220 * 1024;
 }
 
+// Whether a knob of the single-thread or the breadth-first form is set: such a plan keeps to
+// these forms.
+bool older_form_tuned() {
+  for (const char *name : {"FUSED_W", "FUSED_THREADS", "FUSED_MINB", "DOUBLED", "FADD2", "BF_ORDER", "BF_WARPS", "BF_MINB",
+                           "BF_GROUPS"})
+    if (const char *v = std::getenv((std::string("GAR_TUNE_") + name).c_str()); v && *v) return true;
+  return false;
+}
+
 // The fused kernel a plan uses.  Float sums with several result copies whose
 // single-thread program keeps more than 160 values alive per element position (P = 127
 // at S = 7 and 8: 254 and 192) are register-bound in that form and take the
@@ -208,7 +217,7 @@ int compile_fused(gar_plan *pl) {
 // max, min and int32 (0.92 to 1.27, no clear line).
 bool takes_stream(const gar_plan &pl) {
   const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
-  if (ff && *ff) return false;
+  if ((ff && *ff) || older_form_tuned()) return false;
   if (pl.op != GAR_SUM || pl.dtype == GAR_I32 || pl.n < (1u << 19) || !stream_form_applies(pl)) return false;
   const int live = fused_peak_live(pl);
   return pl.dtype == GAR_BF16 ? live > 160 : live > 210 && pl.n >= (1u << 20);
@@ -233,8 +242,8 @@ bool takes_stream(const gar_plan &pl) {
 //    S = 7, 1000 4.2 -> 2.2, 2500 4.3 -> 7.8; P = 127, S = 7, 500 4.2 -> 3.7, but with the
 //    GPU waited for 17.3 -> 19.6).
 bool takes_coop(const gar_plan &pl) {
-  for (const char *name : {"GAR_TUNE_FUSED_FORM", "GAR_TUNE_FUSED_W", "GAR_TUNE_FUSED_THREADS", "GAR_TUNE_FUSED_MINB"})
-    if (const char *v = std::getenv(name); v && *v) return false;
+  const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
+  if ((ff && *ff) || older_form_tuned()) return false;
   const uint64_t wave = 32 * 152;
   if (pl.P < 16 || pl.n > 2 * wave || !coop_form_applies(pl) || fused_levels(pl) > 10) return false;
   if (pl.K == 1) return pl.n <= (pl.P <= 32 ? 2 * wave : wave);
@@ -477,13 +486,13 @@ int run_fused(gar_plan *pl, void *const *rank, gar_stream_t stream) {
 }
 
 // The kernel of a batch over these plans.  Its first plan remembers the kernels of the
-// last few sets of plans by what determines their programs, so that a call does not
+// last few sets of plans by what determines their programs and source, so that a call does not
 // generate the source again just to look the kernel up (25 us; a batch of 16 425-byte
 // Allreduces 24 -> 4 us a call).
 int batched_kernel(gar_plan *owner, const std::vector<const gar_plan *> &ps, JitKernel **out) {
   std::vector<uint64_t> key;
-  key.reserve(ps.size() * 4 + 3);
-  key.insert(key.end(), {owner->n, (uint64_t)owner->dtype, (uint64_t)owner->op});
+  key.reserve(ps.size() * 4 + 4);
+  key.insert(key.end(), {owner->n, (uint64_t)owner->dtype, (uint64_t)owner->op, batched_knobs()});
   for (const gar_plan *pl : ps)
     key.insert(key.end(), {(uint64_t)pl->P, (uint64_t)pl->S, (uint64_t)pl->group, (uint64_t)pl->ring});
   {

@@ -1611,6 +1611,16 @@ CodegenResult generate_fused_coop_source(const gar_plan &pl) {
   return cg;
 }
 
+uint64_t batched_knobs() {
+  uint64_t h = 14695981039346656037ull;  // FNV-1a
+  for (const char *name : {"GAR_TUNE_FADD2", "GAR_TUNE_LDH", "GAR_TUNE_STH"}) {
+    const char *v = std::getenv(name);
+    h = (h ^ (v != nullptr)) * 1099511628211ull;
+    for (; v != nullptr && *v; ++v) h = (h ^ (unsigned char)*v) * 1099511628211ull;
+  }
+  return h;
+}
+
 CodegenResult generate_batched_source(const std::vector<const gar_plan *> &plans) {
   const gar_plan &p0 = *plans[0];
   int peak = 1;

@@ -185,6 +185,7 @@ CodegenResult generate_fused_coop_source(const gar_plan &pl);
 int fused_peak_live(const gar_plan &pl);
 int fused_levels(const gar_plan &pl);  // of combines that depend on one another
 CodegenResult generate_batched_source(const std::vector<const gar_plan *> &plans);
+uint64_t batched_knobs();  // of the tuning knobs that its source depends on
 
 // jit.cpp
 struct JitKernel {

@@ -135,11 +135,37 @@ void batched_threads() {
   for (gar_plan *p : pl) gar_plan_destroy(p);
 }
 
+// A knob that changes a batched kernel's source reaches plans that remember a kernel, and a
+// knob of the single-thread or breadth-first form keeps a plan to that form.
+void knobs() {
+  gar_plan *pl = plan_of(5, 100, GAR_BF16, GAR_STEPS_BO);
+  alignas(8) static gar_batch_desc desc[1];
+  int compiles = 0;
+  for (const char *hint : {".cs", ".cs", ".cg", ".cg", ".cs"}) {
+    setenv("GAR_TUNE_LDH", hint, 1);
+    CHECK(gar_allreduce_batched(&pl, 1, desc, 1, nullptr) == GAR_OK);
+    compiles += compiles == 0 || (compiles == 1 && std::string(hint) == ".cg");
+    CHECK(fake::compiles == compiles);
+  }
+  gar_plan_destroy(pl);
+  struct { const char *knob; int P; uint64_t n; int steps, form; } cases[] = {
+      {"", 127, 1u << 20, 7, GAR_FORM_STREAM},  {"GAR_TUNE_BF_WARPS", 127, 1u << 20, 7, GAR_FORM_BREADTH},
+      {"GAR_TUNE_BF_ORDER", 127, 1u << 20, 7, GAR_FORM_BREADTH}, {"", 24, 100, 7, GAR_FORM_COOP},
+      {"GAR_TUNE_DOUBLED", 24, 100, 7, GAR_FORM_SINGLE}, {"GAR_TUNE_FADD2", 24, 100, 10, GAR_FORM_SINGLE}};
+  for (const auto &c : cases) {
+    if (*c.knob) setenv(c.knob, "1", 1);
+    pl = plan_of(c.P, c.n, GAR_BF16, c.steps);
+    CHECK(gar_plan_prepare(pl, GAR_FUSED) == GAR_OK && form_of(pl) == c.form);
+    if (*c.knob) unsetenv(c.knob);
+    gar_plan_destroy(pl);
+  }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups},
-      {"batched_threads", batched_threads}};
+      {"batched_threads", batched_threads}, {"knobs", knobs}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

@@ -67,3 +67,7 @@ def test_threads_that_batch_over_shared_plans(tmp_path):
     if subprocess.run(probe, shell=True, capture_output=True).returncode != 0:
         pytest.skip("no thread sanitizer here")
     _run(_program(tmp_path, flags), "batched_threads")
+
+
+def test_tuning_knobs_reach_the_kernels_they_shape(program):
+    _run(program, "knobs")
