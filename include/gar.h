@@ -144,13 +144,13 @@ typedef struct {
  * latency-optimal cyclic schedules (every placement holds its own result copy) and
  * taken only when forced (environment GAR_TUNE_FUSED_FORM=2): on GB300 it was slower
  * than the breadth-first form.  GAR_FORM_STREAM: the program as a stream over placements
- * with the contributions in shared memory; a prepared plan (gar_plan_prepare or a first
- * fused call) of a bf16 sum that would take the breadth-first form runs it from 2^19
- * elements per rank on, an fp32 sum with more than 210 values alive from 2^20 on; before
- * that its info and source are the breadth-first form's.  GAR_FORM_COOP: a CTA takes a tile
- * of a few positions and spreads the program over its threads; a prepared plan of 16 and
- * more ranks with few element positions (some thousands; the line depends on P and S) runs
- * it.  All forms give the same bits. */
+ * with the contributions in shared memory; a bf16 sum that would take the breadth-first form
+ * runs it from 2^19 elements per rank on, an fp32 sum with more than 210 values alive from
+ * 2^20 on.  GAR_FORM_COOP: a CTA takes a tile of a few positions and spreads the program over
+ * its threads; plans of 16 and more ranks with few element positions (some thousands; the line
+ * depends on P and S) run it.  Info and source name these two once the plan is compiled
+ * (gar_plan_compile, gar_plan_prepare or a first fused call), and one of the first two before
+ * that.  All forms give the same bits. */
 enum { GAR_FORM_SINGLE = 0, GAR_FORM_BREADTH = 1, GAR_FORM_SPLIT = 2, GAR_FORM_STREAM = 3, GAR_FORM_COOP = 4 };
 
 /* Creates a schedule for P virtual ranks of n elements each.
@@ -230,13 +230,14 @@ GAR_API int gar_plan_set_workspace(gar_plan *plan, void *dev_ptr, size_t bytes);
 
 /* The CUDA C source of the plan's generated fused kernel (host-only): of the kernel the
  * plan runs once it is prepared (gar_plan_prepare or a first fused call, which rebuild a
- * kernel of more than 128 registers in 64-thread CTAs, and choose the streaming or the
- * cooperative form), else of its first compile.
+ * kernel of more than 128 registers in 64-thread CTAs), of its first compile once it is
+ * compiled, and before that of the form in its info.
  * Copies at most *len bytes (including the terminating NUL) to buf and sets *len to the full size
  * including the NUL; pass buf == NULL to query the size. */
 GAR_API int gar_plan_fused_source(const gar_plan *plan, char *buf, size_t *len);
 
-/* Compiles (host-only, needs no GPU) the specialized kernel for `mode`.  Optional:
+/* Compiles (host-only, needs no GPU) the specialized kernel for `mode`, in the form that the
+ * plan runs.  Optional:
  * gar_plan_prepare and the first Allreduce compile on demand. */
 GAR_API int gar_plan_compile(gar_plan *plan, int mode);
 

@@ -145,8 +145,8 @@ bool older_form_tuned() {
 // single-thread program keeps more than 160 values alive per element position (P = 127
 // at S = 7 and 8: 254 and 192) are register-bound in that form and take the
 // breadth-first form (0.59 instead of 0.68 ms, and 0.47 instead of 0.56 ms, at P = 127 x
-// 8 MiB bf16 on GB300); every other plan takes the single-thread form.  Preparation may
-// choose the streaming or the cooperative form instead (takes_stream, takes_coop).
+// 8 MiB bf16 on GB300); every other plan takes the single-thread form.  Compilation and
+// preparation may choose the streaming or the cooperative form instead (chosen_form).
 // GAR_TUNE_FUSED_FORM (0 to 4) forces one form, for parity tests and launch-shape sweeps; the two-lane
 // form (2) exists for latency-optimal cyclic programs only and is never the default (P =
 // 127 x 8 MiB bf16 S = 7: 0.78 ms against 0.60 ms breadth-first in one pass, 0.55 ms in
@@ -165,49 +165,7 @@ int fused_form(const gar_plan &pl) {
                                                                                 : GAR_FORM_SINGLE;
 }
 
-CodegenResult fused_codegen(const gar_plan &pl) {
-  switch (fused_form(pl)) {
-    case GAR_FORM_BREADTH: return generate_fused_bf_source(pl);
-    case GAR_FORM_SPLIT: return generate_fused_split_source(pl);
-    case GAR_FORM_STREAM: return generate_fused_stream_source(pl);
-    case GAR_FORM_COOP: return generate_fused_coop_source(pl);
-    default: return generate_fused_source(pl);
-  }
-}
-
-int compile_fused(gar_plan *pl) {
-  if (pl->fused) return GAR_OK;
-  if (int rc = check_fused_size(pl)) return rc;
-  CodegenResult cg;
-  try {
-    cg = fused_codegen(*pl);
-  } catch (const std::exception &ex) {
-    set_error(std::string("fused code generation: ") + ex.what());
-    return GAR_EINVAL;
-  }
-  JitKernel *k = nullptr;
-  int rc = jit_compile(cg, &k);
-  if (rc) return rc;
-  pl->fused = k;
-  pl->fused_width = k->width;
-  return GAR_OK;
-}
-
-// Register-heavy single-thread kernels (more than 128 registers once loaded) run in
-// 64-thread CTAs capped at 168 registers, so that three warps share each sub-partition's
-// register file and the small CTAs of an SM drift apart.  On GB300: P = 32 x 32 MiB bf16
-// latency-optimal (208 registers) 0.426 -> 0.338 ms; P = 127 x 8 MiB bf16 S = 9 (200)
-// 0.434 -> 0.401 ms, S = 11 (174) 0.344 -> 0.324 ms; kernels at 128 registers or fewer
-// were unchanged or slower (P = 64 fp32 latency-optimal, 40 registers: 0.33 -> 0.40 ms).
-// When the 168-register build spills more than 256 bytes per thread, 32-thread CTAs with
-// the full 255 registers (two warps per sub-partition) are built too and kept if they
-// spill less: P = 127 x 8 MiB bf16 S = 10 (168 registers + 328 B spilled, 0.369 ms;
-// 250 registers, no spill, 0.351 ms).  Smaller spills cost less than the lost warps:
-// P = 32 x 32 MiB bf16 S = 5 (152 B: 0.341 ms against 0.390 ms at 210 registers),
-// P = 64 x 16 MiB bf16 S = 8 (96 B: 0.324 against 0.346), P = 127 S = 9 (48 B: 0.407
-// against 0.460).
-// The counts are the loaded kernel's own (the compiler's log does not always carry them).
-// Whether a prepared plan runs the streaming form (cyclic programs in long vectors).  bf16
+// Whether a plan runs the streaming form (cyclic programs in long vectors).  bf16
 // sums that would take the breadth-first form do from 2^19 positions on (GB300, against the
 // breadth-first form, P = 84 to 127 at S = 7 and 8: 1.13 to 1.67 times as fast from 2^19 to
 // 2^22 positions; 0.91 to 1.21 at 2^18, where an SM has too few tiles); fp32 sums only with
@@ -223,7 +181,7 @@ bool takes_stream(const gar_plan &pl) {
   return pl.dtype == GAR_BF16 ? live > 160 : live > 210 && pl.n >= (1u << 20);
 }
 
-// Whether a prepared plan runs the cooperative form.  GB300, us per fused call in graph
+// Whether a plan runs the cooperative form.  GB300, us per fused call in graph
 // replay, the other form -> cooperative (bf16; fp32 within a few per cent):
 //  * P below 16 gains little or loses (P = 12, S = 8 2.3 -> 1.7, S = 5 1.7 -> 1.7; P = 6
 //    1.3 -> 1.5), and so do the many levels of the Ring and of most folds (P = 48 2.5 -> 4.3).
@@ -252,41 +210,55 @@ bool takes_coop(const gar_plan &pl) {
   return pl.K < pl.P && pl.n <= wave && work <= most;
 }
 
-int prepare_coop(gar_plan *pl) {
-  JitKernel *k = nullptr;
-  JitOnDevice on;
+// The form that a plan runs.
+int chosen_form(const gar_plan &pl) {
+  return takes_stream(pl) ? GAR_FORM_STREAM : takes_coop(pl) ? GAR_FORM_COOP : fused_form(pl);
+}
+
+CodegenResult fused_codegen(const gar_plan &pl, int form) {
+  switch (form) {
+    case GAR_FORM_BREADTH: return generate_fused_bf_source(pl);
+    case GAR_FORM_SPLIT: return generate_fused_split_source(pl);
+    case GAR_FORM_STREAM: return generate_fused_stream_source(pl);
+    case GAR_FORM_COOP: return generate_fused_coop_source(pl);
+    default: return generate_fused_source(pl);
+  }
+}
+
+// Compiles the source that `generate` returns; *out: the kernel.
+template <typename Generate>
+int compile_source(const Generate &generate, JitKernel **out) {
   CodegenResult cg;
   try {
-    cg = generate_fused_coop_source(*pl);
+    cg = generate();
   } catch (const std::exception &ex) {
     set_error(std::string("fused code generation: ") + ex.what());
     return GAR_EINVAL;
   }
-  if (int rc = jit_compile(cg, &k)) return rc;
-  if (int rc = jit_load(k, &on)) return rc;
-  pl->fused = k;
-  pl->fused_on = on;
-  pl->fused_width = k->width;
-  return GAR_OK;
+  return jit_compile(cg, out);
 }
 
-int prepare_stream(gar_plan *pl) {
+// Compiles the kernel of the form that the plan runs (host only).
+int compile_fused(gar_plan *pl) {
+  if (pl->fused) return GAR_OK;
+  if (int rc = check_fused_size(pl)) return rc;
   JitKernel *k = nullptr;
-  JitOnDevice on;
-  for (int groups = 0, threads = 0;;) {
-    CodegenResult cg;
-    try {
-      cg = generate_fused_stream_source(*pl, groups);
-    } catch (const std::exception &ex) {
-      set_error(std::string("fused code generation: ") + ex.what());
-      return GAR_EINVAL;
-    }
-    if (int rc = jit_compile(cg, &k)) return rc;
+  if (int rc = compile_source([&] { return fused_codegen(*pl, chosen_form(*pl)); }, &k)) return rc;
+  pl->fused = k;
+  pl->fused_width = k->width;
+  return GAR_OK;
+}
+
+// A streaming kernel that spilled gives way to one with a group less and its registers
+// (unless the groups are forced).
+int refine_stream(gar_plan *pl) {
+  JitKernel *k = pl->fused;
+  JitOnDevice on = pl->fused_on;
+  while (k->local_bytes > 0 && k->threads > 2 * 128) {
+    const int threads = k->threads;
+    if (int rc = compile_source([&] { return generate_fused_stream_source(*pl, threads / 128 - 1); }, &k)) return rc;
     if (int rc = jit_load(k, &on)) return rc;
-    groups = k->threads / 128 - 1;
-    // spilled: one group less, with its registers (unless the groups are forced)
-    if (k->local_bytes == 0 || groups < 2 || k->threads == threads) break;
-    threads = k->threads;
+    if (k->threads == threads) break;
   }
   pl->fused = k;
   pl->fused_on = on;
@@ -294,34 +266,32 @@ int prepare_stream(gar_plan *pl) {
   return GAR_OK;
 }
 
+// Register-heavy single-thread kernels (more than 128 registers once loaded) run in
+// 64-thread CTAs capped at 168 registers, so that three warps share each sub-partition's
+// register file and the small CTAs of an SM drift apart.  On GB300: P = 32 x 32 MiB bf16
+// latency-optimal (208 registers) 0.426 -> 0.338 ms; P = 127 x 8 MiB bf16 S = 9 (200)
+// 0.434 -> 0.401 ms, S = 11 (174) 0.344 -> 0.324 ms; kernels at 128 registers or fewer
+// were unchanged or slower (P = 64 fp32 latency-optimal, 40 registers: 0.33 -> 0.40 ms).
+// When the 168-register build spills more than 256 bytes per thread, 32-thread CTAs with
+// the full 255 registers (two warps per sub-partition) are built too and kept if they
+// spill less: P = 127 x 8 MiB bf16 S = 10 (168 registers + 328 B spilled, 0.369 ms;
+// 250 registers, no spill, 0.351 ms).  Smaller spills cost less than the lost warps:
+// P = 32 x 32 MiB bf16 S = 5 (152 B: 0.341 ms against 0.390 ms at 210 registers),
+// P = 64 x 16 MiB bf16 S = 8 (96 B: 0.324 against 0.346), P = 127 S = 9 (48 B: 0.407
+// against 0.460).
+// The counts are the loaded kernel's own (the compiler's log does not always carry them).
 int build_fused(gar_plan *pl) {
-  int rc = check_fused_size(pl);
-  if (rc) return rc;
-  if (takes_stream(*pl)) {
-    if ((rc = ensure_device(pl))) return rc;
-    return prepare_stream(pl);
-  }
-  if (takes_coop(*pl)) {
-    if ((rc = ensure_device(pl))) return rc;
-    return prepare_coop(pl);
-  }
-  rc = compile_fused(pl);
+  int rc = compile_fused(pl);
   if (rc) return rc;
   rc = ensure_device(pl);
   if (rc) return rc;
   if ((rc = jit_load(pl->fused, &pl->fused_on))) return rc;
+  if (pl->fused->form == GAR_FORM_STREAM && takes_stream(*pl)) return refine_stream(pl);
   const bool shape_forced = std::getenv("GAR_TUNE_FUSED_THREADS") || std::getenv("GAR_TUNE_FUSED_MINB");
   if (pl->fused->form != 0 || pl->fused->threads != 256 || shape_forced || pl->fused->regs <= 128)
     return GAR_OK;
   auto build = [&](int threads, int minb, int fadd2, JitKernel **out) -> int {
-    CodegenResult cg;
-    try {
-      cg = generate_fused_source(*pl, threads, minb, fadd2);
-    } catch (const std::exception &ex) {
-      set_error(std::string("fused code generation: ") + ex.what());
-      return GAR_EINVAL;
-    }
-    if (int r = jit_compile(cg, out)) return r;
+    if (int r = compile_source([&] { return generate_fused_source(*pl, threads, minb, fadd2); }, out)) return r;
     return jit_load(*out);
   };
   JitKernel *k = nullptr;
@@ -826,7 +796,7 @@ int gar_plan_fused_source(const gar_plan *pl, char *buf, size_t *len) {
   if (len == nullptr) return GAR_EINVAL;
   std::string src;
   try {
-    src = pl->fused != nullptr ? pl->fused->source : fused_codegen(*pl).source;
+    src = pl->fused != nullptr ? pl->fused->source : fused_codegen(*pl, fused_form(*pl)).source;
   } catch (const std::exception &ex) {
     set_error(std::string("fused code generation: ") + ex.what());
     return GAR_EINVAL;

@@ -161,11 +161,32 @@ void knobs() {
   }
 }
 
+// A plan that is compiled ahead names the form that it will run, and preparing it compiles
+// nothing more.
+void compiled_ahead() {
+  struct { int P; uint64_t n; int dtype, steps, form; } cases[] = {
+      {127, 212, GAR_BF16, 14, GAR_FORM_COOP},      {24, 9000, GAR_F32, 10, GAR_FORM_COOP},
+      {127, 1u << 20, GAR_BF16, 7, GAR_FORM_STREAM}, {127, 1u << 18, GAR_BF16, 7, GAR_FORM_BREADTH},
+      {24, 1u << 20, GAR_F32, 10, GAR_FORM_SINGLE}};
+  for (const auto &c : cases) {
+    const int before = fake::compiles;
+    gar_plan *pl = plan_of(c.P, c.n, c.dtype, c.steps);
+    CHECK(gar_plan_compile(pl, GAR_FUSED) == GAR_OK && form_of(pl) == c.form);
+    size_t len = 0, prepared = 0;
+    CHECK(gar_plan_fused_source(pl, nullptr, &len) == GAR_OK);
+    CHECK(gar_plan_prepare(pl, GAR_FUSED) == GAR_OK && form_of(pl) == c.form);
+    CHECK(gar_plan_fused_source(pl, nullptr, &prepared) == GAR_OK && prepared == len);
+    CHECK(fake::compiles == before + 1);
+    gar_plan_destroy(pl);
+  }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups},
-      {"batched_threads", batched_threads}, {"knobs", knobs}};
+      {"batched_threads", batched_threads}, {"knobs", knobs},
+      {"compiled_ahead", compiled_ahead}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

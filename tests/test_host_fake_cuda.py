@@ -71,3 +71,7 @@ def test_threads_that_batch_over_shared_plans(tmp_path):
 
 def test_tuning_knobs_reach_the_kernels_they_shape(program):
     _run(program, "knobs")
+
+
+def test_a_plan_compiled_ahead_prepares_the_same_kernel(program):
+    _run(program, "compiled_ahead")
