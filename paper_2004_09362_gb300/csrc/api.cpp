@@ -52,6 +52,7 @@ int ensure_device(gar_plan *pl) {
     set_error("plan was prepared on another device");
     return GAR_ESTATE;
   }
+  if (pl->device < 0) pl->sms = num_sms();
   pl->device = dev;
   return GAR_OK;
 }
@@ -202,7 +203,7 @@ bool takes_stream(const gar_plan &pl) {
 bool takes_coop(const gar_plan &pl) {
   const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
   if ((ff && *ff) || older_form_tuned()) return false;
-  const uint64_t wave = 32 * 152;
+  const uint64_t wave = 32 * (uint64_t)pl.sms;
   if (pl.P < 16 || pl.n > 2 * wave || !coop_form_applies(pl) || fused_levels(pl) > 10) return false;
   if (pl.K == 1) return pl.n <= (pl.P <= 32 ? 2 * wave : wave);
   const uint64_t work = pl.n * (2 * (uint64_t)pl.P + pl.prog.a.size());
@@ -281,10 +282,13 @@ int refine_stream(gar_plan *pl) {
 // against 0.460).
 // The counts are the loaded kernel's own (the compiler's log does not always carry them).
 int build_fused(gar_plan *pl) {
-  int rc = compile_fused(pl);
+  // a kernel compiled ahead was chosen for the default SM count
+  const int assumed = pl->sms;
+  int rc = check_fused_size(pl);
   if (rc) return rc;
-  rc = ensure_device(pl);
-  if (rc) return rc;
+  if ((rc = ensure_device(pl))) return rc;
+  if (pl->sms != assumed) pl->fused = nullptr;
+  if ((rc = compile_fused(pl))) return rc;
   if ((rc = jit_load(pl->fused, &pl->fused_on))) return rc;
   if (pl->fused->form == GAR_FORM_STREAM && takes_stream(*pl)) return refine_stream(pl);
   const bool shape_forced = std::getenv("GAR_TUNE_FUSED_THREADS") || std::getenv("GAR_TUNE_FUSED_MINB");

@@ -1517,7 +1517,7 @@ CodegenResult generate_fused_coop_source(const gar_plan &pl) {
   // 16 and 512, 3.6 with 32 and 512 (4.0 with 8, 3.6 and 6.6 in 256 threads); P = 24, 10000
   // at S = 10 1.9 with 32 and 256 (2.1 with 16 and 128, 2.6 with 512).
   int cols = 4, threads = 128;
-  while (cols < 32 && pl.n > 152u * (uint64_t)cols) cols *= 2;
+  while (cols < 32 && pl.n > (uint64_t)pl.sms * (uint64_t)cols) cols *= 2;
   while (threads < 512 && threads < P * cols / 4) threads *= 2;
   CodegenResult cg;
   cg.width = 1;

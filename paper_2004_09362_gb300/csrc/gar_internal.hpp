@@ -118,6 +118,7 @@ struct gar_plan {
   void *ws = nullptr;
   size_t ws_set_bytes = 0;
   int device = -1;
+  int sms = 152;                  // of the device, once it is known (GB300's before that)
   gar::StepOp *d_ops = nullptr;
   unsigned long long *d_step_bytes = nullptr;  // S + 1 rows of STEP_BYTE_SLOTS counters
   bool step_bytes_stale = false;      // a sequence of step launches did not complete

@@ -181,12 +181,32 @@ void compiled_ahead() {
   }
 }
 
+// The line of the cooperative form and its tiles follow the device's SM count, also of a plan
+// that was compiled ahead without one.
+void sm_count() {
+  struct { int sms; uint64_t n; int form; unsigned grid; } cases[] = {
+      {152, 4864, GAR_FORM_COOP, 152}, {152, 4865, GAR_FORM_SINGLE, 0}, {76, 2432, GAR_FORM_COOP, 76},
+      {76, 2433, GAR_FORM_SINGLE, 0},  {76, 300, GAR_FORM_COOP, 75},    {152, 300, GAR_FORM_COOP, 75},
+      {76, 600, GAR_FORM_COOP, 75},    {152, 600, GAR_FORM_COOP, 150}};
+  const std::vector<void *> r = rows(48);
+  for (bool ahead : {false, true})
+    for (const auto &c : cases) {
+      fake::sms[0] = c.sms;
+      fake::launches.clear();
+      gar_plan *pl = plan_of(48, c.n, GAR_F32, 12);
+      if (ahead) CHECK(gar_plan_compile(pl, GAR_FUSED) == GAR_OK);
+      CHECK(gar_allreduce(pl, r.data(), GAR_FUSED, nullptr) == GAR_OK && form_of(pl) == c.form);
+      if (c.form == GAR_FORM_COOP) CHECK(fake::launches[0].grid == c.grid);
+      gar_plan_destroy(pl);
+    }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups},
       {"batched_threads", batched_threads}, {"knobs", knobs},
-      {"compiled_ahead", compiled_ahead}};
+      {"compiled_ahead", compiled_ahead}, {"sm_count", sm_count}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

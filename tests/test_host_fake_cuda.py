@@ -75,3 +75,7 @@ def test_tuning_knobs_reach_the_kernels_they_shape(program):
 
 def test_a_plan_compiled_ahead_prepares_the_same_kernel(program):
     _run(program, "compiled_ahead")
+
+
+def test_the_cooperative_form_follows_the_sm_count(program):
+    _run(program, "sm_count")
