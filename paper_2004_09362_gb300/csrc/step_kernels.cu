@@ -211,9 +211,26 @@ struct LaunchView {
   int group;                  // ops per thread (element-major mapping)
 };
 
-// Elements [c0, c0 + len) of the block that op `op` touches at rank x, by the CTA's NT threads.
+// The bytes that the CTA's NT threads have read from partners, added to a step's counters by
+// one atomic add: every thread stages its count, and after a barrier one thread adds the sums
+// of the warps.
+template <int NT>
+__device__ __forceinline__ void stage_moved(uint32_t *s_moved, uint32_t moved) {
+  const uint32_t sum = __reduce_add_sync(0xffffffffu, moved);
+  if ((threadIdx.x & 31) == 0) s_moved[threadIdx.x >> 5] = sum;
+}
+template <int NT>
+__device__ __forceinline__ void add_moved(unsigned long long *bytes, const uint32_t *s_moved) {
+  unsigned long long total = 0;
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) total += s_moved[w];
+  if (total) atomicAdd(bytes + blockIdx.x % STEP_BYTE_SLOTS, total);
+}
+
+// Elements [c0, c0 + len) of the block that op `op` touches at rank x, by the CTA's NT
+// threads; returns the bytes that this thread has read from the partner.
 template <typename T, int OP, int MAXP, int NT>
-__device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const LaunchView &lv, const StepOp &op, int x,
+__device__ __forceinline__ uint32_t range_work(const StepArgs<MAXP> &a, const LaunchView &lv, const StepOp &op, int x,
                                            uint64_t c0, uint32_t len) {
   using A = typename AccOf<T>::type;
   constexpr bool kMixed = sizeof(T) != sizeof(A);  // rank buffers hold a narrower type than the slices
@@ -221,7 +238,7 @@ __device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const Launch
   const int b = a.xor_group ? (x ^ (int)op.dst_place) : wrap_rank(x - (int)op.dst_place, a.P);
   const uint64_t bstart = (uint64_t)b * a.q + ((uint64_t)b < a.rem ? (uint64_t)b : a.rem);
   const uint64_t blen = a.q + ((uint64_t)b < a.rem ? 1 : 0);
-  if (c0 >= blen) return;
+  if (c0 >= blen) return 0;
   const uint64_t lo = bstart + c0;
   const uint64_t hi = bstart + (blen < c0 + len ? blen : c0 + len);
 
@@ -250,10 +267,12 @@ __device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const Launch
   if (va > hi) va = hi;
   if (vb < va) vb = va;
   const uint32_t head = (uint32_t)(va - lo), ends = head + (uint32_t)(hi - vb);
+  uint32_t moved = 0;  // elements read, partner's or (without one) own
   for (uint32_t k = threadIdx.x; k < ends; k += NT) {
     const uint64_t e = k < head ? lo + k : vb + (k - head);
     A r = A(0);
     if (has_recv) r = load1<T, A>(op.recv_buf, recv, e);
+    ++moved;
     A o0 = r, o1 = r;
     if (own0) o0 = load1<T, A>(op.out0_own, own0, e);
     if (own0 && has_recv) o0 = combine<OP>(o0, r);
@@ -274,7 +293,10 @@ __device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const Launch
       int4 v[U];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (k + u * NT < units) v[u] = src[k + u * NT];
+        if (k + u * NT < units) {
+          v[u] = src[k + u * NT];
+          moved += unit;
+        }
 #pragma unroll
       for (int u = 0; u < U; ++u)
         if (k + u * NT < units) dst[k + u * NT] = v[u];
@@ -296,6 +318,7 @@ __device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const Launch
       for (int u = 0; u < U; ++u)
         if (k + u * NT < units) {
           rv[u] = rp[k + u * NT];
+          moved += 4;
           ov[u] = wp[k + u * NT];
         }
 #pragma unroll
@@ -319,6 +342,7 @@ __device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const Launch
         if (k + u * NT < units) {
           const uint64_t e = va + 4 * (uint64_t)(k + u * NT);
           if (has_recv) load4<T, A>(op.recv_buf, recv, e, r[u]);
+          moved += 4;
           if (own0) load4<T, A>(op.out0_own, own0, e, o0[u]);
           if (own1) load4<T, A>(op.out1_own, own1, e, o1[u]);
         }
@@ -336,20 +360,17 @@ __device__ __forceinline__ void range_work(const StepArgs<MAXP> &a, const Launch
         }
     }
   }
-  // The received bytes: the CTA has read each of its elements from the partner once.
-  if (lv.bytes != nullptr && has_recv && threadIdx.x == 0) {
-    const unsigned long long esize = (op.recv_buf == BUF_RANK) ? sizeof(T) : sizeof(A);
-    atomicAdd(lv.bytes + blockIdx.x % STEP_BYTE_SLOTS, (hi - lo) * esize);
-  }
+  return has_recv ? moved * (uint32_t)(op.recv_buf == BUF_RANK ? sizeof(T) : sizeof(A)) : 0;
 }
 
-// Chunked mapping: work item `item` = (chunk, rank x, op) is done by the whole CTA.
+// Chunked mapping: work item `item` = (chunk, rank x, op) is done by the whole CTA; returns
+// the bytes that this thread has read from the partner.
 template <typename T, int OP, int MAXP>
-__device__ __forceinline__ void chunk_work(const StepArgs<MAXP> &a, const LaunchView &lv, uint32_t item) {
+__device__ __forceinline__ uint32_t chunk_work(const StepArgs<MAXP> &a, const LaunchView &lv, uint32_t item) {
   const int chunk = (int)(item % (uint32_t)lv.nchunks);
   item /= (uint32_t)lv.nchunks;
   const StepOp op = lv.ops[item / (uint32_t)a.P];
-  range_work<T, OP, MAXP, kThreads>(a, lv, op, (int)(item % (uint32_t)a.P), (uint64_t)chunk * lv.chunk, lv.chunk);
+  return range_work<T, OP, MAXP, kThreads>(a, lv, op, (int)(item % (uint32_t)a.P), (uint64_t)chunk * lv.chunk, lv.chunk);
 }
 
 // Element-major mapping, for small blocks: an op touches block b = (x - dst_place) mod P
@@ -461,10 +482,23 @@ __device__ __forceinline__ void counter_upkeep(const CounterUpkeep &c) {
 // 48 registers the compiler picks unbounded, fp32 the same.
 template <typename T, int OP, int MAXP>
 __global__ void __launch_bounds__(kThreads, 6) step_kernel(const __grid_constant__ StepArgs<MAXP> a) {
+  // bytes read from partners in the low 28 bits (a chunk has less), finished warps above
+  __shared__ uint32_t s_moved;
+  if (threadIdx.x == 0) s_moved = 0;
+  __syncthreads();
   wait_prior_grid();
   if (blockIdx.x == 0) counter_upkeep(a.upkeep);
-  chunk_work<T, OP, MAXP>(a, view_of(a), a.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+  const uint32_t moved = chunk_work<T, OP, MAXP>(a, view_of(a), a.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
   allow_next_grid();
+  if (a.bytes != nullptr) {
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, moved);
+    if ((threadIdx.x & 31) == 0) {
+      const uint32_t before = atomicAdd(&s_moved, (1u << 28) + sum);
+      const uint32_t total = (before & 0xfffffffu) + sum;
+      if (before >> 28 == kThreads / 32 - 1 && total)
+        atomicAdd(a.bytes + blockIdx.x % STEP_BYTE_SLOTS, (unsigned long long)total);
+    }
+  }
 }
 
 template <typename T, int OP, int MAXP>
@@ -551,9 +585,15 @@ __device__ __forceinline__ int ld_relaxed_int(const int *p) {
 // expected, the arrivals of this and every earlier barrier of the launch.  The count
 // only grows within a launch, so no CTA resets it and the last arrival releases everyone
 // at once.  Returns false (for the whole CTA) if this or any other CTA timed out.
-__device__ bool grid_barrier(BarrierState *bar, unsigned expected, unsigned spin_limit, int launch) {
+// The CTA's staged byte counts of the step (bytes: its counters, or nullptr) are added on the
+// way: by a warp beside the one that waits, so they may follow this arrival and precede the
+// next, or, with `first`, before the arrival.
+template <int NT>
+__device__ bool grid_barrier(BarrierState *bar, unsigned expected, unsigned spin_limit, int launch,
+                             unsigned long long *bytes, const uint32_t *s_moved, bool first) {
   __shared__ int s_ok;
   __syncthreads();
+  if (bytes != nullptr && threadIdx.x == (first ? 0 : 32)) add_moved<NT>(bytes, s_moved);
   if (threadIdx.x == 0) {
     int ok = 1;
     const unsigned target = (unsigned)(launch + 1) * expected;
@@ -576,18 +616,18 @@ __device__ bool grid_barrier(BarrierState *bar, unsigned expected, unsigned spin
 }
 
 // Counter row of a communication step: the step's own, but for the first step's, whose
-// counts wait in row nsteps until the second launch moves them (see CounterUpkeep).
+// counts wait in row nsteps until a later launch moves them (see CounterUpkeep).
 __host__ __device__ __forceinline__ unsigned long long *counter_row(unsigned long long *rows, int comm_step,
                                                                     int nsteps) {
   if (rows == nullptr || comm_step < 0) return nullptr;
   return rows + (size_t)(comm_step == 0 ? nsteps : comm_step) * STEP_BYTE_SLOTS;
 }
 __host__ __device__ __forceinline__ CounterUpkeep upkeep_of(unsigned long long *rows, int launch, int next_comm_step,
-                                                            int nsteps) {
+                                                            int nsteps, int move_at = 1) {
   CounterUpkeep c{nullptr, nullptr, nullptr};
   if (rows == nullptr) return c;
   if (next_comm_step > 0) c.zero = rows + (size_t)next_comm_step * STEP_BYTE_SLOTS;
-  if (launch == 1) {
+  if (launch == move_at) {
     c.move_from = rows + (size_t)nsteps * STEP_BYTE_SLOTS;
     c.move_to = rows;
   }
@@ -638,12 +678,16 @@ template <typename T, int OP, int MAXP, bool FLAT>
 __global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, FLAT ? 4 : kPersistPerSM)
     step_kernel_persistent(const __grid_constant__ PersistArgs<MAXP> p) {
   __shared__ void *s_rank[FLAT ? MAXP : 1];
+  __shared__ uint32_t s_moved[kPersistThreads / 32];
   if (FLAT) {
     for (int x = threadIdx.x; x < p.s.P; x += kThreads) s_rank[x] = p.s.rank[x];
     __syncthreads();
   }
   const unsigned expected = gridDim.x + p.phantom;
   bool ok = true;
+  // The first step's counts are added beside barrier 0 and moved behind barrier 1; a launch of
+  // two steps has no barrier 1: there the add comes before the arrival at barrier 0.
+  const int move_at = p.nlaunch > 2 ? 2 : 1;
   PersistStep st = fetch_step<MAXP, FLAT>(p, 0);
   for (int l = 0; l < p.nlaunch && ok; ++l) {
     LaunchView lv;
@@ -658,18 +702,23 @@ __global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, FLAT ? 4 : 
       flat_work<T, OP, MAXP>(p.s, lv, s_rank, (uint64_t)blockIdx.x * kThreads + threadIdx.x,
                              (uint64_t)gridDim.x * kThreads);
     } else {
+      uint32_t moved = 0;
       for (uint32_t item = blockIdx.x; item < st.items; item += gridDim.x) {
         const uint32_t blk = item / st.nchunks, op = blk / (uint32_t)p.s.P;
-        range_work<T, OP, MAXP, kPersistThreads>(p.s, lv, lv.ops[op], (int)(blk - op * (uint32_t)p.s.P),
-                                                 (uint64_t)(item - blk * st.nchunks) * st.chunk, st.chunk);
+        moved += range_work<T, OP, MAXP, kPersistThreads>(p.s, lv, lv.ops[op], (int)(blk - op * (uint32_t)p.s.P),
+                                                          (uint64_t)(item - blk * st.nchunks) * st.chunk, st.chunk);
       }
+      stage_moved<kPersistThreads>(s_moved, moved);
     }
+    unsigned long long *const bytes = FLAT ? nullptr : lv.bytes;  // (flat_work has added its own)
     if (l + 1 < p.nlaunch) {
       st = fetch_step<MAXP, FLAT>(p, l + 1);
-      if (blockIdx.x == 0) counter_upkeep(upkeep_of(p.step_bytes, l, st.d.comm_step, p.nsteps));
-      ok = grid_barrier(p.bar, expected, p.spin_limit, l);
-    } else if (blockIdx.x == 0) {
-      counter_upkeep(upkeep_of(p.step_bytes, l, -1, p.nsteps));
+      if (blockIdx.x == 0) counter_upkeep(upkeep_of(p.step_bytes, l, st.d.comm_step, p.nsteps, move_at));
+      ok = grid_barrier<kPersistThreads>(p.bar, expected, p.spin_limit, l, bytes, s_moved, p.nlaunch == 2);
+    } else {
+      if (blockIdx.x == 0) counter_upkeep(upkeep_of(p.step_bytes, l, -1, p.nsteps, move_at));
+      __syncthreads();
+      if (bytes != nullptr && threadIdx.x == 32) add_moved<kPersistThreads>(bytes, s_moved);
     }
   }
   // The last CTA to leave records the outcome and resets the state for the next launch; a
