@@ -60,6 +60,13 @@ constexpr uint64_t kFlatBelow = 4 * kThreads * kUnroll;  // blocks shorter than 
 // P = 127 x 9 KiB bf16 S = 10: 44.5 us with one op per thread throughout (and the next
 // launch at the end); 33.3 us at 512
 // threads, 36.8 at 256, 35.7 at 1024, 41.8 at 2048 (43.5 with up to 8 ops per thread).
+// No-allocation launches are element-major only for blocks of fewer than 512 elements, or in
+// all fewer than 2^18 elements (ops * n): a longer launch is bound by its 4-byte accesses.
+// GB300, us a call in graph replay, fp32, element-major -> chunked: P = 64 blocks of 1200
+// elements S = 6 165 -> 80, S = 12 57 -> 42, blocks of 800 S = 6 113 -> 76, P = 20 x 2000 S = 5
+// 33 -> 17; but P = 64 x 500 S = 6 75 -> 72, x 160 33 -> 70, P = 5 x 2000 S = 3 5.6 -> 7.3.
+constexpr uint64_t kNoAllocFlatBlock = 512;
+constexpr uint64_t kNoAllocFlatItems = 1u << 18;
 constexpr int kFlatGroup = 4;
 constexpr uint64_t kFlatThreads = 512;
 // Persistent steps: smallest piece of a block.  The chunked steps run in CTAs of 256
@@ -781,10 +788,11 @@ StepArgs<MAXP> step_args(const gar_plan &pl, const Launch &ln, void *const *rank
 
 // Mapping and grid of one launch; *flat: element-major.
 template <int MAXP>
-int step_grid(const gar_plan &pl, const Launch &ln, StepArgs<MAXP> &a, bool *flat, unsigned *grid) {
+int step_grid(const gar_plan &pl, const Launch &ln, bool noalloc, StepArgs<MAXP> &a, bool *flat, unsigned *grid) {
   const uint64_t maxblk = pl.q + (pl.rem ? 1 : 0);
   *grid = 0;
-  *flat = maxblk < kFlatBelow;
+  *flat = maxblk < kFlatBelow &&
+          (!noalloc || maxblk < kNoAllocFlatBlock || (uint64_t)ln.nops * pl.n < kNoAllocFlatItems);
   if (maxblk == 0 || ln.nops == 0) return GAR_OK;
   if (*flat) {
     // blocks shorter than one CTA's worth of vectors: element-major launch
@@ -816,7 +824,7 @@ int launch_typed(const gar_plan &pl, const Launch &ln, int launch_index, void *c
   a.reverse = launch_index & 1;
   bool flat = false;
   unsigned grid = 0;
-  if (int rc = step_grid(pl, ln, a, &flat, &grid)) return rc;
+  if (int rc = step_grid(pl, ln, false, a, &flat, &grid)) return rc;
   if (grid == 0) return GAR_OK;
   const cudaError_t e = flat ? launch_pdl(step_kernel_flat<T, OP, MAXP>, grid, stream, a)
                              : launch_pdl(step_kernel<T, OP, MAXP>, grid, stream, a);
@@ -1009,7 +1017,7 @@ int noalloc_launch(const gar_plan &pl, int launch_index, void *const *rank, void
   a.s.reverse = launch_index & 1;
   bool flat = false;
   unsigned grid = 0;
-  if (int rc = step_grid(pl, ln, a.s, &flat, &grid)) return rc;
+  if (int rc = step_grid(pl, ln, true, a.s, &flat, &grid)) return rc;
   if (grid == 0) return GAR_OK;
   const cudaError_t e = flat ? launch_pdl(step_kernel_noalloc_flat<T, OP>, grid, stream, a)
                              : launch_pdl(step_kernel_noalloc<T, OP>, grid, stream, a);
