@@ -147,8 +147,8 @@ typedef struct {
  * with the contributions in shared memory; a bf16 sum that would take the breadth-first form
  * runs it from 2^19 elements per rank on, an fp32 sum with more than 210 values alive from
  * 2^20 on.  GAR_FORM_COOP: a CTA takes a tile of a few positions and spreads the program over
- * its threads; plans of 16 and more ranks with few element positions (some thousands; the line
- * depends on P and S) run it.  Info and source name these two once the plan is compiled
+ * its threads; plans of 16 and more ranks with few element positions (some thousands; the lines
+ * depend on P, S and group) run it.  Info and source name these two once the plan is compiled
  * (gar_plan_compile, gar_plan_prepare or a first fused call), and one of the first two before
  * that.  All forms give the same bits. */
 enum { GAR_FORM_SINGLE = 0, GAR_FORM_BREADTH = 1, GAR_FORM_SPLIT = 2, GAR_FORM_STREAM = 3, GAR_FORM_COOP = 4 };

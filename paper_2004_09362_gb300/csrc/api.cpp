@@ -185,7 +185,11 @@ bool takes_stream(const gar_plan &pl) {
 // Whether a plan runs the cooperative form.  GB300, us per fused call in graph
 // replay, the other form -> cooperative (bf16; fp32 within a few per cent):
 //  * P below 16 gains little or loses (P = 12, S = 8 2.3 -> 1.7, S = 5 1.7 -> 1.7; P = 6
-//    1.3 -> 1.5), and so do the many levels of the Ring and of most folds (P = 48 2.5 -> 4.3).
+//    1.3 -> 1.5), and so do the many levels of the Ring and of most folds (P = 48 2.5 -> 4.3),
+//    fewer than 20 ranks with several copies (fp32, 60, 1000 and 4864 positions: P = 17, S = 6
+//    1.3 -> 1.6, 1.6 -> 1.7, 1.5 -> 1.8; P = 19, S = 7 1.3 -> 1.6, 1.8 -> 1.7, 1.6 -> 1.5; P = 20,
+//    S = 7 1.4 -> 1.6, 2.7 -> 1.7, 2.2 -> 1.7) and the XOR group below 32 (P = 16, S = 7 1.4,
+//    1.6 -> 1.6, 1.5 -> 1.6; P = 32, S = 7 1.8 -> 1.5, 2.9 -> 1.7, 2.4 -> 1.7).
 //  * One result copy: up to a tile of 32 positions per SM (152 SMs; P = 48, S = 12, 2500
 //    positions 2.4 -> 2.0, 10000 2.4 -> 3.3; P = 127, S = 14, 212 6.5 -> 1.9, 2500 5.4 -> 3.1,
 //    5000 4.5 -> 3.7, 10000 4.5 -> 5.6), two tiles up to P = 32 (P = 24, S = 10, 10000
@@ -204,7 +208,8 @@ bool takes_coop(const gar_plan &pl) {
   const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
   if ((ff && *ff) || older_form_tuned()) return false;
   const uint64_t wave = 32 * (uint64_t)pl.sms;
-  if (pl.P < 16 || pl.n > 2 * wave || !coop_form_applies(pl) || fused_levels(pl) > 10) return false;
+  const int least = pl.group == GAR_GROUP_XOR ? 32 : pl.K > 1 ? 20 : 16;
+  if (pl.P < least || pl.n > 2 * wave || !coop_form_applies(pl) || fused_levels(pl) > 10) return false;
   if (pl.K == 1) return pl.n <= (pl.P <= 32 ? 2 * wave : wave);
   const uint64_t work = pl.n * (2 * (uint64_t)pl.P + pl.prog.a.size());
   const uint64_t most = fused_peak_live(pl) > 160 ? 1200000 : pl.P < 48 ? 700000 : 2750000;

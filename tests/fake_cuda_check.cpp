@@ -201,12 +201,31 @@ void sm_count() {
     }
 }
 
+// The ranks from which short vectors take the cooperative form.
+void cooperative_ranks() {
+  struct { int P, steps, group, form; } cases[] = {
+      {15, 8, GAR_GROUP_CYCLIC, GAR_FORM_SINGLE}, {16, 8, GAR_GROUP_CYCLIC, GAR_FORM_COOP},
+      {16, 7, GAR_GROUP_CYCLIC, GAR_FORM_SINGLE}, {19, 8, GAR_GROUP_CYCLIC, GAR_FORM_SINGLE},
+      {19, 10, GAR_GROUP_CYCLIC, GAR_FORM_COOP},  {20, 8, GAR_GROUP_CYCLIC, GAR_FORM_COOP},
+      {20, 5, GAR_GROUP_CYCLIC, GAR_FORM_SINGLE}, {16, 8, GAR_GROUP_XOR, GAR_FORM_SINGLE},
+      {32, 7, GAR_GROUP_XOR, GAR_FORM_COOP},      {32, 10, GAR_GROUP_XOR, GAR_FORM_COOP}};
+  for (const auto &c : cases) {
+    gar_plan *pl = nullptr;
+    CHECK(gar_plan_create_group(&pl, c.P, 100, GAR_F32, GAR_SUM, c.steps, c.group) == GAR_OK);
+    CHECK(gar_plan_compile(pl, GAR_FUSED) == GAR_OK);
+    if (form_of(pl) != c.form) std::printf("P = %d, S = %d, group %d\n", c.P, c.steps, c.group);
+    CHECK(form_of(pl) == c.form);
+    gar_plan_destroy(pl);
+  }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups},
       {"batched_threads", batched_threads}, {"knobs", knobs},
-      {"compiled_ahead", compiled_ahead}, {"sm_count", sm_count}};
+      {"compiled_ahead", compiled_ahead}, {"sm_count", sm_count},
+      {"cooperative_ranks", cooperative_ranks}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

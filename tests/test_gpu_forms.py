@@ -60,7 +60,8 @@ def test_single_thread_form_every_step_count(P, monkeypatch):
                 plan = gar.gar_plan_create(P, n, dtype, "sum", S)
                 gar.gar_plan_prepare(plan, "fused")
                 info = gar.gar_plan_get_info(plan)
-                assert info["fused_form"] == (gar.GAR_FORM_COOP if info["K"] < P else gar.GAR_FORM_SINGLE)
+                coop = info["K"] == 1 or (P >= 20 and info["K"] < P)
+                assert info["fused_form"] == (gar.GAR_FORM_COOP if coop else gar.GAR_FORM_SINGLE)
 
 
 @pytest.mark.gpu

@@ -79,3 +79,7 @@ def test_a_plan_compiled_ahead_prepares_the_same_kernel(program):
 
 def test_the_cooperative_form_follows_the_sm_count(program):
     _run(program, "sm_count")
+
+
+def test_ranks_from_which_short_vectors_take_the_cooperative_form(program):
+    _run(program, "cooperative_ranks")
