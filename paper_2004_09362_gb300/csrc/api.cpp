@@ -286,24 +286,15 @@ int refine_stream(gar_plan *pl) {
 // P = 64 x 16 MiB bf16 S = 8 (96 B: 0.324 against 0.346), P = 127 S = 9 (48 B: 0.407
 // against 0.460).
 // The counts are the loaded kernel's own (the compiler's log does not always carry them).
-int build_fused(gar_plan *pl) {
-  // a kernel compiled ahead was chosen for the default SM count
-  const int assumed = pl->sms;
-  int rc = check_fused_size(pl);
-  if (rc) return rc;
-  if ((rc = ensure_device(pl))) return rc;
-  if (pl->sms != assumed) pl->fused = nullptr;
-  if ((rc = compile_fused(pl))) return rc;
-  if ((rc = jit_load(pl->fused, &pl->fused_on))) return rc;
-  if (pl->fused->form == GAR_FORM_STREAM && takes_stream(*pl)) return refine_stream(pl);
+int refine_single(const gar_plan &pl, bool host, JitKernel **kernel, JitOnDevice *on) {
   const bool shape_forced = std::getenv("GAR_TUNE_FUSED_THREADS") || std::getenv("GAR_TUNE_FUSED_MINB");
-  if (pl->fused->form != 0 || pl->fused->threads != 256 || shape_forced || pl->fused->regs <= 128)
-    return GAR_OK;
+  if ((*kernel)->form != 0 || (*kernel)->threads != 256 || shape_forced || (*kernel)->regs <= 128) return GAR_OK;
   auto build = [&](int threads, int minb, int fadd2, JitKernel **out) -> int {
-    if (int r = compile_source([&] { return generate_fused_source(*pl, threads, minb, fadd2); }, out)) return r;
+    if (int r = compile_source([&] { return generate_fused_source(pl, threads, minb, fadd2, host); }, out)) return r;
     return jit_load(*out);
   };
   JitKernel *k = nullptr;
+  int rc = GAR_OK;
   if ((rc = build(64, 5, -1, &k))) return rc;
   if (k->local_bytes > 256) {
     JitKernel *wide = nullptr;
@@ -315,15 +306,29 @@ int build_fused(gar_plan *pl) {
   // then the pairs halve the adds at no cost in warps (P = 127 x 8 MiB S = 9: 0.405 ->
   // 0.372 ms).  Elsewhere they cost registers: P = 100 S = 9 (128 -> 140 registers) 0.272
   // -> 0.280 ms, P = 64 latency-optimal (39 -> 255) 0.339 -> 0.493 ms.
-  if (pl->dtype == GAR_BF16 && k->width == 2 && k->local_bytes > 0 && k->regs >= 168 &&
+  if (pl.dtype == GAR_BF16 && k->width == 2 && k->local_bytes > 0 && k->regs >= 168 &&
       !std::getenv("GAR_TUNE_FADD2")) {
     JitKernel *paired = nullptr;
     if ((rc = build(k->threads, k->threads == 64 ? 5 : 8, 1, &paired))) return rc;
     if (paired->local_bytes <= k->local_bytes) k = paired;
   }
-  if ((rc = jit_load(k, &pl->fused_on))) return rc;
-  pl->fused = k;
-  pl->fused_width = k->width;
+  if ((rc = jit_load(k, on))) return rc;
+  *kernel = k;
+  return GAR_OK;
+}
+
+int build_fused(gar_plan *pl) {
+  // a kernel compiled ahead was chosen for the default SM count
+  const int assumed = pl->sms;
+  int rc = check_fused_size(pl);
+  if (rc) return rc;
+  if ((rc = ensure_device(pl))) return rc;
+  if (pl->sms != assumed) pl->fused = nullptr;
+  if ((rc = compile_fused(pl))) return rc;
+  if ((rc = jit_load(pl->fused, &pl->fused_on))) return rc;
+  if (pl->fused->form == GAR_FORM_STREAM && takes_stream(*pl)) return refine_stream(pl);
+  if ((rc = refine_single(*pl, false, &pl->fused, &pl->fused_on))) return rc;
+  pl->fused_width = pl->fused->width;
   return GAR_OK;
 }
 
@@ -333,6 +338,38 @@ int prepare_fused(gar_plan *pl) {
   if (int rc = build_fused(pl)) return rc;
   if (pl->fused_on.gave_up != nullptr) pl->wait_slot = jit_take_slot(pl->fused, pl->device, &pl->waits_seen);
   pl->fused_ready = true;
+  return GAR_OK;
+}
+
+// The kernel for vectors in host memory: the plan's, or one of its own where another width
+// suits them, which the first such call builds (in the other's place, if the plan has run on
+// host memory only).  A call that is being captured has to do with what there is.
+int prepare_fused_host(gar_plan *pl, gar_stream_t stream) {
+  if (pl->fused_host != nullptr) return ensure_device(pl);
+  if (pl->host_shares_fused) return prepare_fused(pl);
+  if (int rc = check_fused_size(pl)) return rc;
+  if (int rc = ensure_device(pl)) return rc;
+  CodegenResult cg;
+  try {
+    if (chosen_form(*pl) == GAR_FORM_SINGLE) cg = generate_fused_source(*pl);
+  } catch (const std::exception &ex) {
+    set_error(std::string("fused code generation: ") + ex.what());
+    return GAR_EINVAL;
+  }
+  pl->host_shares_fused = cg.host_width <= cg.width;
+  if (pl->host_shares_fused) return prepare_fused(pl);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing((cudaStream_t)stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return prepare_fused(pl);
+  }
+  JitKernel *k = nullptr;
+  JitOnDevice on;
+  if (int rc = compile_source([&] { return generate_fused_source(*pl, 0, 0, -1, true); }, &k)) return rc;
+  if (int rc = jit_load(k, &on)) return rc;
+  if (int rc = refine_single(*pl, true, &k, &on)) return rc;
+  pl->fused_host = k;
+  pl->fused_host_on = on;
   return GAR_OK;
 }
 
@@ -392,8 +429,7 @@ int grid_for(const JitKernel *k, const JitOnDevice &on, uint64_t work_items) {
 // (327 GB/s), 24 x 1 MiB 238 -> 180, P = 5 x 8 MiB bf16 348 -> 262, P = 64 x 1 MiB fp32
 // latency-optimal 637 -> 480, P = 127 x 1 MiB bf16 1186 -> 860; half or twice the 3 MB cost
 // up to 10 %.
-int host_grid(const gar_plan &pl) {
-  const JitKernel *k = pl.fused;
+int host_grid(const gar_plan &pl, const JitKernel *k) {
   uint64_t per_thread = (uint64_t)pl.P * (uint64_t)k->width * (uint64_t)elem_size(pl.dtype);
   if (k->regs > 0) per_thread = std::min<uint64_t>(per_thread, 4 * (uint64_t)k->regs);
   const uint64_t per_cta = k->form == GAR_FORM_STREAM ? (uint64_t)k->smem
@@ -428,8 +464,11 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
   if (e_hi <= e_lo) return GAR_OK;
   // gar_args: the in[] table, then the out[] table, each table_copies times in a row,
   // then e_lo, e_hi and, in the streaming form, the wait slot
+  const bool other = host_memory && pl->fused_host != nullptr;
+  const JitKernel *k = other ? pl->fused_host : pl->fused;
+  const JitOnDevice &on = other ? pl->fused_host_on : pl->fused_on;
   const size_t pb = 8 * (size_t)pl->P;
-  const int copies = pl->fused->table_copies;
+  const int copies = k->table_copies;
   unsigned char args[4 * 8 * GAR_MAX_P + 24];
   unsigned char *w = args;
   for (int c = 0; c < copies; ++c, w += pb) std::memcpy(w, in, pb);
@@ -441,17 +480,16 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
   void *kargs[] = {args};
   // threads: one per vector of `width` positions, or two per position in groups of 16
   // (two-lane form)
-  const uint64_t items = pl->fused->form == GAR_FORM_SPLIT ? (e_hi - e_lo + 15) / 16 * 32
-                                                           : (e_hi - e_lo) / pl->fused->width + 1;
-  int grid = grid_for(pl->fused, pl->fused_on, items);
-  if (pl->fused->tile > 0) {  // persistent: as many CTAs as the device holds at once
-    const uint64_t tiles = std::max<uint64_t>(1, (e_hi - e_lo + pl->fused->tile - 1) / pl->fused->tile);
-    grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms() * (uint64_t)pl->fused_on.blocks_per_sm);
+  const uint64_t items = k->form == GAR_FORM_SPLIT ? (e_hi - e_lo + 15) / 16 * 32 : (e_hi - e_lo) / k->width + 1;
+  int grid = grid_for(k, on, items);
+  if (k->tile > 0) {  // persistent: as many CTAs as the device holds at once
+    const uint64_t tiles = std::max<uint64_t>(1, (e_hi - e_lo + k->tile - 1) / k->tile);
+    grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms() * (uint64_t)on.blocks_per_sm);
   }
-  if (host_memory) grid = std::min(grid, host_grid(*pl));
-  cudaError_t e = launch_generated(pl->fused, grid, kargs, stream);
+  if (host_memory) grid = std::min(grid, host_grid(*pl, k));
+  cudaError_t e = launch_generated(k, grid, kargs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
-  if (pl->fused_on.gave_up != nullptr) {
+  if (on.gave_up != nullptr) {
     pl->fused_stream = stream;
     pl->ran_waiting = true;
   }
@@ -878,7 +916,7 @@ int gar_allreduce_host(gar_plan *pl, const void *const *host_in, void *const *ho
     if (aligned && device_accessible_host(host_in, pl->P) &&
         device_accessible_host(reinterpret_cast<const void *const *>(host_out), pl->P)) {
       // The kernel reads the inputs from and writes the results to host memory itself.
-      int rc = prepare_fused(pl);
+      int rc = prepare_fused_host(pl, stream);
       if (rc) return rc;
       return launch_fused_range(pl, host_in, host_out, 0, pl->n, stream, true);
     }

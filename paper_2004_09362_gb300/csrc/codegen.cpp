@@ -341,7 +341,8 @@ std::string emit_block_of(const std::string &name, int P, uint64_t n) {
 
 }  // namespace
 
-CodegenResult generate_fused_source(const gar_plan &pl, int threads_override, int minb_override, int fadd2_override) {
+CodegenResult generate_fused_source(const gar_plan &pl, int threads_override, int minb_override, int fadd2_override,
+                                    bool host) {
   const FusedProgram &fp = pl.prog;
   const int P = pl.P;
   Schedule sc = order_program(fp);
@@ -373,14 +374,16 @@ CodegenResult generate_fused_source(const gar_plan &pl, int threads_override, in
   // positions (2^17 below 8 ranks).  GB300, us in graph replay, W by the line above -> W = 1:
   // P = 24 S = 10 fp32, 33000 positions 4.9 -> 2.3, 100000 6.7 -> 3.1, 260000 8.8 -> 6.2; P = 48
   // S = 9 64000 11.0 -> 4.4, 520000 25.6 -> 26.8; P = 12 S = 8 260000 5.3 -> 3.6; P = 5 260000
-  // 2.0 -> 2.1; from and to pinned host memory P = 24, 33000 37 -> 38, 100000 84 -> 77.  bf16
-  // gains as much on the GPU (P = 127 S = 14 33000 9.4 -> 5.3), but its 2-byte accesses cost
-  // more over NVLink-C2C (P = 8, 250000 38 -> 49), and whole vectors only gain from W (P = 64
-  // S = 12 bf16 160000 9.0 at W = 1, 5.3 at 4).
+  // 2.0 -> 2.1.  Not over NVLink-C2C (`host`), which narrow accesses cost more: P = 8 S = 6
+  // 260000 positions 64 -> 76, P = 10 S = 5 90000 34 -> 39, P = 24 S = 6 200000 149 -> 166
+  // (P = 24 S = 6 131000 101 -> 89, 33000 36 -> 33).  bf16 gains as much on the GPU (P = 127
+  // S = 14 33000 9.4 -> 5.3), and whole vectors only gain from W (P = 64 S = 12 bf16 160000
+  // 9.0 at W = 1, 5.3 at 4).
   const bool cut = rotate && (pl.n % (uint64_t)P != 0 || pl.n / (uint64_t)P % (uint64_t)W != 0);
-  if (cut && elem_size(pl.dtype) == 4 && pl.n < (P < 8 ? 1u << 17 : 1u << 18)) W = 1;
+  int host_width = W;
+  if (!host && cut && elem_size(pl.dtype) == 4 && pl.n < (P < 8 ? 1u << 17 : 1u << 18)) W = 1;
   if (int w = tune_int("GAR_TUNE_FUSED_W", 0))
-    if (w > 0 && (w & (w - 1)) == 0 && w * elem_size(pl.dtype) <= 16) W = w;
+    if (w > 0 && (w & (w - 1)) == 0 && w * elem_size(pl.dtype) <= 16) W = host_width = w;
   const int minb = minb_override > 0 ? minb_override : tune_int("GAR_TUNE_FUSED_MINB", small_cta ? 16 : 0);
   int nthr = threads_override > 0 ? threads_override : tune_int("GAR_TUNE_FUSED_THREADS", small_cta ? 32 : 256);
   if (nthr < 32 || nthr > 1024 || nthr % 32 != 0) nthr = 256;
@@ -388,6 +391,7 @@ CodegenResult generate_fused_source(const gar_plan &pl, int threads_override, in
                                       : fmt("__launch_bounds__(%d)", nthr);
   CodegenResult cg;
   cg.width = W;
+  cg.host_width = host_width;
   cg.threads = nthr;
   cg.kernel_name = fmt("gar_fused_P%d_S%d_K%d_", P, pl.S, pl.K) + dtype_tag(pl.dtype) + "_" +
                    op_tag(pl.op) + fmt("_W%d", W) + (pl.group == GAR_GROUP_XOR ? "_xor" : "");

@@ -127,6 +127,9 @@ struct gar_plan {
   bool ran_step_faithful = false;
   gar::JitKernel *fused = nullptr;   // owned by the JIT cache
   gar::JitOnDevice fused_on;         // the loaded kernel on the plan's device
+  gar::JitKernel *fused_host = nullptr;  // for host memory, where it is another kernel (same form)
+  gar::JitOnDevice fused_host_on;
+  bool host_shares_fused = false;        // decided: `fused` serves host memory too
   gar_stream_t fused_stream = nullptr;  // of the last launch of a kernel with bounded waits
   bool ran_waiting = false;             // such a launch was made
   int wait_slot = -1;                   // its counter, and the count that is known
@@ -165,14 +168,17 @@ struct CodegenResult {
   std::string source;
   std::string kernel_name;
   int width = 1;
+  int host_width = 0;    // single-thread form: width that suits host memory
   int table_copies = 1;  // fused kernels: copies of the in[] / out[] pointer tables (1 or 2)
   int threads = 256;     // threads per CTA
   int form = 0;          // fused kernels: GAR_FORM_*
   int smem = 0;          // dynamic shared memory per CTA
   int tile = 0;          // element positions per tile of a persistent kernel (0: one vector per thread)
 };
-// threads / minb > 0 override the CTA size and the minimum resident CTAs per SM
-CodegenResult generate_fused_source(const gar_plan &pl, int threads = 0, int minb = 0, int fadd2 = -1);
+// threads / minb > 0 override the CTA size and the minimum resident CTAs per SM; host: for
+// vectors in host memory
+CodegenResult generate_fused_source(const gar_plan &pl, int threads = 0, int minb = 0, int fadd2 = -1,
+                                    bool host = false);
 // The breadth-first form of the fused kernel (programs with many result copies), and
 // the peak number of live values of a plan's program in the single-thread form.
 CodegenResult generate_fused_bf_source(const gar_plan &pl);
@@ -197,6 +203,7 @@ struct JitKernel {
   std::string source;        // the generated CUDA source it was compiled from
   std::string name;
   int width = 1;
+  int host_width = 0;
   int table_copies = 1;
   int threads = 256;
   int form = 0;

@@ -62,6 +62,7 @@ int jit_compile(const CodegenResult &cg, JitKernel **out) {
   k->name = cg.kernel_name;
   k->source = cg.source;
   k->width = cg.width;
+  k->host_width = cg.host_width;
   k->table_copies = cg.table_copies;
   k->threads = cg.threads;
   k->form = cg.form;

@@ -52,6 +52,8 @@ inline int compiles = 0;
 inline std::vector<Launch> launches;
 inline std::function<cudaError_t(Function &, const Launch &)> on_launch;
 inline std::function<cudaError_t(cudaStream_t)> on_synchronize;
+inline cudaMemoryType memory = cudaMemoryTypeDevice;
+inline std::string last_source;
 inline cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
 
 }  // namespace fake
@@ -100,9 +102,10 @@ cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cu
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = (cudaEvent_t)std::malloc(1), cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { return std::free((void *)e), cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *) {
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) {
   *a = cudaPointerAttributes{};
-  a->type = cudaMemoryTypeDevice;
+  a->type = fake::memory;
+  a->devicePointer = const_cast<void *>(p);
   return cudaSuccess;
 }
 

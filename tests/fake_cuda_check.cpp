@@ -219,13 +219,58 @@ void cooperative_ranks() {
   }
 }
 
+// A plan whose vectors are cut by block boundaries runs wider vectors on host memory than on
+// the device, from a kernel that the first host call builds; other plans share one kernel.
+void host_width() {
+  struct { int P; uint64_t n; int dtype, steps; bool apart; } cases[] = {
+      {8, 200003, GAR_F32, 6, true}, {8, 200003, GAR_BF16, 6, false}, {8, 1u << 20, GAR_F32, 6, false},
+      {8, 8 * 4096, GAR_F32, 6, false}, {24, 100, GAR_F32, 10, false}, {6, 79063, GAR_I32, 5, true}};
+  for (const auto &c : cases)
+    for (bool device_first : {false, true}) {
+      const std::vector<void *> r = rows(c.P);
+      const std::vector<const void *> in(r.begin(), r.end());
+      gar_plan *pl = plan_of(c.P, c.n, c.dtype, c.steps);
+      auto run = [&](bool host) {
+        fake::memory = host ? cudaMemoryTypeHost : cudaMemoryTypeDevice;
+        fake::launches.clear();
+        fake::on_launch = [](fake::Function &f, const fake::Launch &) {
+          fake::last_source = f.source;
+          return cudaSuccess;
+        };
+        CHECK((host ? gar_allreduce_host(pl, in.data(), r.data(), r.data(), GAR_FUSED, nullptr)
+                    : gar_allreduce(pl, r.data(), GAR_FUSED, nullptr)) == GAR_OK);
+        CHECK(fake::launches.size() == 1);
+        return fake::last_source;
+      };
+      const int before = fake::compiles;
+      std::string source[2];
+      for (int k = 0; k < 2; ++k) {
+        const bool host = device_first ? k == 1 : k == 0;
+        if (host && c.apart && device_first) {        // captured before the kernel is there
+          fake::capture = cudaStreamCaptureStatusActive;
+          CHECK(run(true) == source[0] && fake::compiles == before + (device_first ? 0 : 1));
+          fake::capture = cudaStreamCaptureStatusNone;
+        }
+        source[host] = run(host);
+        CHECK(run(host) == source[host]);
+      }
+      CHECK((source[0] != source[1]) == c.apart);
+      if (!device_first) CHECK(fake::compiles == before + (c.apart ? 2 : 1));
+      if (c.apart) {
+        CHECK(source[0].find("#define GAR_W 1\n") != std::string::npos);
+        CHECK(source[1].find("#define GAR_W 4\n") != std::string::npos);
+      }
+      gar_plan_destroy(pl);
+    }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups},
       {"batched_threads", batched_threads}, {"knobs", knobs},
       {"compiled_ahead", compiled_ahead}, {"sm_count", sm_count},
-      {"cooperative_ranks", cooperative_ranks}};
+      {"cooperative_ranks", cooperative_ranks}, {"host_width", host_width}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

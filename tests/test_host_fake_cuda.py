@@ -83,3 +83,7 @@ def test_the_cooperative_form_follows_the_sm_count(program):
 
 def test_ranks_from_which_short_vectors_take_the_cooperative_form(program):
     _run(program, "cooperative_ranks")
+
+
+def test_host_memory_has_its_own_width(program):
+    _run(program, "host_width")
