@@ -420,7 +420,7 @@ int grid_for(const JitKernel *k, const JitOnDevice &on, uint64_t work_items) {
   return (int)std::max<uint64_t>(1, std::min<uint64_t>(need, cap));
 }
 
-// Most CTAs of a fused kernel that works on host memory over NVLink-C2C.  The link needs
+// CTAs of a fused kernel that works on host memory over NVLink-C2C, of `grid` on the device.  The link needs
 // about 3 MB of loads in flight; with a thread for every vector (tens of MB in flight) all
 // reads were queued first and the writes came after them, so the two directions of the
 // link hardly overlapped.  A thread has at most its P vectors in flight, and at most what
@@ -428,14 +428,17 @@ int grid_for(const JitKernel *k, const JitOnDevice &on, uint64_t work_items) {
 // rule: P = 24 x 4 MiB fp32 871 -> 645 us (231 -> 312 GB/s), 24 x 16 MiB 2960 -> 2460
 // (327 GB/s), 24 x 1 MiB 238 -> 180, P = 5 x 8 MiB bf16 348 -> 262, P = 64 x 1 MiB fp32
 // latency-optimal 637 -> 480, P = 127 x 1 MiB bf16 1186 -> 860; half or twice the 3 MB cost
-// up to 10 %.
-int host_grid(const gar_plan &pl, const JitKernel *k) {
+// up to 10 %.  The work is shared out evenly over as many rounds as come nearest to that: with
+// a few CTAs left for a second round, P = 9 x 89000 fp32 S = 4 took 30.7 us instead of 28.3.
+int host_grid(const gar_plan &pl, const JitKernel *k, int grid) {
   uint64_t per_thread = (uint64_t)pl.P * (uint64_t)k->width * (uint64_t)elem_size(pl.dtype);
   if (k->regs > 0) per_thread = std::min<uint64_t>(per_thread, 4 * (uint64_t)k->regs);
   const uint64_t per_cta = k->form == GAR_FORM_STREAM ? (uint64_t)k->smem
                            : k->form == GAR_FORM_COOP ? (uint64_t)pl.P * (uint64_t)k->tile * (uint64_t)elem_size(pl.dtype)
                                                       : per_thread * (uint64_t)k->threads;
-  return (int)std::max<uint64_t>(1, (3000000 + per_cta - 1) / per_cta);
+  const uint64_t most = std::max<uint64_t>(1, (3000000 + per_cta - 1) / per_cta);
+  const uint64_t rounds = std::max<uint64_t>(1, ((uint64_t)grid + most / 2) / most);
+  return (int)(((uint64_t)grid + rounds - 1) / rounds);
 }
 
 // Launches a generated kernel with programmatic stream serialisation: back-to-back
@@ -486,7 +489,7 @@ int launch_fused_range(gar_plan *pl, const void *const *in, void *const *out, ui
     const uint64_t tiles = std::max<uint64_t>(1, (e_hi - e_lo + k->tile - 1) / k->tile);
     grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms() * (uint64_t)on.blocks_per_sm);
   }
-  if (host_memory) grid = std::min(grid, host_grid(*pl, k));
+  if (host_memory) grid = host_grid(*pl, k, grid);
   cudaError_t e = launch_generated(k, grid, kargs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
   if (on.gave_up != nullptr) {

@@ -264,13 +264,33 @@ void host_width() {
     }
 }
 
+// A fused call on host memory shares its CTAs out over whole rounds of about 3 MB of loads.
+void host_grid() {
+  fake::memory = cudaMemoryTypeHost;
+  struct { uint64_t n; unsigned grid; } cases[] = {
+      {8 * 40000, 313}, {8 * 46000, 360}, {8 * 56000, 438}, {8 * 140000, 365}, {8 * 1000000, 373}};
+  const int P = 8;                                   // 8192 bytes of loads a CTA: 367 for 3 MB
+  const std::vector<void *> r = rows(P);
+  const std::vector<const void *> in(r.begin(), r.end());
+  fake::regs = 8;                                    // 32 bytes a thread
+  for (const auto &c : cases) {
+    gar_plan *pl = plan_of(P, c.n, GAR_F32, 6);
+    fake::launches.clear();
+    CHECK(gar_allreduce_host(pl, in.data(), r.data(), r.data(), GAR_FUSED, nullptr) == GAR_OK);
+    if (fake::launches[0].grid != c.grid) std::printf("%llu positions: %u CTAs\n", (unsigned long long)c.n, fake::launches[0].grid);
+    CHECK(fake::launches[0].grid == c.grid);
+    gar_plan_destroy(pl);
+  }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
   const std::map<std::string, void (*)()> checks = {{"two_devices", two_devices}, {"wait_status", wait_status}, {"stream_groups", stream_groups},
       {"batched_threads", batched_threads}, {"knobs", knobs},
       {"compiled_ahead", compiled_ahead}, {"sm_count", sm_count},
-      {"cooperative_ranks", cooperative_ranks}, {"host_width", host_width}};
+      {"cooperative_ranks", cooperative_ranks}, {"host_width", host_width},
+      {"host_grid", host_grid}};
   CHECK(argc == 2 && checks.count(argv[1]));
   checks.at(argv[1])();
   return 0;

@@ -87,3 +87,7 @@ def test_ranks_from_which_short_vectors_take_the_cooperative_form(program):
 
 def test_host_memory_has_its_own_width(program):
     _run(program, "host_width")
+
+
+def test_host_memory_calls_run_in_whole_rounds(program):
+    _run(program, "host_grid")
