@@ -69,13 +69,14 @@ constexpr uint64_t kNoAllocFlatBlock = 512;
 constexpr uint64_t kNoAllocFlatItems = 1u << 18;
 constexpr int kFlatGroup = 4;
 constexpr uint64_t kFlatThreads = 512;
-// Persistent steps: smallest piece of a block.  The chunked steps run in CTAs of 256
-// threads, 2 per SM without spills: P = 24 x 4 MiB int32 max S = 10 87.6 us call after call
-// (98 on vectors that L2 does not hold; 92.8 with 3 per SM, 98.9 with 4, 95.6 in 512-thread
-// CTAs that spilled; 119 cut as the largest step), P = 24 x 240 KB fp32 S = 10 33.0 (37.1,
-// 48.7, 45.3; 40.5), P = 18 x 460 KB int32 S = 6 38.8 (33.4, 41.1, 44.1; 40.0).
+// Persistent steps: smallest piece of a block.  The chunked steps run in CTAs of 256 threads, 2
+// per SM, or 3 where the largest step has more blocks (P * ops) than the CTAs at 2 per SM, of
+// bf16 plans twice as many: a CTA then works through several pieces, and more warps hide
+// their loads.  GB300, us call after call, 2 per SM -> 3 (4): P = 24 x 4 MiB int32 max S = 10
+// (288 blocks) 98 -> 102 (96), P = 12 x 160000 int32 S = 8 31 -> 35 (40), P = 18 x 90000 fp32
+// S = 10 38 -> 42 (48); P = 18 x 1.8M fp32 S = 5 427 -> 342 (353), P = 64 x 851000 int32 S = 6
+// 697 -> 588 (549), P = 18 x 239000 bf16 S = 5 71 -> 62 (74), x 90000 bf16 S = 7 37 -> 40 (43).
 constexpr int kPersistThreads = 256;
-constexpr int kPersistPerSM = 2;
 constexpr uint64_t kMinPiece = 2048;
 
 // Counter upkeep of one launch, by its first CTA (after wait_prior_grid): zeroes the
@@ -680,9 +681,10 @@ __device__ __forceinline__ PersistStep fetch_step(const PersistArgs<MAXP> &p, in
   return s;
 }
 
-// FLAT: element-major mapping (small blocks), else pieces of blocks.
-template <typename T, int OP, int MAXP, bool FLAT>
-__global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, FLAT ? 4 : kPersistPerSM)
+// FLAT: element-major mapping (small blocks), else pieces of blocks.  PER_SM: CTAs per SM that
+// its registers allow for.
+template <typename T, int OP, int MAXP, bool FLAT, int PER_SM>
+__global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, PER_SM)
     step_kernel_persistent(const __grid_constant__ PersistArgs<MAXP> p) {
   __shared__ void *s_rank[FLAT ? MAXP : 1];
   __shared__ uint32_t s_moved[kPersistThreads / 32];
@@ -874,8 +876,12 @@ int launch_persistent_typed(const gar_plan &pl, void *const *rank, gar_stream_t 
     need = std::max<uint64_t>(need, flat ? ((uint64_t)((ln.nops + group - 1) / group) * pl.n + kThreads - 1) / kThreads
                                          : (uint64_t)ln.nops * pl.P * ((maxblk + kMinPiece - 1) / kMinPiece));
   }
-  const void *fn = flat ? (const void *)step_kernel_persistent<T, OP, MAXP, true>
-                        : (const void *)step_kernel_persistent<T, OP, MAXP, false>;
+  int most_ops = 0;
+  for (const Launch &ln : pl.launches) most_ops = std::max(most_ops, ln.nops);
+  const bool many = (uint64_t)most_ops * (uint64_t)pl.P > (sizeof(T) == 2 ? 4u : 2u) * (uint64_t)num_sms();
+  const void *fn = flat   ? (const void *)step_kernel_persistent<T, OP, MAXP, true, 4>
+                   : many ? (const void *)step_kernel_persistent<T, OP, MAXP, false, 3>
+                          : (const void *)step_kernel_persistent<T, OP, MAXP, false, 2>;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, flat ? kThreads : kPersistThreads, 0);
   if (e != cudaSuccess || per_sm < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
