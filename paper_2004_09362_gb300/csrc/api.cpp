@@ -342,10 +342,12 @@ int prepare_fused(gar_plan *pl) {
 }
 
 // The kernel for vectors in host memory: the plan's, or one of its own where another width
-// suits them, which the first such call builds (in the other's place, if the plan has run on
-// host memory only).  A call that is being captured has to do with what there is.
+// suits them, built by gar_plan_prepare or else by the first such call (in the other's place,
+// if the plan has run on host memory only).  A call that is being captured has to do with what
+// there is.
 int prepare_fused_host(gar_plan *pl, gar_stream_t stream) {
   if (pl->fused_host != nullptr) return ensure_device(pl);
+  if (pl->fused_ready && pl->fused->host_width <= pl->fused->width) pl->host_shares_fused = true;
   if (pl->host_shares_fused) return prepare_fused(pl);
   if (int rc = check_fused_size(pl)) return rc;
   if (int rc = ensure_device(pl)) return rc;
@@ -428,8 +430,10 @@ int grid_for(const JitKernel *k, const JitOnDevice &on, uint64_t work_items) {
 // rule: P = 24 x 4 MiB fp32 871 -> 645 us (231 -> 312 GB/s), 24 x 16 MiB 2960 -> 2460
 // (327 GB/s), 24 x 1 MiB 238 -> 180, P = 5 x 8 MiB bf16 348 -> 262, P = 64 x 1 MiB fp32
 // latency-optimal 637 -> 480, P = 127 x 1 MiB bf16 1186 -> 860; half or twice the 3 MB cost
-// up to 10 %.  The work is shared out evenly over as many rounds as come nearest to that: with
-// a few CTAs left for a second round, P = 9 x 89000 fp32 S = 4 took 30.7 us instead of 28.3.
+// up to 10 %.  Up to 3.75 MB go in one round (with a few CTAs left for a second one P = 9 x
+// 89000 fp32 S = 4 took 30.7 us instead of 28.3; but 4.2 MB in one round, P = 5 x 210000 fp32
+// S = 3, 39.8 instead of 36.6), and more is shared out evenly over as many rounds as come
+// nearest to 3 MB.
 int host_grid(const gar_plan &pl, const JitKernel *k, int grid) {
   uint64_t per_thread = (uint64_t)pl.P * (uint64_t)k->width * (uint64_t)elem_size(pl.dtype);
   if (k->regs > 0) per_thread = std::min<uint64_t>(per_thread, 4 * (uint64_t)k->regs);
@@ -437,7 +441,8 @@ int host_grid(const gar_plan &pl, const JitKernel *k, int grid) {
                            : k->form == GAR_FORM_COOP ? (uint64_t)pl.P * (uint64_t)k->tile * (uint64_t)elem_size(pl.dtype)
                                                       : per_thread * (uint64_t)k->threads;
   const uint64_t most = std::max<uint64_t>(1, (3000000 + per_cta - 1) / per_cta);
-  const uint64_t rounds = std::max<uint64_t>(1, ((uint64_t)grid + most / 2) / most);
+  const uint64_t rounds = ((uint64_t)grid + most / 2) / most;
+  if (rounds <= 1) return (uint64_t)grid <= most + most / 4 ? grid : (int)most;
   return (int)(((uint64_t)grid + rounds - 1) / rounds);
 }
 
@@ -882,8 +887,9 @@ int gar_plan_compile(gar_plan *pl, int mode) {
 int gar_plan_prepare(gar_plan *pl, int mode) {
   if (int rc = check_plan(pl)) return rc;
   if (int rc = check_mode(mode)) return rc;
-  if (mode == GAR_FUSED) return prepare_fused(pl);
-  return prepare_step_faithful(pl);
+  if (mode != GAR_FUSED) return prepare_step_faithful(pl);
+  if (int rc = prepare_fused(pl)) return rc;
+  return prepare_fused_host(pl, nullptr);  // a host call has nothing to build either
 }
 
 int gar_allreduce(gar_plan *pl, void *const *rank_buffers, int mode, gar_stream_t stream) {

@@ -374,14 +374,17 @@ CodegenResult generate_fused_source(const gar_plan &pl, int threads_override, in
   // positions (2^17 below 8 ranks).  GB300, us in graph replay, W by the line above -> W = 1:
   // P = 24 S = 10 fp32, 33000 positions 4.9 -> 2.3, 100000 6.7 -> 3.1, 260000 8.8 -> 6.2; P = 48
   // S = 9 64000 11.0 -> 4.4, 520000 25.6 -> 26.8; P = 12 S = 8 260000 5.3 -> 3.6; P = 5 260000
-  // 2.0 -> 2.1.  Not over NVLink-C2C (`host`), which narrow accesses cost more: P = 8 S = 6
-  // 260000 positions 64 -> 76, P = 10 S = 5 90000 34 -> 39, P = 24 S = 6 200000 149 -> 166
-  // (P = 24 S = 6 131000 101 -> 89, 33000 36 -> 33).  bf16 gains as much on the GPU (P = 127
-  // S = 14 33000 9.4 -> 5.3), and whole vectors only gain from W (P = 64 S = 12 bf16 160000
-  // 9.0 at W = 1, 5.3 at 4).
+  // 2.0 -> 2.1.  From and to host memory (`host`) only up to 2^16 positions: narrow accesses
+  // cost more over NVLink-C2C.  P = 2 to 48, 30 plans, mean of the times at W by the line above
+  // over those at W = 1 (least, greatest): 33000 positions 1.14 (0.95, 1.38), 50000 1.00 (0.89,
+  // 1.20), 66000 0.99 (0.89, 1.26), 90000 0.95 (0.85, 1.10), 200000 0.89 (0.84, 0.96).  bf16
+  // gains as much on the GPU (P = 127 S = 14 33000 9.4 -> 5.3), and whole vectors only gain
+  // from W (P = 64 S = 12 bf16 160000 9.0 at W = 1, 5.3 at 4).
   const bool cut = rotate && (pl.n % (uint64_t)P != 0 || pl.n / (uint64_t)P % (uint64_t)W != 0);
-  int host_width = W;
-  if (!host && cut && elem_size(pl.dtype) == 4 && pl.n < (P < 8 ? 1u << 17 : 1u << 18)) W = 1;
+  const bool narrow = cut && elem_size(pl.dtype) == 4;
+  int host_width = narrow && pl.n < (1u << 16) ? 1 : W;
+  if (host) W = host_width;
+  else if (narrow && pl.n < (P < 8 ? 1u << 17 : 1u << 18)) W = 1;
   if (int w = tune_int("GAR_TUNE_FUSED_W", 0))
     if (w > 0 && (w & (w - 1)) == 0 && w * elem_size(pl.dtype) <= 16) W = host_width = w;
   const int minb = minb_override > 0 ? minb_override : tune_int("GAR_TUNE_FUSED_MINB", small_cta ? 16 : 0);

@@ -220,11 +220,13 @@ void cooperative_ranks() {
 }
 
 // A plan whose vectors are cut by block boundaries runs wider vectors on host memory than on
-// the device, from a kernel that the first host call builds; other plans share one kernel.
+// the device, from a kernel that gar_plan_prepare or the first host call builds; other plans
+// share one kernel.
 void host_width() {
   struct { int P; uint64_t n; int dtype, steps; bool apart; } cases[] = {
       {8, 200003, GAR_F32, 6, true}, {8, 200003, GAR_BF16, 6, false}, {8, 1u << 20, GAR_F32, 6, false},
-      {8, 8 * 4096, GAR_F32, 6, false}, {24, 100, GAR_F32, 10, false}, {6, 79063, GAR_I32, 5, true}};
+      {8, 8 * 4096, GAR_F32, 6, false}, {24, 100, GAR_F32, 10, false}, {6, 79063, GAR_I32, 5, true},
+      {8, 65535, GAR_F32, 6, false}, {8, 65537, GAR_F32, 6, true}};
   for (const auto &c : cases)
     for (bool device_first : {false, true}) {
       const std::vector<void *> r = rows(c.P);
@@ -255,6 +257,13 @@ void host_width() {
         CHECK(run(host) == source[host]);
       }
       CHECK((source[0] != source[1]) == c.apart);
+      gar_plan *ready = plan_of(c.P, c.n, c.dtype, c.steps);
+      CHECK(gar_plan_prepare(ready, GAR_FUSED) == GAR_OK);
+      std::swap(pl, ready);
+      fake::capture = cudaStreamCaptureStatusActive;
+      CHECK(run(true) == source[1] && run(false) == source[0]);
+      fake::capture = cudaStreamCaptureStatusNone;
+      gar_plan_destroy(ready);
       if (!device_first) CHECK(fake::compiles == before + (c.apart ? 2 : 1));
       if (c.apart) {
         CHECK(source[0].find("#define GAR_W 1\n") != std::string::npos);
@@ -268,7 +277,7 @@ void host_width() {
 void host_grid() {
   fake::memory = cudaMemoryTypeHost;
   struct { uint64_t n; unsigned grid; } cases[] = {
-      {8 * 40000, 313}, {8 * 46000, 360}, {8 * 56000, 438}, {8 * 140000, 365}, {8 * 1000000, 373}};
+      {8 * 40000, 313}, {8 * 46000, 360}, {8 * 56000, 438}, {8 * 60000, 367}, {8 * 140000, 365}, {8 * 1000000, 373}};
   const int P = 8;                                   // 8192 bytes of loads a CTA: 367 for 3 MB
   const std::vector<void *> r = rows(P);
   const std::vector<const void *> in(r.begin(), r.end());

@@ -16,7 +16,7 @@ if torch.cuda.is_available():
 
 
 @pytest.mark.parametrize("P,n,dtype,op,S", [(6, 79063, "i32", "sum", 5), (8, 200003, "f32", "sum", 6), (24, 100001, "f32", "max", 10),
-                                            (13, 33001, "f32", "sum", 24), (40, 70001, "f32", "sum", 8)])
+                                            (13, 93001, "f32", "sum", 24), (40, 70001, "f32", "sum", 8)])
 @pytest.mark.parametrize("first", ["direct", "captured", "device"])
 def test_host_vectors(P, n, dtype, op, S, first):
     dist = ("int", -1000, 1000) if dtype == "i32" else ("normal", 0.0, 1.0)
