@@ -201,9 +201,12 @@ bool takes_stream(const gar_plan &pl) {
 //    2.2 either way), 1.2e6 against the breadth-first form (P = 127, S = 8, 1000, 1.1e6,
 //    5.7 -> 3.7; 2500 5.3 -> 6.9).
 //  * Not with a copy at every placement: that program reads without rotation, and has the
-//    most combines (P = 24, S = 5, 400 1.6 -> 1.7; P = 40, S = 6, 2800 2.4 -> 2.6; P = 80,
-//    S = 7, 1000 4.2 -> 2.2, 2500 4.3 -> 7.8; P = 127, S = 7, 500 4.2 -> 3.7, but with the
-//    GPU waited for 17.3 -> 19.6).
+//    most combines, so that it gains in a narrow range only, for which no line is drawn here
+//    (P = 80, S = 7, 1000 4.2 -> 2.2, but 2500 4.3 -> 7.8; P = 24, S = 5, 400 1.6 -> 1.7;
+//    P = 40, S = 6, 2800 2.4 -> 2.6; P = 127, S = 7, 500 4.2 -> 3.7, but with the GPU waited
+//    for 17.3 -> 19.6).
+//  * A few positions, up to about 20, lose 0.1 to 0.25 below P = 32 (P = 20, S = 10, 7 1.4 ->
+//    1.5; P = 24, S = 7, 8 1.40 -> 1.42, 20 1.3 -> 1.5; P = 32, S = 10, 20 1.5 -> 1.4).
 bool takes_coop(const gar_plan &pl) {
   const char *ff = std::getenv("GAR_TUNE_FUSED_FORM");
   if ((ff && *ff) || older_form_tuned()) return false;

@@ -9,8 +9,8 @@
 // of one (op, rank) pair (short blocks: one thread per element and one to four ops).
 // Combine ops batch 2 vectors per thread; same-type copies move raw 16-byte units, 6 per
 // thread; a bf16 plan's first step keeps its 16-byte bf16 loads packed until the
-// combine.  The kernels add the bytes they read from partners to the step's counter
-// slots, so the bytes a step actually moved are recorded.  The launches of one Allreduce
+// combine.  Every thread counts the bytes it reads from partners and the kernels add them to
+// the step's counter slots, so the bytes a step actually moved are recorded.  The launches of one Allreduce
 // are chained by programmatic dependent launch.  The same work functions serve the
 // per-step launches, the persistent kernel and the no-allocation launches.
 #include <cuda_bf16.h>
