@@ -97,7 +97,7 @@ int prepare_step_faithful(gar_plan *pl) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset(barrier state)");
   }
   if (pl->d_step_bytes == nullptr && pl->S > 0) {
-    const size_t cbytes = (size_t)(pl->S + 1) * STEP_BYTE_SLOTS * sizeof(unsigned long long);
+    const size_t cbytes = (size_t)(pl->S + 1) * STEP_ROW * sizeof(unsigned long long);
     cudaError_t e = cudaMalloc(&pl->d_step_bytes, cbytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(step counters)");
     e = cudaMemset(pl->d_step_bytes, 0, cbytes);
@@ -636,7 +636,7 @@ int run_step_faithful(gar_plan *pl, void *const *rank, gar_stream_t stream, bool
   if (pl->step_bytes_stale) {
     // an earlier sequence stopped part-way: the kernels' own upkeep of the counters did too
     cudaError_t e = cudaMemsetAsync(pl->d_step_bytes, 0,
-                                    (size_t)(pl->S + 1) * STEP_BYTE_SLOTS * sizeof(unsigned long long),
+                                    (size_t)(pl->S + 1) * STEP_ROW * sizeof(unsigned long long),
                                     (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(step counters)");
   }
@@ -1002,13 +1002,13 @@ int gar_last_step_bytes(const gar_plan *pl, uint64_t *per_step) {
   }
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)pl->last_stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-  std::vector<unsigned long long> tmp((size_t)pl->S * STEP_BYTE_SLOTS);
+  std::vector<unsigned long long> tmp((size_t)pl->S * STEP_ROW);
   e = cudaMemcpy(tmp.data(), pl->d_step_bytes, tmp.size() * sizeof(unsigned long long),
                  cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(step counters)");
   for (int t = 0; t < pl->S; ++t) {
     uint64_t sum = 0;
-    for (int k = 0; k < STEP_BYTE_SLOTS; ++k) sum += tmp[(size_t)t * STEP_BYTE_SLOTS + k];
+    for (int k = 0; k < STEP_BYTE_SLOTS; ++k) sum += tmp[(size_t)t * STEP_ROW + k * STEP_SLOT_STRIDE];
     per_step[t] = sum;
   }
   return GAR_OK;

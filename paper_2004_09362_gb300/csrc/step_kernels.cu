@@ -93,7 +93,7 @@ struct StepArgs {
   void *rank[MAXP];
   void *ws[NUM_WS_BUFS];             // QP0, QP1, QS slice bases (nullptr if unused)
   const StepOp *ops;                 // this launch's ops
-  unsigned long long *bytes;         // STEP_BYTE_SLOTS counters of the step, or nullptr
+  unsigned long long *bytes;         // the step's row of counters, or nullptr
   uint64_t q, rem, n_pad;
   uint64_t n;                        // elements per rank
   uint32_t chunk;                    // elements per CTA
@@ -213,15 +213,23 @@ __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol
 // Per-launch parameters the work functions need besides the buffers.
 struct LaunchView {
   const StepOp *ops;
-  unsigned long long *bytes;  // STEP_BYTE_SLOTS counters of the communication step, or nullptr
+  unsigned long long *bytes;  // the communication step's row of counters, or nullptr
   uint32_t chunk;             // elements per CTA item (chunked mapping)
   int nops, partner, nchunks;
   int group;                  // ops per thread (element-major mapping)
 };
 
-// The bytes that the CTA's NT threads have read from partners, added to a step's counters by
-// one atomic add: every thread stages its count, and after a barrier one thread adds the sums
-// of the warps.
+// Adds the bytes that a warp's threads have read from partners to a step's counters.
+__device__ __forceinline__ void count_moved(unsigned long long *bytes, uint32_t moved) {
+  if (bytes == nullptr) return;
+  const uint32_t sum = __reduce_add_sync(0xffffffffu, moved);
+  if ((threadIdx.x & 31) == 0 && sum)
+    atomicAdd(bytes + (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) % STEP_BYTE_SLOTS * STEP_SLOT_STRIDE,
+              (unsigned long long)sum);
+}
+
+// The same by one add of a CTA of NT threads (persistent kernel): every thread stages its
+// count, and after a barrier one thread adds the sums of the warps.
 template <int NT>
 __device__ __forceinline__ void stage_moved(uint32_t *s_moved, uint32_t moved) {
   const uint32_t sum = __reduce_add_sync(0xffffffffu, moved);
@@ -232,7 +240,7 @@ __device__ __forceinline__ void add_moved(unsigned long long *bytes, const uint3
   unsigned long long total = 0;
 #pragma unroll
   for (int w = 0; w < NT / 32; ++w) total += s_moved[w];
-  if (total) atomicAdd(bytes + blockIdx.x % STEP_BYTE_SLOTS, total);
+  if (total) atomicAdd(bytes + blockIdx.x % STEP_BYTE_SLOTS * STEP_SLOT_STRIDE, total);
 }
 
 // Elements [c0, c0 + len) of the block that op `op` touches at rank x, by the CTA's NT
@@ -456,13 +464,7 @@ __device__ __forceinline__ void flat_work(const StepArgs<MAXP> &a, const LaunchV
     }
   }
   wait_prior_grid();  // threads without an item: the grid must not complete before its predecessor
-  // one atomic add per warp, of the bytes its threads read from partners
-  if (lv.bytes != nullptr) {
-    const uint32_t sum = __reduce_add_sync(0xffffffffu, moved);
-    if ((threadIdx.x & 31) == 0 && sum)
-      atomicAdd(lv.bytes + (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) % STEP_BYTE_SLOTS,
-                (unsigned long long)sum);
-  }
+  count_moved(lv.bytes, moved);
 }
 
 template <int MAXP>
@@ -481,8 +483,9 @@ __device__ __forceinline__ LaunchView view_of(const StepArgs<MAXP> &a) {
 __device__ __forceinline__ void counter_upkeep(const CounterUpkeep &c) {
   static_assert(STEP_BYTE_SLOTS <= kThreads, "one thread per counter slot");
   if (threadIdx.x < STEP_BYTE_SLOTS) {
-    if (c.zero != nullptr) c.zero[threadIdx.x] = 0;
-    if (c.move_from != nullptr) c.move_to[threadIdx.x] = atomicExch(c.move_from + threadIdx.x, 0ull);
+    const int at = threadIdx.x * STEP_SLOT_STRIDE;
+    if (c.zero != nullptr) c.zero[at] = 0;
+    if (c.move_from != nullptr) c.move_to[at] = atomicExch(c.move_from + at, 0ull);
   }
 }
 
@@ -490,23 +493,11 @@ __device__ __forceinline__ void counter_upkeep(const CounterUpkeep &c) {
 // 48 registers the compiler picks unbounded, fp32 the same.
 template <typename T, int OP, int MAXP>
 __global__ void __launch_bounds__(kThreads, 6) step_kernel(const __grid_constant__ StepArgs<MAXP> a) {
-  // bytes read from partners in the low 28 bits (a chunk has less), finished warps above
-  __shared__ uint32_t s_moved;
-  if (threadIdx.x == 0) s_moved = 0;
-  __syncthreads();
   wait_prior_grid();
   if (blockIdx.x == 0) counter_upkeep(a.upkeep);
   const uint32_t moved = chunk_work<T, OP, MAXP>(a, view_of(a), a.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
   allow_next_grid();
-  if (a.bytes != nullptr) {
-    const uint32_t sum = __reduce_add_sync(0xffffffffu, moved);
-    if ((threadIdx.x & 31) == 0) {
-      const uint32_t before = atomicAdd(&s_moved, (1u << 28) + sum);
-      const uint32_t total = (before & 0xfffffffu) + sum;
-      if (before >> 28 == kThreads / 32 - 1 && total)
-        atomicAdd(a.bytes + blockIdx.x % STEP_BYTE_SLOTS, (unsigned long long)total);
-    }
-  }
+  count_moved(a.bytes, moved);
 }
 
 template <typename T, int OP, int MAXP>
@@ -562,7 +553,7 @@ template <int MAXP>
 struct PersistArgs {
   StepArgs<MAXP> s;                 // buffers and sizes (s.ops = whole op table)
   const LaunchDesc *launches;
-  unsigned long long *step_bytes;   // S rows of STEP_BYTE_SLOTS counters, then the first step's own
+  unsigned long long *step_bytes;   // S rows of STEP_ROW counters, then the first step's own
   BarrierState *bar;
   int nlaunch, nsteps;
   unsigned int spin_limit;          // polls before a wait gives up
@@ -628,15 +619,15 @@ __device__ bool grid_barrier(BarrierState *bar, unsigned expected, unsigned spin
 __host__ __device__ __forceinline__ unsigned long long *counter_row(unsigned long long *rows, int comm_step,
                                                                     int nsteps) {
   if (rows == nullptr || comm_step < 0) return nullptr;
-  return rows + (size_t)(comm_step == 0 ? nsteps : comm_step) * STEP_BYTE_SLOTS;
+  return rows + (size_t)(comm_step == 0 ? nsteps : comm_step) * STEP_ROW;
 }
 __host__ __device__ __forceinline__ CounterUpkeep upkeep_of(unsigned long long *rows, int launch, int next_comm_step,
                                                             int nsteps, int move_at = 1) {
   CounterUpkeep c{nullptr, nullptr, nullptr};
   if (rows == nullptr) return c;
-  if (next_comm_step > 0) c.zero = rows + (size_t)next_comm_step * STEP_BYTE_SLOTS;
+  if (next_comm_step > 0) c.zero = rows + (size_t)next_comm_step * STEP_ROW;
   if (launch == move_at) {
-    c.move_from = rows + (size_t)nsteps * STEP_BYTE_SLOTS;
+    c.move_from = rows + (size_t)nsteps * STEP_ROW;
     c.move_to = rows;
   }
   return c;
@@ -738,7 +729,7 @@ __global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, PER_SM)
     p.bar->outcome = error;
     p.bar->outcome_launch = p.bar->error_launch;
     if (error != 0 && p.step_bytes != nullptr)
-      for (int k = 0; k < STEP_BYTE_SLOTS; ++k) p.step_bytes[(size_t)p.nsteps * STEP_BYTE_SLOTS + k] = 0;
+      for (int k = 0; k < STEP_BYTE_SLOTS; ++k) p.step_bytes[(size_t)p.nsteps * STEP_ROW + k * STEP_SLOT_STRIDE] = 0;
     p.bar->count = 0;
     p.bar->leaving = 0;
     p.bar->error = 0;
