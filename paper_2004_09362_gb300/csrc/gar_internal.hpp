@@ -59,6 +59,7 @@ struct Launch {
 struct LaunchDesc {
   int first_op, nops, partner, comm_step;
   int group;          // element-major mapping: ops per thread
+  int pieces, piece;  // else: pieces per block, elements of a piece
 };
 
 struct CommStep {

@@ -69,15 +69,19 @@ constexpr uint64_t kNoAllocFlatBlock = 512;
 constexpr uint64_t kNoAllocFlatItems = 1u << 18;
 constexpr int kFlatGroup = 4;
 constexpr uint64_t kFlatThreads = 512;
-// Persistent steps: smallest piece of a block.  The chunked steps run in CTAs of 256 threads, 2
-// per SM, or 3 where the largest step has more blocks (P * ops) than the CTAs at 2 per SM, of
-// bf16 plans twice as many: a CTA then works through several pieces, and more warps hide
-// their loads.  GB300, us call after call, 2 per SM -> 3 (4): P = 24 x 4 MiB int32 max S = 10
-// (288 blocks) 98 -> 102 (96), P = 12 x 160000 int32 S = 8 31 -> 35 (40), P = 18 x 90000 fp32
-// S = 10 38 -> 42 (48); P = 18 x 1.8M fp32 S = 5 427 -> 342 (353), P = 64 x 851000 int32 S = 6
-// 697 -> 588 (549), P = 18 x 239000 bf16 S = 5 71 -> 62 (74), x 90000 bf16 S = 7 37 -> 40 (43).
+// Persistent steps: smallest piece of a block, and most pieces (see launch_desc).  The chunked
+// steps run in CTAs of 256 threads, 2 per SM without spills, or 3, whose warps hide more of the
+// loads' latency, where the largest step has 2^22 elements (ops * n) or more (2^24 in bf16
+// plans of one or two result copies, whose code spills at 3), or, with more than two copies,
+// more than 4 blocks (P * ops) per SM.  GB300, us call after call, 2 per SM -> 3
+// (before: 3 per SM, every step cut into 16384 elements): P = 24 x 4 MiB int32 max S = 10 96 ->
+// 93 (134), P = 18 x 1.8M fp32 S = 5 409 -> 333 (387), P = 64 x 851000 int32 S = 6 697 -> 586
+// (604), P = 18 x 38000 S = 5 31 -> 27 (32), P = 13 x 1.6M bf16 S = 4 279 -> 243 (258); but
+// P = 17 x 77000 fp32 S = 5 27 -> 29 (45), P = 12 x 160000 int32 S = 8 29 -> 33 (40), P = 33 x
+// 69000 fp32 S = 11 41 -> 45 (57), P = 24 x 960000 bf16 S = 10 75 -> 79 (151).
 constexpr int kPersistThreads = 256;
 constexpr uint64_t kMinPiece = 2048;
+constexpr uint64_t kMostPieces = 24;
 
 // Counter upkeep of one launch, by its first CTA (after wait_prior_grid): zeroes the
 // counters of the communication step that follows, and moves the first step's counts,
@@ -633,45 +637,6 @@ __host__ __device__ __forceinline__ CounterUpkeep upkeep_of(unsigned long long *
   return c;
 }
 
-// One step as a CTA of the persistent kernel sees it, fetched before the barrier that opens
-// it (the tables never change).
-struct PersistStep {
-  LaunchDesc d;
-  uint32_t items, nchunks, chunk;  // nchunks pieces of `chunk` elements per block
-};
-
-template <int MAXP, bool FLAT>
-__device__ __forceinline__ PersistStep fetch_step(const PersistArgs<MAXP> &p, int l) {
-  PersistStep s{};
-  s.d = p.launches[l];
-  if (FLAT) return s;
-  // A step's blocks (P * nops of maxblk elements) are cut into equal pieces, as many as
-  // give every CTA one piece, or, where there are more blocks than CTAs, as many as take
-  // the fewest batches of loads (and starts of pieces) in all rounds: every CTA reaches the
-  // barrier at about the same time.
-  const uint64_t maxblk = p.s.q + (p.s.rem ? 1 : 0);
-  const uint32_t blocks = (uint32_t)p.s.P * (uint32_t)max(1, s.d.nops);
-  constexpr uint32_t batch = 4 * kUnroll * kPersistThreads;
-  uint32_t k = gridDim.x / blocks;
-  if (k == 0) {
-    uint64_t best = ~0ull;
-    for (uint32_t c = 1; c <= 4; ++c) {
-      const uint64_t piece = (maxblk + c - 1) / c;
-      const uint64_t cost = (uint64_t)((blocks * c + gridDim.x - 1) / gridDim.x) * ((piece + batch - 1) / batch + 1);
-      if (cost < best) {
-        best = cost;
-        k = c;
-      }
-    }
-  }
-  uint64_t chunk = ((maxblk + k - 1) / k + 7) / 8 * 8;
-  if (chunk < kMinPiece) chunk = kMinPiece;
-  s.chunk = (uint32_t)chunk;
-  s.nchunks = (uint32_t)((maxblk + chunk - 1) / chunk);
-  s.items = s.d.nops > 0 ? s.nchunks * blocks : 0;
-  return s;
-}
-
 // FLAT: element-major mapping (small blocks), else pieces of blocks.  PER_SM: CTAs per SM that
 // its registers allow for.
 template <typename T, int OP, int MAXP, bool FLAT, int PER_SM>
@@ -688,32 +653,33 @@ __global__ void __launch_bounds__(FLAT ? kThreads : kPersistThreads, PER_SM)
   // The first step's counts are added beside barrier 0 and moved behind barrier 1; a launch of
   // two steps has no barrier 1: there the add comes before the arrival at barrier 0.
   const int move_at = p.nlaunch > 2 ? 2 : 1;
-  PersistStep st = fetch_step<MAXP, FLAT>(p, 0);
+  LaunchDesc st = p.launches[0];  // fetched before the barrier that opens the step (never changes)
   for (int l = 0; l < p.nlaunch && ok; ++l) {
     LaunchView lv;
-    lv.ops = p.s.ops + st.d.first_op;
-    lv.nops = st.d.nops;
-    lv.partner = st.d.partner;
-    lv.bytes = counter_row(p.step_bytes, st.d.comm_step, p.nsteps);
-    lv.chunk = st.chunk;
-    lv.nchunks = (int)st.nchunks;
-    lv.group = st.d.group;
+    lv.ops = p.s.ops + st.first_op;
+    lv.nops = st.nops;
+    lv.partner = st.partner;
+    lv.bytes = counter_row(p.step_bytes, st.comm_step, p.nsteps);
+    lv.chunk = (uint32_t)st.piece;
+    lv.nchunks = st.pieces;
+    lv.group = st.group;
     if (FLAT) {
       flat_work<T, OP, MAXP>(p.s, lv, s_rank, (uint64_t)blockIdx.x * kThreads + threadIdx.x,
                              (uint64_t)gridDim.x * kThreads);
     } else {
       uint32_t moved = 0;
-      for (uint32_t item = blockIdx.x; item < st.items; item += gridDim.x) {
-        const uint32_t blk = item / st.nchunks, op = blk / (uint32_t)p.s.P;
+      const uint32_t pieces = (uint32_t)st.pieces, items = pieces * (uint32_t)p.s.P * (uint32_t)st.nops;
+      for (uint32_t item = blockIdx.x; item < items; item += gridDim.x) {
+        const uint32_t blk = item / pieces, op = blk / (uint32_t)p.s.P;
         moved += range_work<T, OP, MAXP, kPersistThreads>(p.s, lv, lv.ops[op], (int)(blk - op * (uint32_t)p.s.P),
-                                                          (uint64_t)(item - blk * st.nchunks) * st.chunk, st.chunk);
+                                                          (uint64_t)(item - blk * pieces) * lv.chunk, lv.chunk);
       }
       stage_moved<kPersistThreads>(s_moved, moved);
     }
     unsigned long long *const bytes = FLAT ? nullptr : lv.bytes;  // (flat_work has added its own)
     if (l + 1 < p.nlaunch) {
-      st = fetch_step<MAXP, FLAT>(p, l + 1);
-      if (blockIdx.x == 0) counter_upkeep(upkeep_of(p.step_bytes, l, st.d.comm_step, p.nsteps, move_at));
+      st = p.launches[l + 1];
+      if (blockIdx.x == 0) counter_upkeep(upkeep_of(p.step_bytes, l, st.comm_step, p.nsteps, move_at));
       ok = grid_barrier<kPersistThreads>(p.bar, expected, p.spin_limit, l, bytes, s_moved, p.nlaunch == 2);
     } else {
       if (blockIdx.x == 0) counter_upkeep(upkeep_of(p.step_bytes, l, -1, p.nsteps, move_at));
@@ -845,6 +811,15 @@ int launch_dt(const gar_plan &pl, const Launch &ln, int li, void *const *rank, g
   return GAR_EINVAL;
 }
 
+// CTAs per SM of a plan's persistent launches (see kPersistThreads).
+int persist_per_sm(const gar_plan &pl) {
+  int most_ops = 0;
+  for (const Launch &ln : pl.launches) most_ops = std::max(most_ops, ln.nops);
+  const uint64_t blocks = (uint64_t)most_ops * (uint64_t)pl.P, elements = (uint64_t)most_ops * pl.n;
+  const bool few = pl.K <= 2;
+  return elements >= (few && pl.dtype == GAR_BF16 ? 1u << 24 : 1u << 22) || (!few && blocks > 4 * (uint64_t)num_sms()) ? 3 : 2;
+}
+
 template <typename T, int OP, int MAXP>
 int launch_persistent_typed(const gar_plan &pl, void *const *rank, gar_stream_t stream) {
   PersistArgs<MAXP> p{};
@@ -867,12 +842,9 @@ int launch_persistent_typed(const gar_plan &pl, void *const *rank, gar_stream_t 
     need = std::max<uint64_t>(need, flat ? ((uint64_t)((ln.nops + group - 1) / group) * pl.n + kThreads - 1) / kThreads
                                          : (uint64_t)ln.nops * pl.P * ((maxblk + kMinPiece - 1) / kMinPiece));
   }
-  int most_ops = 0;
-  for (const Launch &ln : pl.launches) most_ops = std::max(most_ops, ln.nops);
-  const bool many = (uint64_t)most_ops * (uint64_t)pl.P > (sizeof(T) == 2 ? 4u : 2u) * (uint64_t)num_sms();
   const void *fn = flat   ? (const void *)step_kernel_persistent<T, OP, MAXP, true, 4>
-                   : many ? (const void *)step_kernel_persistent<T, OP, MAXP, false, 3>
-                          : (const void *)step_kernel_persistent<T, OP, MAXP, false, 2>;
+                   : persist_per_sm(pl) == 3 ? (const void *)step_kernel_persistent<T, OP, MAXP, false, 3>
+                                             : (const void *)step_kernel_persistent<T, OP, MAXP, false, 2>;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, flat ? kThreads : kPersistThreads, 0);
   if (e != cudaSuccess || per_sm < 1) return cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e,
@@ -925,8 +897,28 @@ void barrier_outcome(const void *state, int *error, int *launch) {
   *launch = st->outcome_launch;
 }
 
+// A persistent step's blocks (P * nops of at most maxblk elements) are cut into equal pieces,
+// as many as take the fewest batches of loads (and starts of pieces) in all rounds of the
+// grid, so that every CTA reaches the barrier at about the same time.  (With at most 4 pieces,
+// and one where there are more CTAs than blocks, P = 13 x 1.6M bf16 S = 4, 338 blocks, took 289
+// us instead of 243.)
 LaunchDesc launch_desc(const gar_plan &pl, const Launch &ln) {
-  return {ln.first_op, ln.nops, ln.partner, ln.comm_step, pick_group(pl.n, ln.nops)};
+  LaunchDesc d{ln.first_op, ln.nops, ln.partner, ln.comm_step, pick_group(pl.n, ln.nops), 1, 0};
+  const uint64_t maxblk = pl.q + (pl.rem ? 1 : 0), blocks = (uint64_t)pl.P * (uint64_t)std::max(1, ln.nops);
+  const uint64_t grid = (uint64_t)persist_per_sm(pl) * (uint64_t)num_sms();
+  constexpr uint64_t batch = 4 * kUnroll * kPersistThreads;
+  uint64_t best = ~0ull;
+  for (uint64_t c = 1; c <= std::max<uint64_t>(kMostPieces, grid / blocks); ++c) {
+    const uint64_t piece = std::max<uint64_t>(kMinPiece, ((maxblk + c - 1) / c + 7) / 8 * 8);
+    const uint64_t pieces = (maxblk + piece - 1) / piece;
+    const uint64_t cost = ((blocks * pieces + grid - 1) / grid) * ((piece + batch - 1) / batch + 1);
+    if (cost < best) {
+      best = cost;
+      d.pieces = (int)pieces;
+      d.piece = (int)piece;
+    }
+  }
+  return d;
 }
 
 }  // namespace gar
